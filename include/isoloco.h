@@ -266,7 +266,7 @@ int isoloco_debug_gemm(int a_mn_major, int b_mn_major, int precision, int batch,
  * implicit device-wide synchronization of cudaMalloc / cudaFree would stall the
  * work queued on its other streams.  This entry point calls neither, nor any
  * other allocating routine: its scratch (the hi/lo operand planes, the four
- * tensor maps, an error word and a tile counter) lives in one static device
+ * tensor maps and an error word) lives in one static device
  * array of the library, 16 MiB per device, held by every GPU that loads the
  * library until the process exits.
  *
@@ -283,7 +283,7 @@ int isoloco_debug_gemm(int a_mn_major, int b_mn_major, int precision, int batch,
  * message giving the bytes needed, before anything is launched.
  *
  * Every call on a device shares that one array.  The call zeroes the error word
- * and the tile counter on `stream` before its kernels and synchronizes `stream`
+ * on `stream` before its kernels and synchronizes `stream`
  * before returning, so calls made one after another are safe.  Calls whose GPU
  * work can overlap (from several host threads, or on streams that are not
  * ordered with one another) race on the shared scratch and give wrong results;

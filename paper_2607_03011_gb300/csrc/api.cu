@@ -50,7 +50,7 @@ __global__ void k_trace_partial(const MatDesc*, const int4*, int, const MatState
                                 const __nv_bfloat16*, const __nv_bfloat16*, double*);
 __global__ void k_trace_final(const MatDesc*, int, MatState*, const double*, const double*);
 __global__ void k_reset_state(MatState*, int, uint32_t*, const MatDesc*, const int*, const int*, int, int*, int*,
-                              int*, int);
+                              int*);
 __global__ void k_reduce(const Chunk*, const MatDesc*, ReplicaPtrs, int, int, const float*, float,
                          __nv_bfloat16*, __nv_bfloat16*, float*, uint32_t*);
 __global__ void k_reduce_f32(const Chunk*, const MatDesc*, ReplicaPtrs, int, const float*, float, __nv_bfloat16*,
@@ -95,7 +95,6 @@ __global__ void k_debug_wait(uint32_t*, uint64_t, unsigned long long*);
 constexpr int kChunkElems = 16384;
 constexpr int kTraceChunkElems = 16384;
 constexpr int kDefaultMaxIter = 28;
-constexpr int kLaunchCounters = 4096;  // dynamic-scheduler counters, one per GEMM launch of a step
 constexpr float kDefaultTol = 4e-3f;
 
 // Roles of the tensor maps of one bucket.
@@ -171,15 +170,14 @@ struct isoloco_plan {
     int4* tchunks = nullptr;
     MatState* state = nullptr;
     MatDesc* mats_d = nullptr;
-    // work lists (per shape bucket) rebuilt by k_control, and the GEMM tile counters
+    // work lists (per shape bucket) rebuilt by k_control, and its block ticket
     int* bucket_first_d = nullptr;
     int* bucket_count_d = nullptr;
     int* list_gram = nullptr;
     int* cnt_gram = nullptr;
     int* list_step = nullptr;
     int* cnt_step = nullptr;
-    int* counters = nullptr;
-    int launch_seq = 0;
+    int* ticket = nullptr;
     int64_t* gpart_off_d = nullptr;
     int64_t* gpart_sstride_d = nullptr;
     int* nsplit_d = nullptr;
@@ -466,8 +464,8 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
         const int kblocks = (kdim + BK - 1) / BK;
         // split-K for long reductions: at most 256 k-blocks per split, and more splits
         // (down to 32 k-blocks each) only while the bucket alone would not fill the GPU
-        // (two output tiles per SM, or per pair of SMs with pair MMAs)
-        const int slots = 2 * p->num_sms / (kPairMma ? 2 : 1);
+        // (two output tiles per pair of SMs)
+        const int slots = p->num_sms;
         int splits = std::max(1, (kblocks + 255) / 256);
         if (tiles * splits < slots) splits = std::max(splits, std::min(slots / std::max(1, tiles), kblocks / 32));
         if (bk.gs) splits = std::max(splits, 2);  // iteration 0's Gram stays in fp32 partials (k_gs_init)
@@ -590,7 +588,7 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
         (rc = dalloc(p, &p->bucket_count_d, (int64_t)p->buckets.size())) ||
         (rc = dalloc(p, &p->cnt_gram, (int64_t)p->buckets.size())) ||
         (rc = dalloc(p, &p->cnt_step, (int64_t)p->buckets.size())) ||
-        (rc = dalloc(p, &p->counters, kLaunchCounters + 1)) || (rc = dalloc(p, &p->loopc, 2)) ||
+        (rc = dalloc(p, &p->ticket, 1)) || (rc = dalloc(p, &p->loopc, 2)) ||
         (rc = dalloc(p, &p->tmaps_d, (int64_t)kMapsPerBucket * std::max<size_t>(1, p->buckets.size()))) ||
         (rc = dalloc(p, &p->anhi, gs_elems)) || (rc = dalloc(p, &p->anlo, gs_elems)) ||
         (rc = dalloc(p, &p->whi, gs_elems)) || (rc = dalloc(p, &p->wlo, gs_elems)) ||
@@ -789,7 +787,6 @@ static int flush_set(isoloco_plan* pl, int phase, LaunchSet& s, cudaStream_t st)
             p.g[p.num_groups++] = g;
         }
         p.total_tiles = cta;
-        p.counter = pl->counters + (pl->launch_seq++ % kLaunchCounters);
         CUDA_TRY(launch_gemm(p, pl->num_sms, st));
     }
     return ISOLOCO_OK;
@@ -960,7 +957,7 @@ static int polar_iteration(isoloco_plan* p, int t, int max_iter, float tol, cuda
         k_control<<<(p->nmat + kControlThreads / 32 - 1) / (kControlThreads / 32), kControlThreads, 0, st>>>(p->mats_d, p->nmat, p->state, p->fin_part, t, max_iter, tol, p->err_d,
                                       p->bucket_first_d, p->bucket_count_d, (int)p->buckets.size(), p->list_gram,
                                       p->cnt_gram, p->list_step, p->cnt_step, cond, set_cond, p->loopc,
-                                      p->fast_steps, p->counters + kLaunchCounters,
+                                      p->fast_steps, p->ticket,
                                       make_int4(gp_one(p, 0, 0), gp_one(p, 0, 1), gp_one(p, 1, 0), gp_one(p, 1, 1)),
                                       make_int4(up_one(p, 0, 0), up_one(p, 0, 1), up_one(p, 1, 0), up_one(p, 1, 1)), gs_on ? 1 : 0); }
         CUDA_TRY(cudaGetLastError());
@@ -1187,7 +1184,7 @@ static int run_polar(isoloco_plan* p, int max_iter, float tol, cudaStream_t st) 
     if (rc) return rc;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CUDA_TRY(cudaStreamIsCapturing(st, &cs));
-    const bool use_graph = kPairMma && !p->prof && !p->per_launch && cs == cudaStreamCaptureStatusNone;
+    const bool use_graph = !p->prof && !p->per_launch && cs == cudaStreamCaptureStatusNone;
     if (use_graph) {
         if (!p->gexec || p->g_max_iter != max_iter || p->g_tol != tol || p->g_fast != p->fast_steps ||
             p->g_full != (p->full_prec ? 1 : 0) || p->g_prec != p->prec_code)
@@ -1421,9 +1418,8 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
     { PhaseTimer tm(p, ISOLOCO_PHASE_CLIP, st, 0);
     k_reset_state<<<(std::max(1, a->nmat) + 255) / 256, 256, 0, st>>>(
         a->state, a->nmat, a->err_d, a->mats_d, a->bucket_first_d, a->bucket_count_d, (int)a->buckets.size(),
-        a->list_gram, a->cnt_gram, a->counters, kLaunchCounters + 1);
+        a->list_gram, a->cnt_gram, a->ticket);
     a->launches += 1;
-    a->launch_seq = 0;
     CUDA_TRY(cudaGetLastError());
     k_clip_form_a<<<grid, 256, 0, st>>>(p->mats_d, p->state, p->hbuf, p->hoff_d, p->hss_d, p->nsplit_d, a->mats_d,
                                          p->aux_of_d, a->dhi, a->dlo);
@@ -1593,8 +1589,7 @@ static int run_isoc_step(isoloco_plan* p, int merge, float* theta, float* mom, c
     { PhaseTimer tm(p, ISOLOCO_PHASE_OTHER, st);
     k_reset_state<<<(std::max(1, p->nmat) + 255) / 256, 256, 0, st>>>(
         p->state, p->nmat, p->err_d, p->mats_d, p->bucket_first_d, p->bucket_count_d, (int)p->buckets.size(),
-        p->list_gram, p->cnt_gram, p->counters, kLaunchCounters + 1); }
-    p->launch_seq = 0;
+        p->list_gram, p->cnt_gram, p->ticket); }
     CUDA_TRY(cudaGetLastError());
     if (p->nchunks) {
         PhaseTimer tm(p, ISOLOCO_PHASE_REDUCE, st);
@@ -2070,13 +2065,13 @@ int isoloco_debug_gemm(int a_mn, int b_mn, int precision, int batch, int M, int 
         cudaFree(ah); cudaFree(al); cudaFree(bh); cudaFree(bl); cudaFree(maps_d); cudaFree(dummy_state); cudaFree(err);
     };
     if (cudaMalloc(&ah, asz * 2) || cudaMalloc(&al, asz * 2) || cudaMalloc(&bh, bsz * 2) || cudaMalloc(&bl, bsz * 2) ||
-        cudaMalloc(&maps_d, 4 * sizeof(CUtensorMap)) || cudaMalloc(&err, 8)) {
+        cudaMalloc(&maps_d, 4 * sizeof(CUtensorMap)) || cudaMalloc(&err, 4)) {
         cleanup();
         return fail(ISOLOCO_ERR_OOM, "debug_gemm scratch allocation failed");
     }
     cudaMemsetAsync(ah, 0, asz * 2, st); cudaMemsetAsync(al, 0, asz * 2, st);
     cudaMemsetAsync(bh, 0, bsz * 2, st); cudaMemsetAsync(bl, 0, bsz * 2, st);
-    cudaMemsetAsync(err, 0, 8, st);  // err word and the tile counter
+    cudaMemsetAsync(err, 0, 4, st);
     const int f16 = precision > 0 ? 1 : 0;
     k_split_planes<<<1024, 256, 0, st>>>(A, (int64_t)batch * a_rows * a_cols, a_rows, a_cols, lda, ah, al, f16);
     k_split_planes<<<1024, 256, 0, st>>>(B, (int64_t)batch * b_rows * b_cols, b_rows, b_cols, ldb, bh, bl, f16);
@@ -2110,7 +2105,6 @@ int isoloco_debug_gemm(int a_mn, int b_mn, int precision, int batch, int M, int 
     g.ld_f32 = N;
     gp.num_groups = 1;
     gp.total_tiles = batch * g.tiles_m * g.tiles_n;
-    gp.counter = reinterpret_cast<int*>(err) + 1;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2128,8 +2122,7 @@ int isoloco_debug_gemm(int a_mn, int b_mn, int precision, int batch, int M, int 
 
 // ================================================================== GEMM without allocation
 // Scratch of isoloco_debug_gemm_noalloc: one array per device, shared by every call.
-//   [0, 4)     error word      \  zeroed by every call before its launches
-//   [4, 8)     tile counter    /
+//   [0, 4)     error word, zeroed by every call before its launches
 //   [256, 768) the four tensor maps (A hi, A lo, B hi, B lo), written by every call
 //   [1024, ..) A hi, A lo, B hi, B lo planes, each starting on a 256-byte boundary and
 //              fully written by the split kernel before the GEMM reads them
@@ -2202,7 +2195,7 @@ int isoloco_debug_gemm_noalloc(int a_mn, int b_mn, int precision, int batch, int
     if (!make_map(&maps[0], ah, a_cols, a_rows, batch, lda, ra) || !make_map(&maps[1], al, a_cols, a_rows, batch, lda, ra) ||
         !make_map(&maps[2], bh, b_cols, b_rows, batch, ldb, rb) || !make_map(&maps[3], bl, b_cols, b_rows, batch, ldb, rb))
         return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed");
-    CUDA_TRY(cudaMemsetAsync(err, 0, 8, st));  // error word and tile counter
+    CUDA_TRY(cudaMemsetAsync(err, 0, 4, st));  // error word
     CUDA_TRY(cudaMemcpyAsync(maps_d, maps, sizeof(maps), cudaMemcpyHostToDevice, st));
     const int f16 = precision > 0 ? 1 : 0;
     k_split_planes<<<1024, 256, 0, st>>>(A, (int64_t)batch * a_rows * a_cols, a_rows, a_cols, lda, ah, al, f16);
@@ -2230,7 +2223,6 @@ int isoloco_debug_gemm_noalloc(int a_mn, int b_mn, int precision, int batch, int
     g.ld_f32 = N;
     gp.num_groups = 1;
     gp.total_tiles = batch * g.tiles_m * g.tiles_n;
-    gp.counter = reinterpret_cast<int*>(err) + 1;
     int dev = 0, sms = 148;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

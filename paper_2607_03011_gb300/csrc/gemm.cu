@@ -37,19 +37,16 @@ __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
     return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
-// Descriptors of one operand plane for the k-th 16-deep slice of a stage.
-template <bool MN>
-__device__ __forceinline__ uint64_t operand_desc(uint32_t plane_addr, int ks) {
-    if (MN) {
-        // 128B swizzle, MN-major: 64-element MN chunks are BK*128 bytes apart (LBO),
-        // 8-row K groups are 1024 bytes apart (SBO); a 16-deep K slice is 2048 bytes.
-        return make_sdesc(plane_addr + ks * 2048, BK * 128, 1024, 2);
-    } else {
-        // K-major, rows of BK bf16 (64 or 128 bytes) with the matching swizzle: 8-row
-        // groups are 8 * BK * 2 bytes apart (SBO); a 16-deep K slice is 32 bytes into the row.
-        return make_sdesc(plane_addr + ks * 32, 16, 8 * BK * 2, BK * 2 == 128 ? 2 : 4);
-    }
+// Descriptor of an operand plane at shared address `plane` (first 16-deep K slice) in its
+// layout, and the start-address step (16-byte units) to the next slice.
+__device__ __forceinline__ uint64_t operand_desc(uint32_t plane, bool mn) {
+    // 128B swizzle, MN-major: 64-element MN chunks are BK * 128 bytes apart (LBO), 8-row K
+    // groups 1024 bytes (SBO).  K-major: rows of BK 16-bit values (128 bytes), 8-row groups
+    // 1024 bytes apart (SBO).
+    return mn ? make_sdesc(plane, BK * 128, 1024, 2) : make_sdesc(plane, 16, 8 * BK * 2, 2);
 }
+__device__ __forceinline__ uint32_t slice_step(bool mn) { return mn ? (2048 >> 4) : (32 >> 4); }
+static_assert(BK * 2 == 128, "K-major rows fill one 128-byte swizzle row");
 
 // Symmetric outputs: the t-th of the tiles that touch the upper triangle (col >= row),
 // in row-major order of tiles.
@@ -92,8 +89,9 @@ __device__ __forceinline__ void active_prefix(const GemmParams& p, int* pre) {
     }
 }
 
-// Decodes active tile t for the CTA of rank `crank` in its pair (0 without pairs).
+// Decodes active tile t for the CTA of rank `crank` in its pair.
 // Returns false when the matrix does no work in this launch.
+template <int EPI>
 __device__ __forceinline__ bool decode_tile(const GemmParams& p, const int* pre, int t, uint32_t crank,
                                             TileInfo& ti) {
     int gi = 0;
@@ -126,7 +124,7 @@ __device__ __forceinline__ bool decode_tile(const GemmParams& p, const int* pre,
     ti.hi_only = false;
     // the final Q of a matrix: the polish update, or an ungated launch (the Gram side's
     // Q = Delta Z, which writes only matrices that have a Q)
-    ti.trace = p.epi == kEpiXSplit && g.d_hi != nullptr && p.gate == kGateNone;
+    ti.trace = EPI == kEpiXSplit && g.d_hi != nullptr && p.gate == kGateNone;
     if (g.gate_fb && p.state[ti.mat].final_buf != g.gate_fb - 1) return false;
     if (p.gate != kGateNone) {
         const MatState& st = p.state[ti.mat];
@@ -140,22 +138,22 @@ __device__ __forceinline__ bool decode_tile(const GemmParams& p, const int* pre,
             if (st.mode == 0) return false;
             if (p.gate == kGateQuintic && st.mode != 1) return false;
             if (p.gate == kGatePolish && st.mode != 2) return false;
-            if (p.epi == kEpiPoly && st.mode == 2) ti.run_mma = false;  // cubic polish: no G^2
-            ti.horner = (p.epi == kEpiPoly && p.poly_horner && st.mode == 1);
+            if (EPI == kEpiPoly && st.mode == 2) ti.run_mma = false;  // cubic polish: no G^2
+            ti.horner = (EPI == kEpiPoly && p.poly_horner && st.mode == 1);
             if (p.split_on_polish && st.mode == 2) ti.a_split = ti.b_split = true;  // final step: 3 passes
-            ti.trace = p.epi == kEpiXSplit && g.d_hi != nullptr && p.gate == kGateStep && st.mode == 2;
+            ti.trace = EPI == kEpiXSplit && g.d_hi != nullptr && p.gate == kGateStep && st.mode == 2;
         }
         // precision schedule: single-pass steps.  A Gram only after iteration 0's and only
         // while the last residual is large (>= kOnePassGramResid): a Gram whose test can pass
         // feeds the final polish, which nothing corrects afterwards, so it keeps its passes.
-        const int k = (p.epi == kEpiGram) ? st.step : st.step - 1;
+        const int k = (EPI == kEpiGram) ? st.step : st.step - 1;
         if (k >= g.one_from && k < g.one_to &&
-            ((p.epi == kEpiGram) ? (st.step > 0 && st.resid >= kOnePassGramResid) : st.mode == 1)) {
+            ((EPI == kEpiGram) ? (st.step > 0 && st.resid >= kOnePassGramResid) : st.mode == 1)) {
             ti.a_split = ti.b_split = false;
             // a single-pass Gram never feeds the polish and its polynomial reads G's hi only
-            if (p.epi == kEpiGram) ti.hi_only = true;
+            if (EPI == kEpiGram) ti.hi_only = true;
         }
-        if (p.epi == kEpiXSplit && p.gate == kGateStep && st.mode == 1 && st.x_hi_only) ti.hi_only = true;
+        if (EPI == kEpiXSplit && p.gate == kGateStep && st.mode == 1 && st.x_hi_only) ti.hi_only = true;
         ti.ca = st.a;
         ti.cb = st.b;
         ti.cc = st.c;
@@ -248,6 +246,7 @@ __device__ __forceinline__ void stage_store_block(const uint32_t (&w)[16], const
 // diagonal are skipped, a block above it is also stored transposed at (col, row), and the
 // diagonal block is made symmetric in shared memory (its upper half mirrored) before its
 // single store, so every entry is written once and the matrix is bitwise symmetric.
+template <int EPI>
 __device__ __forceinline__ void tile_epilogue(const GemmParams& p, const TileInfo& ti, uint32_t tacc, bool ok,
                                               int eg, int half, int lane, uint32_t crank, uint8_t* stg,
                                               uint32_t& sseq) {
@@ -258,12 +257,12 @@ __device__ __forceinline__ void tile_epilogue(const GemmParams& p, const TileInf
     const int row = row_base + lane;
     const bool row_ok = row < g.M;
     const bool sym = g.sym != 0;
-    const bool f32_out = (p.epi == kEpiF32) || (p.epi == kEpiGram && g.splits > 1);
-    const bool gram_fused = (p.epi == kEpiGram && g.splits == 1);
+    const bool f32_out = (EPI == kEpiF32) || (EPI == kEpiGram && g.splits > 1);
+    const bool gram_fused = (EPI == kEpiGram && g.splits == 1);
     const bool of16 = p.out_f16 != 0;
     // planes written: hi, lo (if kept; not for a Horner-form P, whose lo plane nobody reads),
     // and for the Gram with p.gram_y the plane Y = yb I + yc G (hi only)
-    const bool write_y = (p.epi == kEpiGram && p.gram_y);
+    const bool write_y = (EPI == kEpiGram && p.gram_y);
     const int nplanes = (ti.horner || ti.hi_only || g.st_lo == nullptr) ? 1 : 2;
     float s_sq = 0.f, s_tr = 0.f, s_dev = 0.f;
     float s_tq = 0.f;  // share of tr(Q^T Delta) (ti.trace)
@@ -290,7 +289,7 @@ __device__ __forceinline__ void tile_epilogue(const GemmParams& p, const TileInf
 #pragma unroll
             for (int j = 0; j < 32; ++j)
                 if (j == d) v[j] += ca;
-        } else if (p.epi == kEpiPoly && row_ok) {
+        } else if (EPI == kEpiPoly && row_ok) {
             const int64_t goff = b * g.bf_batch_stride + static_cast<int64_t>(row) * g.ld_bf + col0;
             const uint16_t* gh = reinterpret_cast<const uint16_t*>(g.g_hi) + goff;
             const uint16_t* gl = reinterpret_cast<const uint16_t*>(g.g_lo) + goff;
@@ -319,7 +318,7 @@ __device__ __forceinline__ void tile_epilogue(const GemmParams& p, const TileInf
 #pragma unroll
             for (int j = 0; j < 32; ++j)
                 if (j == d) v[j] += ca;
-        } else if (p.epi == kEpiXSplit) {
+        } else if (EPI == kEpiXSplit) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) v[j] *= xs;
             if (ti.trace && row_ok) {
@@ -441,8 +440,111 @@ __device__ __forceinline__ void tile_epilogue(const GemmParams& p, const TileInf
     }
 }
 
-// Persistent kernel.  Without pairs, CTA c starts with tile c and claims further tiles
-// from the launch's counter.  With kPairMma the grid is made of clusters of two CTAs
+// Position in the shared-memory ring; one pass around it flips the phase.
+struct RingPos {
+    int stage;
+    uint32_t phase;
+};
+
+// Loads one tile's k-blocks into the ring (one thread of each CTA of the pair): this CTA's
+// rows of A and its half of B's rows, AMN / BMN their layouts.  The bytes of both CTAs
+// complete on rank 0's `full` barriers (shared::cluster address fbar0 of the first).  The
+// wait for the next stage is tested while this stage's loads are issued.  False on a timeout.
+template <bool AMN, bool BMN>
+__device__ __forceinline__ bool load_tile(const GemmGroup& g, const TileInfo& ti, uint32_t sbase, uint32_t stride,
+                                          int nstages, uint64_t* full, uint64_t* empty, uint32_t fbar0,
+                                          uint32_t crank, RingPos& pos) {
+    const CUtensorMap *a_hi = g.a_hi, *a_lo = g.a_lo, *b_hi = g.b_hi, *b_lo = g.b_lo;
+    const bool as = ti.a_split, bs = ti.b_split;
+    const uint32_t off_b = kTileABytes * (as ? 2u : 1u);
+    const uint32_t pair_bytes = 2u * (off_b + kTileBBytes * (bs ? 2u : 1u));
+    const int m0 = ti.m0, nb0 = ti.n0 + static_cast<int>(crank) * kBRows, b = ti.b;
+    const int k_end = ti.kb_end * BK;
+    bool ready = mbar_test(&empty[pos.stage], pos.phase ^ 1u);
+#pragma unroll 1
+    for (int k0 = ti.kb_begin * BK; k0 < k_end; k0 += BK) {
+        const int s = pos.stage;
+        if (!ready && !mbar_wait(&empty[s], pos.phase ^ 1u)) return false;
+        if (++pos.stage == nstages) {
+            pos.stage = 0;
+            pos.phase ^= 1u;
+        }
+        ready = mbar_test(&empty[pos.stage], pos.phase ^ 1u);
+        if (crank == 0) mbar_arrive_expect_tx(&full[s], pair_bytes);
+        const uint32_t fbar = fbar0 + 8u * s;
+        const uint32_t sa = sbase + s * stride, sb = sa + off_b;
+        if (AMN) {
+#pragma unroll
+            for (int c = 0; c < BM / 64; ++c) {
+                tma_load_3d_pair(sa + c * (BK * 128), a_hi, fbar, m0 + 64 * c, k0, b);
+                if (as) tma_load_3d_pair(sa + kTileABytes + c * (BK * 128), a_lo, fbar, m0 + 64 * c, k0, b);
+            }
+        } else {
+            tma_load_3d_pair(sa, a_hi, fbar, k0, m0, b);
+            if (as) tma_load_3d_pair(sa + kTileABytes, a_lo, fbar, k0, m0, b);
+        }
+        if (BMN) {
+#pragma unroll
+            for (int c = 0; c < kBRows / 64; ++c) {
+                tma_load_3d_pair(sb + c * (BK * 128), b_hi, fbar, nb0 + 64 * c, k0, b);
+                if (bs) tma_load_3d_pair(sb + kTileBBytes + c * (BK * 128), b_lo, fbar, nb0 + 64 * c, k0, b);
+            }
+        } else {
+            tma_load_3d_pair(sb, b_hi, fbar, k0, nb0, b);
+            if (bs) tma_load_3d_pair(sb + kTileBBytes, b_lo, fbar, k0, nb0, b);
+        }
+    }
+    return true;
+}
+
+// Issues one tile's MMAs (one thread of rank 0) over nkb k-blocks of the ring: the passes
+// hi hi (+ hi lo_B) (+ lo_A hi) of each 16-deep slice, accumulated in tensor memory at tacc.
+// a_lo, b_lo: low descriptor words of the hi planes in stage 0.  A stage or slice only moves
+// the start address (a 14-bit field; every shared address is below 256 KB, so the sum never
+// carries out of it).  The barrier of the next stage is tested between this stage's MMAs, so
+// that its latency hides behind them: a k-block's four 1-pass MMAs take 512 cycles (128 each,
+// the tensor core's rate), and what the thread does between two k-blocks' MMAs has to stay
+// below the few queued ones.  Measured per 64-deep k-block without loads and epilogue (114 x
+// 1024^3): 390 ns -> 278 ns with one pass, 638 -> 540 with two, 806 -> 805 with three, against
+// the loop that chose the passes per MMA, built 64-bit descriptors and ran under
+// `lane == 0`.  With loads 360 ns: a k-block's 32 KB arrive at ~64 bytes per cycle and SM.
+// False on a timeout.
+template <bool AS, bool BS>
+__device__ __forceinline__ bool issue_tile(uint64_t* full, uint64_t* empty, int nstages, uint32_t stride16, int nkb,
+                                           uint32_t tacc, uint32_t idesc, uint32_t a_lo, uint32_t a_hi,
+                                           uint32_t b_lo, uint32_t b_hi, uint32_t step_a, uint32_t step_b,
+                                           RingPos& pos) {
+    constexpr uint32_t kA16 = kTileABytes >> 4, kB16 = kTileBBytes >> 4;  // hi -> lo plane
+    uint32_t so = pos.stage * stride16;
+    uint32_t acc = 0u;
+    bool ready = mbar_test(&full[pos.stage], pos.phase);
+#pragma unroll 1
+    for (int kb = 0; kb < nkb; ++kb) {
+        const int s = pos.stage;
+        if (!ready && !mbar_wait(&full[s], pos.phase)) return false;
+        tc_fence_after();
+        const uint32_t a = a_lo + so, b = b_lo + so;
+        so += stride16;
+        if (++pos.stage == nstages) {
+            pos.stage = 0;
+            pos.phase ^= 1u;
+            so = 0u;
+        }
+#pragma unroll
+        for (int ks = 0; ks < BK / 16; ++ks) {
+            const uint32_t da = a + ks * step_a, db = b + ks * step_b;
+            umma_16bit_pair(tacc, da, a_hi, db, b_hi, idesc, acc);
+            if (BS) umma_16bit_pair(tacc, da, a_hi, db + kB16, b_hi, idesc, 1u);
+            if (AS) umma_16bit_pair(tacc, da + kA16, a_hi, db, b_hi, idesc, 1u);
+            acc = 1u;
+            if (ks == BK / 16 - 2) ready = mbar_test(&full[pos.stage], pos.phase);
+        }
+        umma_commit_pair_mc(&empty[s], 0x3);  // the stage is free in both CTAs once they have read it
+    }
+    return true;
+}
+
+// Persistent kernel, one instantiation per epilogue.  The grid is made of clusters of two CTAs
 // (ranks 0 and 1, on neighbouring SMs); cluster c processes tiles c, c + clusters, ...
 // and both CTAs walk that sequence together: each loads its rows of A and its half of B,
 // the TMA bytes of both complete on rank 0's `full` barrier, rank 0 alone issues the
@@ -451,6 +553,7 @@ __device__ __forceinline__ void tile_epilogue(const GemmParams& p, const TileInf
 // `tempty`.  The TMA ring runs continuously across tile boundaries, and the accumulator
 // is double buffered in tensor memory (2 x 256 columns): the epilogue of one tile
 // overlaps the MMAs of the next.
+template <int EPI>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_constant__ GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
@@ -467,10 +570,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pre + kMaxGroups + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);  // warp-uniform
     const int lane = threadIdx.x & 31;
-    const uint32_t crank = kPairMma ? cluster_ctarank() : 0u;  // rank in the CTA pair
-    const bool leader = crank == 0;                              // issues the MMAs
+    const uint32_t crank = cluster_ctarank();  // rank in the CTA pair
+    const bool leader = crank == 0;            // issues the MMAs
     // ring geometry of this launch: room for the planes its tiles can load
     const uint32_t stage_stride = kTileABytes * (p.a_split || p.split_on_polish ? 2u : 1u) +
                                   kTileBBytes * (p.b_split || p.split_on_polish ? 2u : 1u);
@@ -483,7 +586,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&tfull[i], 1);
-            mbar_init(&tempty[i], kEpiWarps * (kPairMma ? 2 : 1));  // one arrival per epilogue warp of the pair
+            mbar_init(&tempty[i], kEpiWarps * 2);  // one arrival per epilogue warp of the pair
         }
         mbar_init(drain, 1);
         for (int q = 0; q < kTileQueue; ++q) {
@@ -495,35 +598,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
         fence_mbar_init();
     }
     if (warp == 1) {
-        if (kPairMma) {
-            tmem_alloc_pair(tmem_slot, 2 * kTmemCols);
-            tmem_relinquish_pair();
-        } else {
-            tmem_alloc(tmem_slot, 2 * kTmemCols);
-            tmem_relinquish();
-        }
+        tmem_alloc_pair(tmem_slot, 2 * kTmemCols);
+        tmem_relinquish_pair();
     }
     tc_fence_before();
     __syncthreads();
-    if (kPairMma) cluster_sync();  // both CTAs' barriers exist before either signals the other's
+    cluster_sync();  // both CTAs' barriers exist before either signals the other's
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
-        // ================= TMA producer
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            uint32_t issued_mask = 0, issued_parity = 0;
+        // ================= TMA producer (one thread)
+        if (elect_one()) {
+            const uint32_t sbase = smem_u32(smem);
+            const uint32_t fbar0 = mapa_shared(smem_u32(full), 0);
+            RingPos pos = {0, 0u};
+            bool wrapped = false;  // the ring has been filled once
             int prefetched = -1;
             const int T = pre[p.num_groups];
             int q = 0;
             uint32_t qphase = 0;
-            // first tile; without pairs later ones come from the launch's counter, with pairs
             // cluster c takes tiles c, c + clusters, ... (both CTAs of the pair agree)
-            const int tile_stride = kPairMma ? static_cast<int>(gridDim.x >> 1) : 0;
-            int t = kPairMma ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
-            for (;;) {
+            const int tile_stride = static_cast<int>(gridDim.x >> 1);
+            for (int t = static_cast<int>(blockIdx.x >> 1);; t += tile_stride) {
                 // publish the next tile (or -1: no more) to the MMA and epilogue warps
                 const int tile = (t < T && !*abort_flag) ? t : -1;
                 if (!mbar_wait(&tq_empty[q], qphase ^ 1u)) {
@@ -538,12 +635,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     qphase ^= 1u;
                 }
                 if (tile < 0) break;
-                if (kPairMma)
-                    t += tile_stride;
-                else
-                    t = atomicAdd(p.counter, 1) + static_cast<int>(gridDim.x);  // claimed early
                 TileInfo ti;
-                if (!decode_tile(p, pre, tile, crank, ti) || !ti.run_mma) continue;
+                if (!decode_tile<EPI>(p, pre, tile, crank, ti) || !ti.run_mma) continue;
                 const GemmGroup& g = p.g[ti.gi];
                 if (prefetched != ti.gi) {
                     tma_prefetch_desc(g.a_hi);
@@ -552,55 +645,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     if (ti.b_split) tma_prefetch_desc(g.b_lo);
                     prefetched = ti.gi;
                 }
-                const uint32_t stage_bytes =
-                    kTileABytes * (ti.a_split ? 2u : 1u) + kTileBBytes * (ti.b_split ? 2u : 1u);
-                const int nb0 = ti.n0 + static_cast<int>(crank) * kBRows;  // this CTA's rows of B
-                for (int kb = ti.kb_begin; kb < ti.kb_end; ++kb) {
-                    if (!mbar_wait(&empty[stage], phase ^ 1u)) {
-                        *abort_flag = 1;
-                        atomicOr(p.err, kErrTimeout);
-                        break;
-                    }
-                    uint8_t* sa_hi = smem + stage * stage_stride;
-                    uint8_t* sa_lo = sa_hi + kTileABytes;
-                    uint8_t* sb_hi = sa_hi + kTileABytes * (ti.a_split ? 2u : 1u);
-                    uint8_t* sb_lo = sb_hi + kTileBBytes;
-                    // rank 0's barrier expects the bytes of both CTAs of the pair
-                    if (leader) mbar_arrive_expect_tx(&full[stage], stage_bytes * (kPairMma ? 2u : 1u));
-                    const uint32_t fbar = kPairMma ? mapa_shared(smem_u32(&full[stage]), 0) : 0u;
-                    auto load = [&](uint8_t* dst, const CUtensorMap* map, int c0, int c1) {
-                        if (kPairMma)
-                            tma_load_3d_pair(dst, map, fbar, c0, c1, ti.b);
-                        else
-                            tma_load_3d(dst, map, &full[stage], c0, c1, ti.b);
-                    };
-                    const int k0 = kb * BK;
-                    if (g.a_mn) {
-#pragma unroll
-                        for (int c = 0; c < BM / 64; ++c) {
-                            load(sa_hi + c * (BK * 128), g.a_hi, ti.m0 + 64 * c, k0);
-                            if (ti.a_split) load(sa_lo + c * (BK * 128), g.a_lo, ti.m0 + 64 * c, k0);
-                        }
-                    } else {
-                        load(sa_hi, g.a_hi, k0, ti.m0);
-                        if (ti.a_split) load(sa_lo, g.a_lo, k0, ti.m0);
-                    }
-                    if (g.b_mn) {
-#pragma unroll
-                        for (int c = 0; c < kBRows / 64; ++c) {
-                            load(sb_hi + c * (BK * 128), g.b_hi, nb0 + 64 * c, k0);
-                            if (ti.b_split) load(sb_lo + c * (BK * 128), g.b_lo, nb0 + 64 * c, k0);
-                        }
-                    } else {
-                        load(sb_hi, g.b_hi, k0, nb0);
-                        if (ti.b_split) load(sb_lo, g.b_lo, k0, nb0);
-                    }
-                    issued_mask |= 1u << stage;
-                    issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-                    if (++stage == nstages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
+                bool ok;
+                if (g.a_mn)
+                    ok = g.b_mn ? load_tile<true, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
+                                : load_tile<true, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
+                else
+                    ok = g.b_mn ? load_tile<false, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
+                                : load_tile<false, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
+                wrapped |= pos.phase != 0u || ti.kb_end - ti.kb_begin >= nstages;
+                if (!ok) {
+                    *abort_flag = 1;
+                    atomicOr(p.err, kErrTimeout);
                 }
             }
             if (*abort_flag) {
@@ -608,8 +663,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                 // barriers also count rank 1's copies; rank 1 cannot observe its own, so it
                 // leaves them a generous margin).
                 if (leader) {
+                    // stages before pos were last filled in this pass of the ring, the others in
+                    // the pass before it (if there was one)
                     for (int s = 0; s < nstages; ++s)
-                        if (issued_mask & (1u << s)) (void)mbar_wait(&full[s], (issued_parity >> s) & 1u);
+                        if (s < pos.stage || wrapped) (void)mbar_wait(&full[s], s < pos.stage ? pos.phase : pos.phase ^ 1u);
                 } else {
                     const uint64_t t0 = globaltimer_ns();
                     while (globaltimer_ns() - t0 < 100000ull) {
@@ -618,29 +675,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
             }
         }
     } else if (warp == 1) {
-        // ================= MMA issuer (one thread; with pairs only in rank 0)
-        if (lane == 0 && kPairMma && !leader) {
-            // rank 1 issues no MMAs; it only keeps its tile queue moving
-            int q = 0;
-            uint32_t qphase = 0;
-            for (;;) {
-                if (!mbar_wait(&tq_full[q], qphase)) {
-                    *abort_flag = 1;
-                    atomicOr(p.err, kErrTimeout);
-                    break;
-                }
-                const int tile = tq_tile[q];
-                mbar_arrive(&tq_empty[q]);
-                if (++q == kTileQueue) {
-                    q = 0;
-                    qphase ^= 1u;
-                }
-                if (tile < 0) break;
-            }
-        } else if (lane == 0) {
+        // ================= MMA issuer (one thread of rank 0)
+        if (elect_one()) {
             const uint32_t sbase = smem_u32(smem);
-            int stage = 0;
-            uint32_t phase = 0;
+            RingPos pos = {0, 0u};
             uint32_t n = 0;  // active tiles processed
             int q = 0;
             uint32_t qphase = 0;
@@ -657,8 +695,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     qphase ^= 1u;
                 }
                 if (tile < 0 || *abort_flag) break;
+                if (!leader) continue;  // rank 1 issues no MMAs; it only keeps its tile queue moving
                 TileInfo ti;
-                if (!decode_tile(p, pre, tile, crank, ti)) continue;
+                if (!decode_tile<EPI>(p, pre, tile, crank, ti)) continue;
                 const uint32_t buf = n & 1u, use = n >> 1;
                 ++n;
                 if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u)) {
@@ -667,69 +706,37 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     break;
                 }
                 tc_fence_after();
-                const uint32_t tacc = tmem_base + buf * kTmemCols;
                 if (ti.run_mma) {
                     // instruction and operand descriptors for the layouts of this tile's group
                     const bool a_mn = p.g[ti.gi].a_mn != 0, b_mn = p.g[ti.gi].b_mn != 0;
+                    const bool as = ti.a_split, bs = ti.b_split;
+                    const uint32_t tacc = tmem_base + buf * kTmemCols;
                     const uint32_t idesc = make_idesc_16bit(kTileM, BN, a_mn, b_mn, p.in_f16 != 0);
-                    const uint64_t desc_a0 = a_mn ? operand_desc<true>(sbase, 0) : operand_desc<false>(sbase, 0);
-                    const uint64_t desc_b0 = b_mn ? operand_desc<true>(sbase, 0) : operand_desc<false>(sbase, 0);
-                    // start-address step of one 16-deep K slice: 2048 bytes MN-major, 32 bytes K-major
-                    const uint64_t step_a = a_mn ? (2048 >> 4) : (32 >> 4);
-                    const uint64_t step_b = b_mn ? (2048 >> 4) : (32 >> 4);
-                    // descriptors of this tile's planes in stage 0; a stage or a 16-deep K
-                    // slice only moves the start address (14-bit field in 16-byte units; every
-                    // shared address is below 256 KB, so the sum never carries out of it)
-                    const uint64_t a_hi0 = desc_a0;
-                    const uint64_t a_lo0 = desc_a0 + (kTileABytes >> 4);
-                    const uint64_t b_hi0 = desc_b0 + ((kTileABytes * (ti.a_split ? 2u : 1u)) >> 4);
-                    const uint64_t b_lo0 = b_hi0 + (kTileBBytes >> 4);
-                    const bool bs = ti.b_split, as = ti.a_split;
-                    uint32_t acc = 0u;
-                    for (int kb = ti.kb_begin; kb < ti.kb_end; ++kb) {
-                        if (!mbar_wait(&full[stage], phase)) {
-                            *abort_flag = 1;
-                            atomicOr(p.err, kErrTimeout);
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint64_t so = static_cast<uint64_t>(stage) * (stage_stride >> 4);
-#pragma unroll
-                        for (int ks = 0; ks < BK / 16; ++ks) {
-                            const uint64_t da = so + ks * step_a, db = so + ks * step_b;
-                            if (kPairMma) {
-                                umma_16bit_pair(tacc, a_hi0 + da, b_hi0 + db, idesc, acc);
-                                if (bs) umma_16bit_pair(tacc, a_hi0 + da, b_lo0 + db, idesc, 1u);
-                                if (as) umma_16bit_pair(tacc, a_lo0 + da, b_hi0 + db, idesc, 1u);
-                            } else {
-                                umma_16bit(tacc, a_hi0 + da, b_hi0 + db, idesc, acc);
-                                if (bs) umma_16bit(tacc, a_hi0 + da, b_lo0 + db, idesc, 1u);
-                                if (as) umma_16bit(tacc, a_lo0 + da, b_hi0 + db, idesc, 1u);
-                            }
-                            acc = 1u;
-                        }
-                        // the stage is free in both CTAs once these MMAs have read it
-                        if (kPairMma)
-                            umma_commit_pair_mc(&empty[stage], 0x3);
-                        else
-                            umma_commit(&empty[stage]);
-                        if (++stage == nstages) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
+                    const uint64_t da = operand_desc(sbase, a_mn);
+                    const uint64_t db = operand_desc(sbase + kTileABytes * (as ? 2u : 1u), b_mn);
+                    const uint32_t a_lo = static_cast<uint32_t>(da), a_hi = static_cast<uint32_t>(da >> 32);
+                    const uint32_t b_lo = static_cast<uint32_t>(db), b_hi = static_cast<uint32_t>(db >> 32);
+                    const uint32_t sa = slice_step(a_mn), sb = slice_step(b_mn), st16 = stage_stride >> 4;
+                    const int nkb = ti.kb_end - ti.kb_begin;
+                    bool ok;
+                    if (as)
+                        ok = bs ? issue_tile<true, true>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos)
+                                : issue_tile<true, false>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos);
+                    else
+                        ok = bs ? issue_tile<false, true>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos)
+                                : issue_tile<false, false>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos);
+                    if (!ok) {
+                        *abort_flag = 1;
+                        atomicOr(p.err, kErrTimeout);
                     }
                 }
                 // completes once every MMA of this tile has finished (in both CTAs' barriers)
-                if (kPairMma)
-                    umma_commit_pair_mc(&tfull[buf], 0x3);
-                else
-                    umma_commit(&tfull[buf]);
+                umma_commit_pair_mc(&tfull[buf], 0x3);
             }
-            if (kPairMma)
+            if (leader) {
                 umma_commit_pair(drain);
-            else
-                umma_commit(drain);
-            (void)mbar_wait(drain, 0);
+                (void)mbar_wait(drain, 0);
+            }
         }
     } else {
         // ================= epilogue (warps 2..9): warp w reads TMEM lanes 32 (w % 4) ..,
@@ -762,7 +769,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
             }
             if (tile < 0) break;
             TileInfo ti;
-            if (!decode_tile(p, pre, tile, crank, ti)) continue;
+            if (!decode_tile<EPI>(p, pre, tile, crank, ti)) continue;
             const uint32_t buf = n & 1u, use = n >> 1;
             ++n;
             const bool ok = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], use & 1u));
@@ -772,7 +779,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
             }
             __syncwarp();
             tc_fence_after();
-            tile_epilogue(p, ti, tmem_base + buf * kTmemCols, ok, eg, half, lane, crank,
+            tile_epilogue<EPI>(p, ti, tmem_base + buf * kTmemCols, ok, eg, half, lane, crank,
                           staging + (warp - 2) * kStageBlocks * kStageBlockBytes, sseq);
             tc_fence_before();
             __syncwarp();
@@ -787,73 +794,70 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
         __syncwarp();
     }
 
-    // ---- teardown: the MMA thread has waited for all its MMAs (drain barrier); with
-    // pairs neither CTA leaves (or frees tensor memory) while rank 0's MMAs could still
-    // read rank 1's shared memory or write its tensor memory
+    // ---- teardown: the MMA thread has waited for all its MMAs (drain barrier); neither CTA
+    // leaves (or frees tensor memory) while rank 0's MMAs could still read rank 1's shared
+    // memory or write its tensor memory
     tc_fence_before();
     __syncthreads();
-    if (kPairMma) cluster_sync();
+    cluster_sync();
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
-        if (kPairMma)
-            tmem_dealloc_pair(tmem_base, 2 * kTmemCols);
-        else
-            tmem_dealloc(tmem_base, 2 * kTmemCols);
+        tmem_dealloc_pair(tmem_base, 2 * kTmemCols);
     }
 }
 
 // ------------------------------------------------------------------ host launcher
-// Launches one persistent GEMM over the groups of `p` (p.total_tiles output tiles) on at
-// most `max_ctas` CTAs (one per SM; with kPairMma, clusters of two CTAs per tile).
-cudaError_t launch_gemm(const GemmParams& p, int max_ctas, cudaStream_t stream) {
-    if (p.total_tiles <= 0) return cudaSuccess;
-    static int max_clusters = 0;  // clusters of two that can be resident at once
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kGemmSmemBytes);
-        if (e != cudaSuccess) return e;
-        if (kPairMma) {
-            cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeClusterDimension;
-            at[0].val.clusterDim.x = 2;
-            at[0].val.clusterDim.y = 1;
-            at[0].val.clusterDim.z = 1;
-            cfg.gridDim = dim3(static_cast<unsigned>(max_ctas & ~1));
-            cfg.blockDim = dim3(kGemmThreads);
-            cfg.dynamicSmemBytes = kGemmSmemBytes;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            int n = 0;
-            e = cudaOccupancyMaxActiveClusters(&n, k_gemm_split, &cfg);
-            if (e != cudaSuccess) return e;
-            max_clusters = n > 0 ? n : 1;
-        }
-        attr_set = true;
-    }
-    if (!kPairMma) {
-        const int grid = p.total_tiles < max_ctas ? p.total_tiles : max_ctas;
-        k_gemm_split<<<grid, kGemmThreads, kGemmSmemBytes, stream>>>(p);
-        return cudaGetLastError();
-    }
-    int clusters = p.total_tiles;
-    clusters = clusters < max_clusters ? clusters : max_clusters;
-    clusters = clusters < max_ctas / 2 ? clusters : (max_ctas / 2 > 0 ? max_ctas / 2 : 1);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+namespace {
+
+cudaLaunchConfig_t pair_config(unsigned grid, cudaStream_t stream, cudaLaunchAttribute* at) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(static_cast<unsigned>(2 * clusters));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(kGemmThreads);
     cfg.dynamicSmemBytes = kGemmSmemBytes;
     cfg.stream = stream;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_gemm_split, p);
+    return cfg;
+}
+
+template <int EPI>
+cudaError_t launch_epi(const GemmParams& p, int max_ctas, cudaStream_t stream) {
+    static int max_clusters = 0;  // clusters of two that can be resident at once
+    cudaLaunchAttribute at[1];
+    if (!max_clusters) {
+        cudaError_t e = cudaFuncSetAttribute(k_gemm_split<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kGemmSmemBytes);
+        if (e != cudaSuccess) return e;
+        const cudaLaunchConfig_t cfg = pair_config(static_cast<unsigned>(max_ctas & ~1), stream, at);
+        int n = 0;
+        e = cudaOccupancyMaxActiveClusters(&n, k_gemm_split<EPI>, &cfg);
+        if (e != cudaSuccess) return e;
+        max_clusters = n > 0 ? n : 1;
+    }
+    int clusters = p.total_tiles;
+    clusters = clusters < max_clusters ? clusters : max_clusters;
+    clusters = clusters < max_ctas / 2 ? clusters : (max_ctas / 2 > 0 ? max_ctas / 2 : 1);
+    const cudaLaunchConfig_t cfg = pair_config(static_cast<unsigned>(2 * clusters), stream, at);
+    return cudaLaunchKernelEx(&cfg, k_gemm_split<EPI>, p);
+}
+
+}  // namespace
+
+// Launches one persistent GEMM over the groups of `p` (p.total_tiles output tiles) on at
+// most `max_ctas` CTAs (one per SM, in clusters of two).
+cudaError_t launch_gemm(const GemmParams& p, int max_ctas, cudaStream_t stream) {
+    if (p.total_tiles <= 0) return cudaSuccess;
+    switch (p.epi) {
+        case kEpiF32: return launch_epi<kEpiF32>(p, max_ctas, stream);
+        case kEpiPoly: return launch_epi<kEpiPoly>(p, max_ctas, stream);
+        case kEpiXSplit: return launch_epi<kEpiXSplit>(p, max_ctas, stream);
+        default: return launch_epi<kEpiGram>(p, max_ctas, stream);
+    }
 }
 
 }  // namespace isoloco

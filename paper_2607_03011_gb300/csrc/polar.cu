@@ -552,15 +552,16 @@ __global__ void __launch_bounds__(256) k_trace_final(const MatDesc* __restrict__
     }
 }
 
-// Resets the per-matrix state before a step: every matrix is active for the first Gram,
-// and the GEMM launches' tile counters restart at zero.
+// Resets the per-matrix state before a step: every matrix is active for the first Gram.
 __global__ void k_reset_state(MatState* state, int nmat, uint32_t* err, const MatDesc* __restrict__ mats,
                               const int* __restrict__ bucket_first, const int* __restrict__ bucket_count,
                               int nbuckets, int* __restrict__ list_gram, int* __restrict__ cnt_gram,
-                              int* __restrict__ counters, int ncounters) {
+                              int* __restrict__ ticket) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) *err = 0u;
-    for (int c = i; c < ncounters; c += gridDim.x * blockDim.x) counters[c] = 0;
+    if (i == 0) {
+        *err = 0u;
+        *ticket = 0;
+    }
     if (i < nbuckets) cnt_gram[i] = bucket_count[i];
     if (i < nmat) list_gram[i] = i - bucket_first[mats[i].bucket];
     if (i >= nmat) return;

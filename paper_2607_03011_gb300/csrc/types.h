@@ -9,10 +9,10 @@ namespace isoloco {
 
 // ------------------------------------------------------------------ GEMM tiles
 // One CTA holds a BM x BN fp32 tile in tensor memory, computed from 16-bit hi/lo
-// operand planes staged BK deep per pipeline stage.  With kPairMma a pair of CTAs on
-// neighbouring SMs (a cluster of two) computes one kTileM x BN = 256 x 256 output tile
-// with tcgen05 cta_group::2: each CTA stages its own BM rows of A and half of B's BN
-// rows, so an SM loads and stages 8 KB instead of 12 KB per 16-deep MMA step.
+// operand planes staged BK deep per pipeline stage.  A pair of CTAs on neighbouring SMs (a
+// cluster of two) computes one kTileM x BN = 256 x 256 output tile with tcgen05
+// cta_group::2: each CTA stages its own BM rows of A and half of B's BN rows, so an SM
+// loads and stages 8 KB instead of 12 KB per 16-deep MMA step.
 // BK = 64: one TMA instruction moves twice the bytes of a 32-deep stage; with 32-deep
 // stages the single producer thread's issue rate held back the MN-major operands (a Gram
 // stage needs six 64 x 32 boxes).
@@ -21,7 +21,7 @@ constexpr int BM = 128;
 constexpr int BN = 256;
 constexpr int BK = 64;
 constexpr int kTileM = kPairMma ? 2 * BM : BM;  // rows of one output tile
-constexpr int kBRows = kPairMma ? BN / 2 : BN;  // rows of B (N extent) staged by one CTA
+constexpr int kBRows = BN / 2;  // rows of B (N extent) staged by one CTA
 // Shared-memory ring of the persistent GEMM (one CTA per SM): as many stages of the
 // launch's plane set as fit in kRingBytes, at most kMaxStages.
 constexpr int kMaxStages = 12;
@@ -30,7 +30,7 @@ constexpr int kTileABytes = BM * BK * 2;                       // one bf16 plane
 constexpr int kTileBBytes = kBRows * BK * 2;                   // one bf16 plane of this CTA's B
 
 constexpr int kEpiWarps = 8;       // two warps per tensor-memory lane quarter
-constexpr int kPartSlots = kEpiWarps * (kPairMma ? 2 : 1);  // Gram partial sums per output tile
+constexpr int kPartSlots = kEpiWarps * 2;  // Gram partial sums per output tile
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 MMA, warps 2.. epilogue
 constexpr int kTmemCols = 256;     // one accumulator; the kernel double-buffers (512 columns)
 constexpr int kMaxGroups = 8;
@@ -159,7 +159,6 @@ struct GemmParams {
     // matrices list[g.mat_base + j], j < cnt[g.bucket] (indices within the group).
     const int* list;
     const int* cnt;
-    int* counter;         // dynamic tile scheduler of this launch (zeroed before the step)
     int epi;
     int gate;
     int in_f16;           // operand planes are fp16 (else bf16); also the G planes of kEpiPoly
