@@ -322,7 +322,11 @@ enum {
 /* Per-phase timing.  enable != 0 makes every later call record a CUDA event pair
  * around each phase's launches on the call's stream (a few microseconds of
  * overhead per launch); enabling or disabling resets the accumulators and
- * synchronizes the device.  Launch counts accumulate whether or not timing is on. */
+ * synchronizes the device.  Launch counts accumulate whether or not timing is on.  The polar
+ * iterations that run inside one kernel are timed by that kernel (device timer): their
+ * phases then run one after the other instead of overlapping, a phase's time counts to its
+ * last tile's arrival (the Gram's includes the control steps), and the kernel counts as one
+ * launch of GRAM. */
 int isoloco_profile_enable(isoloco_plan_t plan, int enable);
 
 /* Synchronizes `stream`, then writes the accumulated milliseconds and launch

@@ -3,7 +3,8 @@
 //
 // One IsoLoCo outer step (Alg. 2) on a stream:
 //   k_reset_state -> k_reduce (Delta, all tensors)
-//   for t = 0..max_iter:   Gram X^T X (tcgen05) -> k_gram_finalize -> k_control
+//   for t = 0..max_iter (t >= 1 inside one kernel, k_polar_loop):
+//                          Gram X^T X (tcgen05) -> k_gram_finalize -> k_control
 //                          -> G^2 with P = a I + b G + c G^2 epilogue (tcgen05)
 //                          -> X P (tcgen05)  [matrices that finished exit at once; the
 //                             polish's epilogue also sums tr(Q^T Delta)]
@@ -22,6 +23,7 @@
 
 #include "common.cuh"
 #include "isoloco.h"
+#include "polar_loop.h"
 #include "types.h"
 
 namespace isoloco {
@@ -44,13 +46,13 @@ __global__ void k_gs_final_prep(const MatDesc*, MatState*, const int*, const __n
 __global__ void k_gs_final_flip(MatState*, const int*, int);
 __global__ void k_control(const MatDesc*, int, MatState*, const float*, int, int, float, uint32_t*, const int*,
                           const int*, int, int*, int*, int*, int*, cudaGraphConditionalHandle, int, long long*,
-                          int, int*, int4, int4, int);
+                          int, int*, int4, int4, int, uint32_t*);
 __global__ void k_trace_partial(const MatDesc*, const int4*, int, const MatState*, const __nv_bfloat16*,
                                 const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*,
                                 const __nv_bfloat16*, const __nv_bfloat16*, double*);
 __global__ void k_trace_final(const MatDesc*, int, MatState*, const double*, const double*);
 __global__ void k_reset_state(MatState*, int, uint32_t*, const MatDesc*, const int*, const int*, int, int*, int*,
-                              int*);
+                              int*, uint32_t*);
 __global__ void k_reduce(const Chunk*, const MatDesc*, ReplicaPtrs, int, int, const float*, float,
                          __nv_bfloat16*, __nv_bfloat16*, float*, uint32_t*);
 __global__ void k_reduce_f32(const Chunk*, const MatDesc*, ReplicaPtrs, int, const float*, float, __nv_bfloat16*,
@@ -178,6 +180,15 @@ struct isoloco_plan {
     int* list_step = nullptr;
     int* cnt_step = nullptr;
     int* ticket = nullptr;
+    // the polar loop's control words and arrival counters, and its tables (polar_loop.h), built
+    // for one kind of call (loop_key) and rebuilt when it changes
+    uint32_t* ctl = nullptr;
+    uint32_t* arr = nullptr;
+    std::vector<LoopGroup> loop_groups;
+    LoopPhase loop_phases[2 * kLoopPhases] = {};
+    unsigned long long* loop_prof = nullptr;  // per-phase nanoseconds (phase profiling)
+    int loop_clusters = 0;
+    long long loop_key[3] = {-1, -1, -2};
     int64_t* gpart_off_d = nullptr;
     int64_t* gpart_sstride_d = nullptr;
     int* nsplit_d = nullptr;
@@ -588,7 +599,9 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
         (rc = dalloc(p, &p->bucket_count_d, (int64_t)p->buckets.size())) ||
         (rc = dalloc(p, &p->cnt_gram, (int64_t)p->buckets.size())) ||
         (rc = dalloc(p, &p->cnt_step, (int64_t)p->buckets.size())) ||
-        (rc = dalloc(p, &p->ticket, 1)) || (rc = dalloc(p, &p->loopc, 2)) ||
+        (rc = dalloc(p, &p->ticket, 1)) || (rc = dalloc(p, &p->ctl, p->nmat)) ||
+        (rc = dalloc(p, &p->arr, (int64_t)kArrKinds * p->nmat)) ||
+        (rc = dalloc(p, &p->loop_prof, kLoopPhases)) || (rc = dalloc(p, &p->loopc, 2)) ||
         (rc = dalloc(p, &p->tmaps_d, (int64_t)kMapsPerBucket * std::max<size_t>(1, p->buckets.size()))) ||
         (rc = dalloc(p, &p->anhi, gs_elems)) || (rc = dalloc(p, &p->anlo, gs_elems)) ||
         (rc = dalloc(p, &p->whi, gs_elems)) || (rc = dalloc(p, &p->wlo, gs_elems)) ||
@@ -608,6 +621,7 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
                                       2 * p->K * 256 * 4));
     CUDA_TRY(cudaStreamCreateWithFlags(&p->cap_st, cudaStreamNonBlocking));
     CUDA_TRY(cudaMemset(p->loopc, 0, 2 * sizeof(long long)));
+    CUDA_TRY(cudaMemset(p->loop_prof, 0, sizeof(unsigned long long) * kLoopPhases));
     // zero the planes once so that padding columns hold zeros
     for (void* a : {(void*)p->dhi, (void*)p->dlo, (void*)p->xhi[0], (void*)p->xlo[0], (void*)p->xhi[1],
                     (void*)p->xlo[1]})
@@ -839,93 +853,73 @@ static void set_one_pass(const isoloco_plan* p, GemmGroup& g, const Bucket& bk, 
     g.one_to = full ? 0 : (update ? p->up_to[kind] : p->gp_to[kind]);
 }
 
-// Iteration t of the polar loop for every matrix still active: Gram, convergence test
-// and choice of the step (k_control), polynomial, update.  With set_cond, k_control also
-// sets the graph condition `cond` (graph body only).
-static int polar_iteration(isoloco_plan* p, int t, int max_iter, float tol, cudaStream_t st,
-                           cudaGraphConditionalHandle cond, int set_cond) {
+// The GEMM launches of one iteration of the polar loop: per shape bucket a group in each phase.
+struct IterSets {
+    LaunchSet w, gram_gs;  // Gram-side buckets after iteration 0
+    LaunchSet gram, poly, update;
+};
+
+static bool gram_side_on(const isoloco_plan* p) { return p->n_gs > 0 && !(p->fast_steps > 0 || p->full_prec); }
+
+static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
     const CUtensorMap* maps = p->tmaps_d;
-    {
-        const int src = (t == 0) ? 0 : 1 + (t & 1);  // Delta, X0 or X1 as the current iterate
-        const int dst = (t + 1) & 1;
-        // ---- Gram G = X^T X (tall, MN-major operands) or X X^T (wide, K-major)
-        const bool first = (t == 0);
-        // The fast variant stops after a fixed number of steps, so nothing corrects a step's
-        // rounding afterwards: every step splits both operands (fp16 three passes) and the
-        // polynomial is formed from G's hi/lo planes (no single-plane Y).  So does the clip
-        // variants' sign iteration (full_prec): there a single-plane rounding perturbs the
-        // invariant subspaces the result must separate, which later steps do not undo.  The
-        // converging path keeps one operand single from iteration 1 on (its rounding only
-        // perturbs the spectrum, which later steps correct).
-        const bool full = p->fast_steps > 0 || p->full_prec;
-        const bool gs_on = p->n_gs > 0 && !full;  // Gram-side buckets iterate on n x n matrices
-        const Precision gram_pr = first ? Precision{0, 0, 1, 1, 0}
-                                        : (full ? Precision{1, 1, 1, 1, 0} : Precision{1, 1, 1, 0, 0});
-        // Tall and wide matrices share one launch (their tiles pack into fewer waves).
-        LaunchSet gram;
-        init_set(gram, kEpiGram, kGateActive, p, gram_pr);
-        gram.p.gram_y = (first || full) ? 0 : 1;
-        // Gram-side buckets after iteration 0 (gramside.cu): W = A Z, then G = Z^T W, both with
-        // three passes in launches of their own (a split B operand would thin the main Gram's ring)
-        const bool gs_iter = gs_on && !first;
-        LaunchSet wset, gsg;
-        if (gs_iter) {
-            init_set(wset, kEpiXSplit, kGateActive, p, Precision{1, 1, 1, 1, 0});
-            wset.p.unit_scale = 1;
-            init_set(gsg, kEpiGram, kGateActive, p, Precision{1, 1, 1, 1, 0});
-            gsg.p.gram_y = 1;
-        }
-        for (size_t b = 0; b < p->buckets.size(); ++b) {
-            const Bucket& bk = p->buckets[b];
-            const CUtensorMap* m = maps + b * kMapsPerBucket;
-            GemmGroup g{};
-            if (gs_iter && bk.gs) {
-                const int zb = t & 1;  // ping-pong buffer holding Z_t
-                GemmGroup w{};
-                w.a_hi = m + an_map(0);
-                w.a_lo = m + an_map(1);
-                w.b_hi = m + z_map(zb, 1, 0);
-                w.b_lo = m + z_map(zb, 1, 1);
-                set_group_common(w, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
-                w.bucket = (int)b;
-                w.out_hi = p->whi + bk.gs_off;
-                w.out_lo = p->wlo + bk.gs_off;
-                w.st_hi = m + w_st_map(0);
-                w.st_lo = m + w_st_map(1);
-                w.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
-                w.ld_bf = bk.ld_n;
-                wset.add(w, false, true);
-                g.a_hi = m + z_map(zb, 1, 0);
-                g.a_lo = m + z_map(zb, 1, 1);
-                g.b_hi = m + w_mn_map(0);
-                g.b_lo = m + w_mn_map(1);
-                set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
-                g.bucket = (int)b;
-                g.out_hi = p->ghi + bk.gplane_off;
-                g.out_lo = p->glo + bk.gplane_off;
-                g.st_hi = m + st_map(2, 0);
-                g.st_lo = m + st_map(2, 1);
-                g.st_y = m + y_st_map();
-                g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
-                g.ld_bf = bk.ld_n;
-                g.part = p->fin_part;
-                g.part_base = p->mats_h[bk.mat_base].gpart_slot;
-                set_sym(g, bk.n);
-                gsg.add(g, true, true);
-                continue;
-            }
-            const int role_a = bk.tall ? kRoleMN : kRoleKA;
-            const int role_b = bk.tall ? kRoleMN : kRoleKB;
-            g.a_hi = m + src_map(src, role_a, 0);
-            g.a_lo = m + src_map(src, role_a, 1);
-            g.b_hi = m + src_map(src, role_b, 0);
-            g.b_lo = m + src_map(src, role_b, 1);
-            set_group_common(g, bk.n, bk.n, bk.tall ? bk.rows : bk.cols, bk.count, bk.splits, bk.mat_base);
+    const int src = (t == 0) ? 0 : 1 + (t & 1);  // Delta, X0 or X1 as the current iterate
+    const int dst = (t + 1) & 1;
+    // ---- Gram G = X^T X (tall, MN-major operands) or X X^T (wide, K-major)
+    const bool first = (t == 0);
+    // The fast variant stops after a fixed number of steps, so nothing corrects a step's
+    // rounding afterwards: every step splits both operands (fp16 three passes) and the
+    // polynomial is formed from G's hi/lo planes (no single-plane Y).  So does the clip
+    // variants' sign iteration (full_prec): there a single-plane rounding perturbs the
+    // invariant subspaces the result must separate, which later steps do not undo.  The
+    // converging path keeps one operand single from iteration 1 on (its rounding only
+    // perturbs the spectrum, which later steps correct).
+    const bool full = p->fast_steps > 0 || p->full_prec;
+    const bool gs_on = gram_side_on(p);  // Gram-side buckets iterate on n x n matrices
+    const Precision gram_pr = first ? Precision{0, 0, 1, 1, 0}
+                                    : (full ? Precision{1, 1, 1, 1, 0} : Precision{1, 1, 1, 0, 0});
+    // Tall and wide matrices share one launch (their tiles pack into fewer waves).
+    LaunchSet& gram = s.gram;
+    init_set(gram, kEpiGram, kGateActive, p, gram_pr);
+    gram.p.gram_y = (first || full) ? 0 : 1;
+    // Gram-side buckets after iteration 0 (gramside.cu): W = A Z, then G = Z^T W, both with
+    // three passes in launches of their own (a split B operand would thin the main Gram's ring)
+    const bool gs_iter = gs_on && !first;
+    LaunchSet &wset = s.w, &gsg = s.gram_gs;
+    wset.groups.clear();
+    gsg.groups.clear();
+    if (gs_iter) {
+        init_set(wset, kEpiXSplit, kGateActive, p, Precision{1, 1, 1, 1, 0});
+        wset.p.unit_scale = 1;
+        init_set(gsg, kEpiGram, kGateActive, p, Precision{1, 1, 1, 1, 0});
+        gsg.p.gram_y = 1;
+    }
+    for (size_t b = 0; b < p->buckets.size(); ++b) {
+        const Bucket& bk = p->buckets[b];
+        const CUtensorMap* m = maps + b * kMapsPerBucket;
+        GemmGroup g{};
+        if (gs_iter && bk.gs) {
+            const int zb = t & 1;  // ping-pong buffer holding Z_t
+            GemmGroup w{};
+            w.a_hi = m + an_map(0);
+            w.a_lo = m + an_map(1);
+            w.b_hi = m + z_map(zb, 1, 0);
+            w.b_lo = m + z_map(zb, 1, 1);
+            set_group_common(w, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
+            w.bucket = (int)b;
+            w.out_hi = p->whi + bk.gs_off;
+            w.out_lo = p->wlo + bk.gs_off;
+            w.st_hi = m + w_st_map(0);
+            w.st_lo = m + w_st_map(1);
+            w.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
+            w.ld_bf = bk.ld_n;
+            wset.add(w, false, true);
+            g.a_hi = m + z_map(zb, 1, 0);
+            g.a_lo = m + z_map(zb, 1, 1);
+            g.b_hi = m + w_mn_map(0);
+            g.b_lo = m + w_mn_map(1);
+            set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
-            g.out_f32 = p->gpart + bk.gpart_off;
-            g.f32_batch_stride = (int64_t)bk.n * bk.ld_n;
-            g.f32_split_stride = (int64_t)bk.count * bk.n * bk.ld_n;
-            g.ld_f32 = bk.ld_n;
             g.out_hi = p->ghi + bk.gplane_off;
             g.out_lo = p->glo + bk.gplane_off;
             g.st_hi = m + st_map(2, 0);
@@ -936,130 +930,253 @@ static int polar_iteration(isoloco_plan* p, int t, int max_iter, float tol, cuda
             g.part = p->fin_part;
             g.part_base = p->mats_h[bk.mat_base].gpart_slot;
             set_sym(g, bk.n);
-            set_one_pass(p, g, bk, false);
-            gram.add(g, bk.tall, bk.tall);
+            gsg.add(g, true, true);
+            continue;
         }
-        int rc;
-        if (gs_iter && ((rc = flush_set(p, ISOLOCO_PHASE_GRAM, wset, st)) ||
-                        (rc = flush_set(p, ISOLOCO_PHASE_GRAM, gsg, st))))
-            return rc;
-        if ((rc = flush_set(p, ISOLOCO_PHASE_GRAM, gram, st))) return rc;
-        // after iteration 0 the Gram-side matrices need no finalize: skip an empty launch
-        if (p->nftiles && (first || !gs_on || p->nftiles_reg > 0)) {
-            PhaseTimer tm(p, ISOLOCO_PHASE_FINALIZE, st);
-            k_gram_finalize<<<p->nftiles, 256, 0, st>>>(p->mats_d, p->ftiles, p->state, p->gpart, p->gpart_off_d,
-                                                        p->gpart_sstride_d, p->nsplit_d, p->ghi, p->glo,
-                                                        p->fin_part, first ? 0 : 1, (first || full) ? nullptr : p->ypl,
-                                                        (!first && gs_on) ? 1 : 0);
-            CUDA_TRY(cudaGetLastError());
-        }
-        { PhaseTimer tm(p, ISOLOCO_PHASE_CONTROL, st);
-        k_control<<<(p->nmat + kControlThreads / 32 - 1) / (kControlThreads / 32), kControlThreads, 0, st>>>(p->mats_d, p->nmat, p->state, p->fin_part, t, max_iter, tol, p->err_d,
-                                      p->bucket_first_d, p->bucket_count_d, (int)p->buckets.size(), p->list_gram,
-                                      p->cnt_gram, p->list_step, p->cnt_step, cond, set_cond, p->loopc,
-                                      p->fast_steps, p->ticket,
-                                      make_int4(gp_one(p, 0, 0), gp_one(p, 0, 1), gp_one(p, 1, 0), gp_one(p, 1, 1)),
-                                      make_int4(up_one(p, 0, 0), up_one(p, 0, 1), up_one(p, 1, 0), up_one(p, 1, 1)), gs_on ? 1 : 0); }
-        CUDA_TRY(cudaGetLastError());
-        // ---- P = a I + b G + c G^2
-        LaunchSet poly;
-        init_set(poly, kEpiPoly, kGateStep, p,
-                 first ? Precision{0, 0, 1, 1, 0} : (full ? Precision{1, 1, 1, 1, 0} : Precision{1, 1, 1, 0, 0}));
-        poly.p.poly_horner = (first || full) ? 0 : 1;
-        for (size_t b = 0; b < p->buckets.size(); ++b) {
-            const Bucket& bk = p->buckets[b];
-            const CUtensorMap* m = maps + b * kMapsPerBucket;
-            GemmGroup g{};
-            g.a_hi = m + g_map(kRoleKA, 0);
-            g.a_lo = m + g_map(kRoleKA, 1);
-            g.b_hi = (first || full) ? m + g_map(kRoleKB, 0) : m + y_map();  // G G or G Y (Horner)
-            g.b_lo = m + g_map(kRoleKB, 1);
+        const int role_a = bk.tall ? kRoleMN : kRoleKA;
+        const int role_b = bk.tall ? kRoleMN : kRoleKB;
+        g.a_hi = m + src_map(src, role_a, 0);
+        g.a_lo = m + src_map(src, role_a, 1);
+        g.b_hi = m + src_map(src, role_b, 0);
+        g.b_lo = m + src_map(src, role_b, 1);
+        set_group_common(g, bk.n, bk.n, bk.tall ? bk.rows : bk.cols, bk.count, bk.splits, bk.mat_base);
+        g.bucket = (int)b;
+        g.out_f32 = p->gpart + bk.gpart_off;
+        g.f32_batch_stride = (int64_t)bk.n * bk.ld_n;
+        g.f32_split_stride = (int64_t)bk.count * bk.n * bk.ld_n;
+        g.ld_f32 = bk.ld_n;
+        g.out_hi = p->ghi + bk.gplane_off;
+        g.out_lo = p->glo + bk.gplane_off;
+        g.st_hi = m + st_map(2, 0);
+        g.st_lo = m + st_map(2, 1);
+        g.st_y = m + y_st_map();
+        g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
+        g.ld_bf = bk.ld_n;
+        g.part = p->fin_part;
+        g.part_base = p->mats_h[bk.mat_base].gpart_slot;
+        set_sym(g, bk.n);
+        set_one_pass(p, g, bk, false);
+        gram.add(g, bk.tall, bk.tall);
+    }
+    // ---- P = a I + b G + c G^2
+    LaunchSet& poly = s.poly;
+    init_set(poly, kEpiPoly, kGateStep, p,
+             first ? Precision{0, 0, 1, 1, 0} : (full ? Precision{1, 1, 1, 1, 0} : Precision{1, 1, 1, 0, 0}));
+    poly.p.poly_horner = (first || full) ? 0 : 1;
+    for (size_t b = 0; b < p->buckets.size(); ++b) {
+        const Bucket& bk = p->buckets[b];
+        const CUtensorMap* m = maps + b * kMapsPerBucket;
+        GemmGroup g{};
+        g.a_hi = m + g_map(kRoleKA, 0);
+        g.a_lo = m + g_map(kRoleKA, 1);
+        g.b_hi = (first || full) ? m + g_map(kRoleKB, 0) : m + y_map();  // G G or G Y (Horner)
+        g.b_lo = m + g_map(kRoleKB, 1);
+        set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
+        g.bucket = (int)b;
+        g.out_hi = p->phi + bk.gplane_off;
+        g.out_lo = p->plo + bk.gplane_off;
+        g.st_hi = m + st_map(3, 0);
+        g.st_lo = m + st_map(3, 1);
+        g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
+        g.ld_bf = bk.ld_n;
+        g.g_hi = p->ghi + bk.gplane_off;
+        g.g_lo = p->glo + bk.gplane_off;
+        set_sym(g, bk.n);
+        set_one_pass(p, g, bk, false);
+        poly.add(g, false, false);
+    }
+    // ---- X_{t+1} = xscale * X_t P (tall) or P X_t (wide), one launch
+    // X_{t+1} is always written as fp16 planes; X is the split operand (A when tall,
+    // B when wide), P the single one except in the polish step (3 passes) and in
+    // iteration 0 and the full-precision paths (both split)
+    LaunchSet& upd = s.update;
+    init_set(upd, kEpiXSplit, kGateStep, p,
+             first ? Precision{0, 1, 0, 0, 0} : (full ? Precision{1, 1, 0, 0, 0} : Precision{1, 1, 0, 0, 1}));
+    const bool p_split = first || full;
+    for (size_t b = 0; b < p->buckets.size(); ++b) {
+        const Bucket& bk = p->buckets[b];
+        const CUtensorMap* m = maps + b * kMapsPerBucket;
+        GemmGroup g{};
+        if (gs_on && bk.gs) {
+            if (first) continue;  // Z_1 = P_0: k_gs_init below
+            // Z_{t+1} = Z_t P_t in the first n rows of the other buffer
+            g.a_hi = m + z_map(t & 1, 0, 0);
+            g.a_lo = m + z_map(t & 1, 0, 1);
+            g.b_hi = m + p_map(kRoleKB, 0);
+            g.b_lo = m + p_map(kRoleKB, 1);
             set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
-            g.bucket = (int)b;
-            g.out_hi = p->phi + bk.gplane_off;
-            g.out_lo = p->plo + bk.gplane_off;
-            g.st_hi = m + st_map(3, 0);
-            g.st_lo = m + st_map(3, 1);
-            g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
-            g.ld_bf = bk.ld_n;
-            g.g_hi = p->ghi + bk.gplane_off;
-            g.g_lo = p->glo + bk.gplane_off;
-            set_sym(g, bk.n);
-            set_one_pass(p, g, bk, false);
-            poly.add(g, false, false);
-        }
-        if ((rc = flush_set(p, ISOLOCO_PHASE_POLY, poly, st))) return rc;
-        // ---- X_{t+1} = xscale * X_t P (tall) or P X_t (wide), one launch
-        // X_{t+1} is always written as fp16 planes; X is the split operand (A when tall,
-        // B when wide), P the single one except in the polish step (3 passes) and in
-        // iteration 0 and the full-precision paths (both split)
-        LaunchSet upd;
-        init_set(upd, kEpiXSplit, kGateStep, p,
-                 first ? Precision{0, 1, 0, 0, 0} : (full ? Precision{1, 1, 0, 0, 0} : Precision{1, 1, 0, 0, 1}));
-        const bool p_split = first || full;
-        for (size_t b = 0; b < p->buckets.size(); ++b) {
-            const Bucket& bk = p->buckets[b];
-            const CUtensorMap* m = maps + b * kMapsPerBucket;
-            GemmGroup g{};
-            if (gs_on && bk.gs) {
-                if (first) continue;  // Z_1 = P_0: k_gs_init below
-                // Z_{t+1} = Z_t P_t in the first n rows of the other buffer
-                g.a_hi = m + z_map(t & 1, 0, 0);
-                g.a_lo = m + z_map(t & 1, 0, 1);
-                g.b_hi = m + p_map(kRoleKB, 0);
-                g.b_lo = m + p_map(kRoleKB, 1);
-                set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
-                g.bucket = (int)b;
-                g.out_hi = p->xhi[dst] + bk.plane_off;
-                g.out_lo = p->xlo[dst] + bk.plane_off;
-                g.st_hi = m + z_map(dst, 2, 0);
-                g.st_lo = m + z_map(dst, 2, 1);
-                g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
-                g.ld_bf = bk.ld;
-                upd.add(g, false, false, true, p_split);
-                continue;
-            }
-            if (bk.tall) {
-                g.a_hi = m + src_map(src, kRoleKA, 0);
-                g.a_lo = m + src_map(src, kRoleKA, 1);
-                g.b_hi = m + p_map(kRoleKB, 0);
-                g.b_lo = m + p_map(kRoleKB, 1);
-            } else {
-                g.a_hi = m + p_map(kRoleKA, 0);
-                g.a_lo = m + p_map(kRoleKA, 1);
-                g.b_hi = m + src_map(src, kRoleMN, 0);
-                g.b_lo = m + src_map(src, kRoleMN, 1);
-            }
-            set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
             g.out_hi = p->xhi[dst] + bk.plane_off;
             g.out_lo = p->xlo[dst] + bk.plane_off;
-            g.st_hi = m + st_map(dst, 0);
-            g.st_lo = m + st_map(dst, 1);
+            g.st_hi = m + z_map(dst, 2, 0);
+            g.st_lo = m + z_map(dst, 2, 1);
             g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
             g.ld_bf = bk.ld;
-            set_one_pass(p, g, bk, true);
-            // the polish writes the final Q: its epilogue also sums tr(Q^T Delta)
-            g.d_hi = p->dhi + bk.plane_off;
-            g.d_lo = p->dlo + bk.plane_off;
-            g.tf_part = p->tfpart + bk.tf_base;
-            if (bk.tall)
-                upd.add(g, false, false, true, p_split);
-            else
-                upd.add(g, false, true, p_split, true);
+            upd.add(g, false, false, true, p_split);
+            continue;
         }
-        if ((rc = flush_set(p, ISOLOCO_PHASE_UPDATE, upd, st)))
-            return rc;
-        if (gs_on && first) {
-            // Gram-side: A = Delta^T Delta / s^2 from the fp32 partials, Z_1 = P_0
-            PhaseTimer tm(p, ISOLOCO_PHASE_UPDATE, st);
-            k_gs_init<<<dim3(p->gs_blocks, p->n_gs), 256, 0, st>>>(p->mats_d, p->state, p->gs_list, p->gpart, p->gpart_off_d,
-                                                         p->gpart_sstride_d, p->nsplit_d, p->anhi, p->anlo,
-                                                         p->xhi[1], p->xlo[1], p->phi, p->plo);
-            CUDA_TRY(cudaGetLastError());
+        if (bk.tall) {
+            g.a_hi = m + src_map(src, kRoleKA, 0);
+            g.a_lo = m + src_map(src, kRoleKA, 1);
+            g.b_hi = m + p_map(kRoleKB, 0);
+            g.b_lo = m + p_map(kRoleKB, 1);
+        } else {
+            g.a_hi = m + p_map(kRoleKA, 0);
+            g.a_lo = m + p_map(kRoleKA, 1);
+            g.b_hi = m + src_map(src, kRoleMN, 0);
+            g.b_lo = m + src_map(src, kRoleMN, 1);
         }
+        set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
+        g.bucket = (int)b;
+        g.out_hi = p->xhi[dst] + bk.plane_off;
+        g.out_lo = p->xlo[dst] + bk.plane_off;
+        g.st_hi = m + st_map(dst, 0);
+        g.st_lo = m + st_map(dst, 1);
+        g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
+        g.ld_bf = bk.ld;
+        set_one_pass(p, g, bk, true);
+        // the polish writes the final Q: its epilogue also sums tr(Q^T Delta)
+        g.d_hi = p->dhi + bk.plane_off;
+        g.d_lo = p->dlo + bk.plane_off;
+        g.tf_part = p->tfpart + bk.tf_base;
+        if (bk.tall)
+            upd.add(g, false, false, true, p_split);
+        else
+            upd.add(g, false, true, p_split, true);
+    }
+}
+
+// Iteration t of the polar loop for every matrix still active: Gram, convergence test
+// and choice of the step (k_control), polynomial, update.  With set_cond, k_control also
+// sets the graph condition `cond` (graph body only).
+static int polar_iteration(isoloco_plan* p, int t, int max_iter, float tol, cudaStream_t st,
+                           cudaGraphConditionalHandle cond, int set_cond) {
+    IterSets s;
+    build_iteration(p, t, s);
+    const bool first = (t == 0);
+    const bool full = p->fast_steps > 0 || p->full_prec;
+    const bool gs_on = gram_side_on(p);
+    int rc;
+    if ((rc = flush_set(p, ISOLOCO_PHASE_GRAM, s.w, st)) || (rc = flush_set(p, ISOLOCO_PHASE_GRAM, s.gram_gs, st)) ||
+        (rc = flush_set(p, ISOLOCO_PHASE_GRAM, s.gram, st)))
+        return rc;
+    // after iteration 0 the Gram-side matrices need no finalize: skip an empty launch
+    if (p->nftiles && (first || !gs_on || p->nftiles_reg > 0)) {
+        PhaseTimer tm(p, ISOLOCO_PHASE_FINALIZE, st);
+        k_gram_finalize<<<p->nftiles, 256, 0, st>>>(p->mats_d, p->ftiles, p->state, p->gpart, p->gpart_off_d,
+                                                    p->gpart_sstride_d, p->nsplit_d, p->ghi, p->glo,
+                                                    p->fin_part, first ? 0 : 1, (first || full) ? nullptr : p->ypl,
+                                                    (!first && gs_on) ? 1 : 0);
+        CUDA_TRY(cudaGetLastError());
+    }
+    { PhaseTimer tm(p, ISOLOCO_PHASE_CONTROL, st);
+    k_control<<<(p->nmat + kControlThreads / 32 - 1) / (kControlThreads / 32), kControlThreads, 0, st>>>(p->mats_d, p->nmat, p->state, p->fin_part, t, max_iter, tol, p->err_d,
+                                  p->bucket_first_d, p->bucket_count_d, (int)p->buckets.size(), p->list_gram,
+                                  p->cnt_gram, p->list_step, p->cnt_step, cond, set_cond, p->loopc,
+                                  p->fast_steps, p->ticket,
+                                  make_int4(gp_one(p, 0, 0), gp_one(p, 0, 1), gp_one(p, 1, 0), gp_one(p, 1, 1)),
+                                  make_int4(up_one(p, 0, 0), up_one(p, 0, 1), up_one(p, 1, 0), up_one(p, 1, 1)), gs_on ? 1 : 0, p->ctl); }
+    CUDA_TRY(cudaGetLastError());
+    if ((rc = flush_set(p, ISOLOCO_PHASE_POLY, s.poly, st))) return rc;
+    if ((rc = flush_set(p, ISOLOCO_PHASE_UPDATE, s.update, st))) return rc;
+    if (gs_on && first) {
+        // Gram-side: A = Delta^T Delta / s^2 from the fp32 partials, Z_1 = P_0
+        PhaseTimer tm(p, ISOLOCO_PHASE_UPDATE, st);
+        k_gs_init<<<dim3(p->gs_blocks, p->n_gs), 256, 0, st>>>(p->mats_d, p->state, p->gs_list, p->gpart, p->gpart_off_d,
+                                                     p->gpart_sstride_d, p->nsplit_d, p->anhi, p->anlo,
+                                                     p->xhi[1], p->xlo[1], p->phi, p->plo);
+        CUDA_TRY(cudaGetLastError());
     }
     return ISOLOCO_OK;
+}
+
+// Builds the polar loop's tables for this call's precision (iterations 1 and 2: every later odd
+// / even pair uses the same buffers).
+static void build_loop(isoloco_plan* p) {
+    const long long key[3] = {p->fast_steps > 0 ? 1 : 0, p->full_prec ? 1 : 0, p->prec_code};
+    if (!memcmp(key, p->loop_key, sizeof(key))) return;
+    p->loop_groups.clear();
+    int most = 1;  // tiles of the largest phase
+    for (int it = 0; it < 2; ++it) {
+        IterSets s;
+        build_iteration(p, it + 1, s);
+        LaunchSet* sets[kLoopPhases] = {&s.w, &s.gram, &s.gram_gs, &s.poly, &s.update};
+        std::vector<int> tiles[kLoopPhases];  // per matrix
+        for (int ph = 0; ph < kLoopPhases; ++ph) {
+            tiles[ph].assign(p->nmat, 0);
+            for (const GemmGroup& g : sets[ph]->groups)
+                for (int b = 0; b < g.batch; ++b) tiles[ph][g.mat_base + b] = group_tiles(g);
+        }
+        for (int ph = 0; ph < kLoopPhases; ++ph) {
+            LaunchSet& ls = *sets[ph];
+            std::stable_sort(ls.groups.begin(), ls.groups.end(), [](const GemmGroup& x, const GemmGroup& y) {
+                return x.kblocks_per_split > y.kblocks_per_split;  // longest tiles first
+            });
+            LoopPhase& L = p->loop_phases[it * kLoopPhases + ph];
+            L = LoopPhase{};
+            L.kind = ph;
+            L.first = (int)p->loop_groups.size();
+            L.ngroups = (int)ls.groups.size();
+            if (L.ngroups)
+                L.f = {ls.p.gate, ls.p.in_f16, ls.p.out_f16, ls.p.split_on_polish, ls.p.gram_y, ls.p.poly_horner,
+                       ls.p.unit_scale};
+            const int dep = ph == kLoopUpdate ? kLoopPoly : ph == kLoopGramGs ? kLoopW : kLoopUpdate;
+            int total = 0;
+            for (const GemmGroup& g : ls.groups) {
+                const MatDesc& md = p->mats_h[g.mat_base];
+                LoopGroup lg{};
+                lg.g = g;
+                lg.cm = {md.n, md.n_gtiles, md.gpart_slot, md.deep, md.gs};
+                lg.tiles = tiles[ph][g.mat_base];
+                lg.dep_tiles = tiles[dep][g.mat_base];
+                p->loop_groups.push_back(lg);
+                L.count += g.batch;
+                total += g.batch * lg.tiles;
+            }
+            most = std::max(most, total);
+        }
+    }
+    p->loop_clusters = std::min(most, p->num_sms / 2);
+    memcpy(p->loop_key, key, sizeof(key));
+}
+
+template <int NG>
+static cudaError_t run_loop_n(isoloco_plan* p, int max_iter, float tol, cudaStream_t st) {
+    LoopParams<NG> lp;
+    memcpy(lp.groups, p->loop_groups.data(), sizeof(LoopGroup) * p->loop_groups.size());
+    memcpy(lp.phases, p->loop_phases, sizeof(lp.phases));
+    lp.state = p->state;
+    lp.fin_part = p->fin_part;
+    lp.ctl = p->ctl;
+    lp.arr = p->arr;
+    lp.prof = p->prof ? p->loop_prof : nullptr;
+    lp.err = p->err_d;
+    lp.max_t = max_iter + 1;
+    lp.max_iter = max_iter;
+    lp.tol = tol;
+    lp.fast_steps = p->fast_steps;
+    lp.gram_one = make_int4(gp_one(p, 0, 0), gp_one(p, 0, 1), gp_one(p, 1, 0), gp_one(p, 1, 1));
+    lp.upd_one = make_int4(up_one(p, 0, 0), up_one(p, 0, 1), up_one(p, 1, 0), up_one(p, 1, 1));
+    lp.gs_on = gram_side_on(p) ? 1 : 0;
+    return launch_polar_loop<NG>(lp, p->loop_clusters, st);
+}
+
+// Iterations 1, 2, ... as one launch of the polar loop (polar_loop.cu).  Not taken (false) by
+// plans with more groups than its parameters hold, or with a bucket that is not Gram-side and
+// splits its Gram over K: split partials need the finalize pass between the Gram and the
+// control step, and an unsplit Gram of that length would leave most of the GPU waiting for a
+// few tiles.  Those keep the graph of launches.
+static bool run_loop(isoloco_plan* p, int max_iter, float tol, cudaStream_t st, cudaError_t* e) {
+    if (gram_side_on(p) ? p->nftiles_reg > 0 : p->nftiles > 0) return false;
+    build_loop(p);
+    const int n = (int)p->loop_groups.size();
+    if (n > kLoopGroups) return false;
+    // one launch; under phase profiling its phases are timed inside (isoloco_profile_read)
+    p->launches += 1;
+    p->prof_n[ISOLOCO_PHASE_GRAM] += 1;
+    *e = n <= kLoopGroupsSmall ? run_loop_n<kLoopGroupsSmall>(p, max_iter, tol, st)
+                               : run_loop_n<kLoopGroups>(p, max_iter, tol, st);
+    return true;
 }
 
 // Captures iterations 1 and 2 (the buffer parity of every later odd / even pair) as the
@@ -1123,11 +1240,6 @@ static int build_polar_graph(isoloco_plan* p, int max_iter, float tol) {
     return ISOLOCO_OK;
 }
 
-// The polar iteration for every matrix, from Delta (planes dhi/dlo) to Q and sigma_bar.
-// Iteration 0 is launched directly; the rest run as one graph launch that stops as soon
-// as every matrix is done.  With phase profiling on (events cannot sit inside the graph
-// body), or when `st` is itself being captured, iterations 1 .. max_iter are launched one
-// by one instead (empty launches once every matrix is done).
 // Gram-side matrices after the loop: Q = Delta (Z_T / s) into the ping-pong buffer that
 // does not hold Z_T (bf16 operands, three passes), and final_buf pointed at it.
 static int gs_final(isoloco_plan* p, cudaStream_t st) {
@@ -1173,6 +1285,11 @@ static int gs_final(isoloco_plan* p, cudaStream_t st) {
     return ISOLOCO_OK;
 }
 
+// The polar iteration for every matrix, from Delta (planes dhi/dlo) to Q and sigma_bar.
+// Iteration 0 is launched directly; the rest run as one persistent kernel (run_loop) or, where
+// that does not apply, as one graph launch that stops as soon as every matrix is done.  When
+// `st` is being captured (and with phase profiling, without the kernel), iterations 1 ..
+// max_iter are launched one by one instead (empty launches once every matrix is done).
 static int run_polar(isoloco_plan* p, int max_iter, float tol, cudaStream_t st) {
     if (p->nmat == 0) return ISOLOCO_OK;
     // the Gram partial slots of Gram-side matrices: iteration 0's finalize fills fewer of them
@@ -1184,8 +1301,12 @@ static int run_polar(isoloco_plan* p, int max_iter, float tol, cudaStream_t st) 
     if (rc) return rc;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CUDA_TRY(cudaStreamIsCapturing(st, &cs));
-    const bool use_graph = !p->prof && !p->per_launch && cs == cudaStreamCaptureStatusNone;
-    if (use_graph) {
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
+    const bool use_graph = !p->prof && !p->per_launch && !capturing;
+    cudaError_t le = cudaSuccess;
+    if (!capturing && run_loop(p, max_iter, tol, st, &le)) {
+        CUDA_TRY(le);
+    } else if (use_graph) {
         if (!p->gexec || p->g_max_iter != max_iter || p->g_tol != tol || p->g_fast != p->fast_steps ||
             p->g_full != (p->full_prec ? 1 : 0) || p->g_prec != p->prec_code)
             if ((rc = build_polar_graph(p, max_iter, tol))) return rc;
@@ -1418,7 +1539,7 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
     { PhaseTimer tm(p, ISOLOCO_PHASE_CLIP, st, 0);
     k_reset_state<<<(std::max(1, a->nmat) + 255) / 256, 256, 0, st>>>(
         a->state, a->nmat, a->err_d, a->mats_d, a->bucket_first_d, a->bucket_count_d, (int)a->buckets.size(),
-        a->list_gram, a->cnt_gram, a->ticket);
+        a->list_gram, a->cnt_gram, a->ticket, a->arr);
     a->launches += 1;
     CUDA_TRY(cudaGetLastError());
     k_clip_form_a<<<grid, 256, 0, st>>>(p->mats_d, p->state, p->hbuf, p->hoff_d, p->hss_d, p->nsplit_d, a->mats_d,
@@ -1589,7 +1710,7 @@ static int run_isoc_step(isoloco_plan* p, int merge, float* theta, float* mom, c
     { PhaseTimer tm(p, ISOLOCO_PHASE_OTHER, st);
     k_reset_state<<<(std::max(1, p->nmat) + 255) / 256, 256, 0, st>>>(
         p->state, p->nmat, p->err_d, p->mats_d, p->bucket_first_d, p->bucket_count_d, (int)p->buckets.size(),
-        p->list_gram, p->cnt_gram, p->ticket); }
+        p->list_gram, p->cnt_gram, p->ticket, p->arr); }
     CUDA_TRY(cudaGetLastError());
     if (p->nchunks) {
         PhaseTimer tm(p, ISOLOCO_PHASE_REDUCE, st);
@@ -1913,6 +2034,7 @@ int isoloco_profile_enable(isoloco_plan_t p, int enable) {
         p->prof_ms[ph] = 0.0;
         p->prof_n[ph] = 0;
     }
+    CUDA_TRY(cudaMemset(p->loop_prof, 0, sizeof(unsigned long long) * kLoopPhases));
     p->prof = enable != 0;
     return ISOLOCO_OK;
 }
@@ -1930,8 +2052,15 @@ int isoloco_profile_read(isoloco_plan_t p, void* stream, double* ms, int64_t* la
         }
         p->pend[ph].clear();
     }
+    // the polar loop's phases, timed on the device (added to what the events gave)
+    unsigned long long ns[kLoopPhases] = {0};
+    double loop_ms[ISOLOCO_NUM_PHASES] = {0};
+    CUDA_TRY(cudaMemcpy(ns, p->loop_prof, sizeof(ns), cudaMemcpyDeviceToHost));
+    loop_ms[ISOLOCO_PHASE_GRAM] = 1e-6 * (double)(ns[kLoopW] + ns[kLoopGram] + ns[kLoopGramGs]);
+    loop_ms[ISOLOCO_PHASE_POLY] = 1e-6 * (double)ns[kLoopPoly];
+    loop_ms[ISOLOCO_PHASE_UPDATE] = 1e-6 * (double)ns[kLoopUpdate];
     for (int ph = 0; ph < nphases && ph < ISOLOCO_NUM_PHASES; ++ph) {
-        if (ms) ms[ph] = p->prof_ms[ph];
+        if (ms) ms[ph] = p->prof_ms[ph] + loop_ms[ph];
         if (launches) launches[ph] = p->prof_n[ph];
     }
     return ISOLOCO_OK;

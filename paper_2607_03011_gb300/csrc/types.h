@@ -45,17 +45,15 @@ constexpr int kGramSideRatio = 8;
 // residual ||X^T X - I||_F / sqrt(n) is at least this: one quintic step cannot bring such a
 // residual below the convergence tolerance, so the Gram cannot be the one the polish uses.
 constexpr float kOnePassGramResid = 0.5f;
-// Epilogue staging: per epilogue warp kStageBlocks blocks of 32 x 32 16-bit values (2 KB,
-// 64-byte swizzled rows), written to global memory by TMA stores.  With four, a symmetric
-// output uses them as two (direct, transposed) pairs and anything else as four single
-// blocks, so that a warp fills one while the TMA stores of the others still read shared
-// memory; with two (the setting: the epilogue keeps up with the main loop, and the ring
-// gets the 32 KB), one pair, or two alternating single blocks.
+// Epilogue staging: per epilogue warp two blocks of 32 x 32 16-bit values (2 KB, 64-byte
+// swizzled rows), written to global memory by TMA stores: a symmetric output's block and its
+// transpose, or alternately single blocks.
 constexpr int kStageBlockBytes = 32 * 32 * 2;
 constexpr int kStageBlocks = 2;
 constexpr int kEpiStagingBytes = kEpiWarps * kStageBlocks * kStageBlockBytes;
 constexpr int kTileQueue = 8;  // tiles handed from the producer warp to the MMA and epilogue warps
-constexpr int kGemmSmemBytes = kRingBytes + kEpiStagingBytes + 1024 /*align*/ + 512 /*barriers, queues*/;
+constexpr int kGemmTailBytes = 1280;  // barriers, tile queue
+constexpr int kGemmSmemBytes = kRingBytes + kEpiStagingBytes + 1024 /*align*/ + kGemmTailBytes;
 
 // Epilogue of the split-precision GEMM.
 enum EpiMode : int {
@@ -71,8 +69,6 @@ enum GateMode : int {
     kGateNone = 0,    // all (debug GEMM)
     kGateActive = 1,  // matrices not yet done (Gram)
     kGateStep = 2,    // matrices whose mode this iteration is quintic or polish
-    kGateQuintic = 3, // matrices taking a quintic step
-    kGatePolish = 4,  // matrices taking the final polish step
 };
 
 // First tile column of tile row tm that touches the upper triangle of a square output.
@@ -151,6 +147,11 @@ struct MatState {
     int trace_fused;  // 1: the GEMM that wrote Q also summed tr(Q^T Delta) (its tf_part slots)
 };
 
+// What a launch (or a phase of the polar loop) says about all of its tiles (GemmParams).
+struct TileFlags {
+    int gate, in_f16, out_f16, split_on_polish, gram_y, poly_horner, unit_scale;
+};
+
 struct GemmParams {
     GemmGroup g[kMaxGroups];
     int num_groups;
@@ -171,6 +172,13 @@ struct GemmParams {
                           // iteration's control step has reset xscale to 1)
     MatState* state;
     uint32_t* err;
+};
+
+// What the control step needs to know about a matrix besides its state.
+struct ControlMat {
+    int n, n_gtiles;     // size of the Gram; groups of kPartSlots partial sums
+    int64_t gpart_slot;  // first of them
+    int deep, gs;
 };
 
 // Description of one 2-D tensor in the workspace (device array, one per matrix).
