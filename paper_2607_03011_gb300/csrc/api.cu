@@ -75,22 +75,22 @@ __global__ void k_svd_tridiag(const MatDesc*, const MatState*, float*, const int
 __global__ void k_svd_bisect(const MatDesc*, const float*, const int64_t*, float*, const int64_t*);
 __global__ void k_svd_sigma_bar(const MatDesc*, int, MatState*, const float*, const int64_t*);
 __global__ void k_diloco(ReplicaPtrs, int, int, float*, float*, int64_t, float, float, float, uint32_t*);
-__global__ void k_dare(ReplicaPtrs, int, int, float*, float*, int64_t, float, uint32_t, float, unsigned int,
-                       uint64_t, float, float, uint32_t*);
+cudaError_t launch_dare(const ReplicaPtrs&, int, bool, float*, float*, int64_t, float, uint32_t, float, unsigned int,
+                        uint64_t, float, float, uint32_t*, int, cudaStream_t);
+cudaError_t launch_ties_bracket(const ReplicaPtrs&, int, int, const float*, int64_t, const uint64_t*, uint32_t*,
+                                uint32_t*, int64_t, unsigned long long*, int, cudaStream_t);
 __global__ void k_ties_init(int, uint64_t, uint64_t, uint64_t, unsigned long long*, uint64_t*, uint64_t*, uint64_t*,
                             uint64_t*, uint64_t*, uint64_t*, unsigned long long*, int*);
 __global__ void k_ties_sample(ReplicaPtrs, int, int, const float*, int64_t, int64_t, uint32_t*);
 __global__ void k_ties_hist_buf(const uint32_t*, const uint32_t*, int, int64_t, int, int, int, const uint64_t*,
                                 unsigned long long*);
-__global__ void k_ties_bracket(ReplicaPtrs, int, int, const float*, int64_t, const uint64_t*, uint32_t*, uint32_t*,
-                               int64_t, unsigned long long*);
 __global__ void k_ties_check(int, int, int64_t, uint64_t, const unsigned long long*, const uint32_t*, uint64_t*,
                              int*);
 __global__ void k_ties_hist(ReplicaPtrs, int, int, const float*, int64_t, int, const uint64_t*, unsigned long long*,
                             const int*);
-__global__ void k_ties_select(int, int, unsigned long long*, uint64_t*, uint64_t*, const int*);
-__global__ void k_ties_merge(ReplicaPtrs, int, int, float*, float*, int64_t, const uint64_t*, const uint64_t*,
-                             const int*, float, float, uint32_t*);
+__global__ void k_ties_select(int, int, unsigned long long*, uint64_t*, uint64_t*, const int*, int);
+cudaError_t launch_ties_merge(const ReplicaPtrs&, int, int, float*, float*, int64_t, const uint64_t*, const uint64_t*,
+                              const int*, float, float, uint32_t*, int, cudaStream_t);
 __global__ void k_split_planes(const float*, int64_t, int, int, int, __nv_bfloat16*, __nv_bfloat16*, int);
 __global__ void k_debug_wait(uint32_t*, uint64_t, unsigned long long*);
 
@@ -614,8 +614,6 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
     CUDA_TRY(cudaEventCreateWithFlags(&p->done_ev, cudaEventDisableTiming));
     if (p->K * 256 * 4 > 48 * 1024)  // TIES histograms: K (replica passes) or 2K x 256 shared counters
         CUDA_TRY(cudaFuncSetAttribute(k_ties_hist, cudaFuncAttributeMaxDynamicSharedMemorySize, p->K * 256 * 4));
-    if (p->K * 256 * 4 > 48 * 1024)  // per-thread counters of the TIES bracket pass
-        CUDA_TRY(cudaFuncSetAttribute(k_ties_bracket, cudaFuncAttributeMaxDynamicSharedMemorySize, p->K * 256 * 4));
     if (2 * p->K * 256 * 4 > 48 * 1024)
         CUDA_TRY(cudaFuncSetAttribute(k_ties_hist_buf, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       2 * p->K * 256 * 4));
@@ -1888,8 +1886,8 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
         // keep when top24 >= ceil(p * 2^24) (exact in double); draw numbers step by N * GAMMA
         const uint32_t pthr = (uint32_t)std::ceil((double)o.sparsity * 16777216.0);
         const uint64_t ng = (uint64_t)p->N * 0x9E3779B97F4A7C15ull;
-        k_dare<<<grid, 256, 0, st>>>(rp, p->K, p->dtype, theta, momentum, p->N, scale, pthr,
-                                     1.f / (1.f - o.sparsity), o.seed, ng, o.outer_lr, o.momentum, p->err_d);
+        CUDA_TRY(launch_dare(rp, p->K, p->dtype != ISOLOCO_F32, theta, momentum, p->N, scale, pthr,
+                             1.f / (1.f - o.sparsity), o.seed, ng, o.outer_lr, o.momentum, p->err_d, grid, st));
     } else {
         // keep the n_keep largest |Delta_k| of each worker; n_keep = N keeps all (threshold 0)
         const uint64_t n_keep = (uint64_t)(p->N - (int64_t)std::floor((double)o.sparsity * (double)p->N));
@@ -1903,21 +1901,21 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
         const uint64_t r_hi = (uint64_t)std::max(1.0, std::floor(r_mid - m));
         const uint64_t r_lo = (uint64_t)std::min(S, std::ceil(r_mid + m));
         {
-            PhaseTimer tm(p, ISOLOCO_PHASE_TRIM, st, select ? 29 : 1);
+            PhaseTimer tm(p, ISOLOCO_PHASE_TRIM, st, select ? 25 : 1);
             k_ties_init<<<1, 256, 0, st>>>(K, n_keep, r_hi, r_lo, p->ties_hist, p->ties_rank_s, p->ties_prefix_s,
                                            p->ties_rank_c, p->ties_prefix_c, p->ties_rank_f, p->ties_prefix_f,
                                            p->ties_above, p->ties_fail);
             if (select) {
                 k_ties_sample<<<(unsigned)((p->ties_S + 255) / 256), 256, 0, st>>>(rp, K, p->dtype, theta, p->N,
                                                                                  p->ties_S, p->ties_samp);
-                for (int pass = 0; pass < 4; ++pass) {
+                for (int pass = 0; pass < 2; ++pass) {
                     k_ties_hist_buf<<<dim3(1, 256), 256, 2 * K * 256 * 4, st>>>(
                         p->ties_samp, nullptr, 1, p->ties_S, 2 * K, 2, pass, p->ties_prefix_s, p->ties_hist);
                     k_ties_select<<<(2 * K * 32 + 255) / 256, 256, 0, st>>>(2 * K, pass, p->ties_hist, p->ties_rank_s, p->ties_prefix_s,
-                                                     nullptr);
+                                                     nullptr, pass == 1);
                 }
-                k_ties_bracket<<<p->ties_nseg, 256, K * 256 * 4, st>>>(rp, K, p->dtype, theta, p->N, p->ties_prefix_s,
-                                                            p->ties_cand, p->ties_cnt, p->ties_segcap, p->ties_above);
+                CUDA_TRY(launch_ties_bracket(rp, K, p->dtype, theta, p->N, p->ties_prefix_s, p->ties_cand, p->ties_cnt,
+                                             p->ties_segcap, p->ties_above, p->ties_nseg, st));
                 k_ties_check<<<K, 256, 0, st>>>(K, p->ties_nseg, p->ties_segcap, n_keep, p->ties_above, p->ties_cnt,
                                                p->ties_rank_c, p->ties_fail);
                 for (int pass = 0; pass < 4; ++pass) {
@@ -1925,7 +1923,7 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
                         p->ties_cand, p->ties_cnt, p->ties_nseg, p->ties_segcap, K, 1, pass, p->ties_prefix_c,
                         p->ties_hist);
                     k_ties_select<<<(K * 32 + 255) / 256, 256, 0, st>>>(K, pass, p->ties_hist, p->ties_rank_c, p->ties_prefix_c,
-                                                    nullptr);
+                                                    nullptr, 0);
                 }
                 // fallback, only when some bracket missed: the four passes over the replicas
                 const int smem = K * 256 * 4;
@@ -1933,13 +1931,13 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
                     k_ties_hist<<<grid, 256, smem, st>>>(rp, K, p->dtype, theta, p->N, pass, p->ties_prefix_f,
                                                          p->ties_hist, p->ties_fail);
                     k_ties_select<<<(K * 32 + 255) / 256, 256, 0, st>>>(K, pass, p->ties_hist, p->ties_rank_f, p->ties_prefix_f,
-                                                    p->ties_fail);
+                                                    p->ties_fail, 0);
                 }
             }
         }
         PhaseTimer tm(p, ISOLOCO_PHASE_DILOCO, st);
-        k_ties_merge<<<grid, 256, 0, st>>>(rp, p->K, p->dtype, theta, momentum, p->N, p->ties_prefix_c,
-                                           p->ties_prefix_f, p->ties_fail, o.outer_lr, o.momentum, p->err_d);
+        CUDA_TRY(launch_ties_merge(rp, p->K, p->dtype, theta, momentum, p->N, p->ties_prefix_c, p->ties_prefix_f,
+                                   p->ties_fail, o.outer_lr, o.momentum, p->err_d, grid, st));
     }
     CUDA_TRY(cudaGetLastError());
     return finish_call(p, st, o.sync);

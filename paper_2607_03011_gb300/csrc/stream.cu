@@ -371,14 +371,20 @@ __global__ void __launch_bounds__(kStreamThreads) k_diloco(ReplicaPtrs reps, int
 // mix(s + n * GAMMA), mix = xor-shift 30, * M1, xor-shift 27, * M2, xor-shift 31.  DARE uses
 // only the top 24 bits of an output: the last xor-shift leaves bits 63..33 as they are, and
 // the top half of the last product is umulhi(lo, M2lo) + lo * M2hi + hi * M2lo (mod 2^32).
+// The draws bound k_dare, so the 64-bit steps are spelled out on 32-bit halves.
 constexpr uint64_t kSmGamma = 0x9E3779B97F4A7C15ull;
-__device__ __forceinline__ uint32_t splitmix64_top24(uint64_t z /* s + n * GAMMA */) {
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z ^= z >> 27;
-    const uint32_t lo = static_cast<uint32_t>(z), hi = static_cast<uint32_t>(z >> 32);
-    const uint32_t m_lo = 0x133111EBu, m_hi = 0x94D049BBu;
-    return (__umulhi(lo, m_lo) + lo * m_hi + hi * m_lo) >> 8;
+__device__ __forceinline__ uint32_t splitmix64_top32(uint64_t z /* s + n * GAMMA */) {
+    uint32_t lo = static_cast<uint32_t>(z), hi = static_cast<uint32_t>(z >> 32);
+    lo ^= __funnelshift_r(lo, hi, 30);
+    hi ^= hi >> 30;
+    const uint64_t w = static_cast<uint64_t>(lo) * 0x1CE4E5B9u;  // * 0xBF58476D1CE4E5B9
+    hi = static_cast<uint32_t>(w >> 32) + lo * 0xBF58476Du + hi * 0x1CE4E5B9u;
+    lo = static_cast<uint32_t>(w);
+    lo ^= __funnelshift_r(lo, hi, 27);
+    hi ^= hi >> 27;
+    return __umulhi(lo, 0x133111EBu) + lo * 0x94D049BBu + hi * 0x133111EBu;  // * 0x94D049BB133111EB
 }
+__device__ __forceinline__ uint32_t splitmix64_top24(uint64_t z) { return splitmix64_top32(z) >> 8; }
 
 __device__ __forceinline__ void nesterov1(float& th, float& b, float u, float eta, float mu) {
     const float nb = fmaf(mu, b, u);
@@ -386,52 +392,91 @@ __device__ __forceinline__ void nesterov1(float& th, float& b, float u, float et
     b = nb;
 }
 
+// Consecutive entries of a replica, one 16-byte load of 4 fp32 or 8 bf16 values.
+template <bool BF16>
+__device__ __forceinline__ uint4 ld_rep_raw(const void* base, int64_t i) {
+    return BF16 ? __ldg(reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(base) + i))
+                : __ldg(reinterpret_cast<const uint4*>(static_cast<const float*>(base) + i));
+}
+template <bool BF16>
+__device__ __forceinline__ float rep_value(const uint4& u, int j) {
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+    if (!BF16) return __uint_as_float(w[j]);
+    return __uint_as_float((j & 1) ? (w[j >> 1] & 0xFFFF0000u) : (w[j >> 1] << 16));
+}
+
 // DARE: U = scale * sum_k keep_scale * m_k * Delta_k, keep_scale = 1 / (1 - p), scale =
 // 1 / K (mean) or 1.  Entry i of worker k is kept when the top 24 bits of SplitMix64 output
 // k * N + i + 1 (state seed) are >= pthr = ceil(p * 2^24), i.e. when that value times 2^-24
-// is >= p.  ng = N * GAMMA (mod 2^64) steps the draw number from one worker to the next.
-// Grid-stride over float4 vectors of all N entries, scalar tail in CTA 0.
-__global__ void __launch_bounds__(kStreamThreads) k_dare(ReplicaPtrs reps, int K, int dtype,
-                                                         float* __restrict__ theta, float* __restrict__ mom,
-                                                         int64_t N, float scale, uint32_t pthr, float keep_scale,
-                                                         unsigned int seed, uint64_t ng, float eta, float mu,
+// is >= p (pthr < 2^24, so the comparison is made on the top 32 bits).  ng = N * GAMMA (mod
+// 2^64) steps the draw number from one worker to the next.  Grid-stride over 16-byte vectors of
+// the replicas, four workers' loads issued before their draws; scalar tail in CTA 0.  Bound by
+// the draws' integer instructions (about 12 of a draw's 21 share the half-rate pipe): 220M
+// parameters, 16 bf16 workers 4.09 -> 2.92 ms, 8 fp32 workers 2.27 -> 1.86 ms, against 64-bit
+// steps, one load at a time and the type tested at each.
+template <bool BF16>
+__global__ void __launch_bounds__(kStreamThreads) k_dare(ReplicaPtrs reps, int K, float* __restrict__ theta,
+                                                         float* __restrict__ mom, int64_t N, float scale,
+                                                         uint32_t pthr, float keep_scale, unsigned int seed,
+                                                         uint64_t ng, float eta, float mu,
                                                          uint32_t* __restrict__ err) {
+    constexpr int V = BF16 ? 8 : 4;
+    constexpr int kBatch = 4;
+    const uint32_t thr = pthr << 8;
     bool bad = false;
-    const int64_t nv = N >> 2;
+    const int64_t nv = N / V;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t v = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; v < nv; v += stride) {
-        const int64_t i = 4 * v;
-        float4 th = *reinterpret_cast<const float4*>(theta + i);
-        float4 bb = *reinterpret_cast<const float4*>(mom + i);
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int64_t i = V * v;
+        float th[V], s[V];
+#pragma unroll
+        for (int q = 0; q < V / 4; ++q) {
+            const float4 t = *reinterpret_cast<const float4*>(theta + i + 4 * q);
+            th[4 * q] = t.x; th[4 * q + 1] = t.y; th[4 * q + 2] = t.z; th[4 * q + 3] = t.w;
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j) s[j] = 0.f;
         float chk = 0.f;  // every Delta_k entry, dropped or not, for the non-finite test
         uint64_t z = seed + static_cast<uint64_t>(i + 1) * kSmGamma;  // draw k * N + i + 1, k = 0
-        for (int k = 0; k < K; ++k, z += ng) {
-            const float4 r = ld_rep4(reps.p[k], dtype, i);
-            const float4 d = make_float4(th.x - r.x, th.y - r.y, th.z - r.z, th.w - r.w);
-            chk += (d.x + d.y) + (d.z + d.w);
-            if (splitmix64_top24(z) >= pthr) s.x += d.x * keep_scale;
-            if (splitmix64_top24(z + kSmGamma) >= pthr) s.y += d.y * keep_scale;
-            if (splitmix64_top24(z + 2 * kSmGamma) >= pthr) s.z += d.z * keep_scale;
-            if (splitmix64_top24(z + 3 * kSmGamma) >= pthr) s.w += d.w * keep_scale;
+        for (int k0 = 0; k0 < K; k0 += kBatch) {
+            uint4 r[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u)
+                if (k0 + u < K) r[u] = ld_rep_raw<BF16>(reps.p[k0 + u], i);
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                if (k0 + u >= K) break;
+                uint64_t zj = z;
+#pragma unroll
+                for (int j = 0; j < V; ++j) {
+                    const float d = th[j] - rep_value<BF16>(r[u], j);
+                    chk += d;
+                    if (splitmix64_top32(zj) >= thr) s[j] += d * keep_scale;
+                    zj += kSmGamma;
+                }
+                z += ng;
+            }
         }
-        s.x *= scale; s.y *= scale; s.z *= scale; s.w *= scale;
         bad |= !isfinite(chk);
-        nesterov1(th.x, bb.x, s.x, eta, mu);
-        nesterov1(th.y, bb.y, s.y, eta, mu);
-        nesterov1(th.z, bb.z, s.z, eta, mu);
-        nesterov1(th.w, bb.w, s.w, eta, mu);
-        *reinterpret_cast<float4*>(mom + i) = bb;
-        *reinterpret_cast<float4*>(theta + i) = th;
+#pragma unroll
+        for (int q = 0; q < V / 4; ++q) {
+            const float4 b = *reinterpret_cast<const float4*>(mom + i + 4 * q);
+            float bb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) nesterov1(th[4 * q + j], bb[j], s[4 * q + j] * scale, eta, mu);
+            *reinterpret_cast<float4*>(mom + i + 4 * q) = make_float4(bb[0], bb[1], bb[2], bb[3]);
+            *reinterpret_cast<float4*>(theta + i + 4 * q) =
+                make_float4(th[4 * q], th[4 * q + 1], th[4 * q + 2], th[4 * q + 3]);
+        }
     }
     if (blockIdx.x == 0) {
-        for (int64_t i = 4 * nv + threadIdx.x; i < N; i += blockDim.x) {
+        for (int64_t i = V * nv + threadIdx.x; i < N; i += blockDim.x) {
             float th = theta[i], bb = mom[i], s = 0.f, chk = 0.f;
             uint64_t z = seed + static_cast<uint64_t>(i + 1) * kSmGamma;
             for (int k = 0; k < K; ++k, z += ng) {
-                const float d = th - ld_rep1(reps.p[k], dtype, i);
+                const float d = th - ld_rep1(reps.p[k], BF16 ? 1 : 0, i);
                 chk += d;
-                if (splitmix64_top24(z) >= pthr) s += d * keep_scale;
+                if (splitmix64_top32(z) >= thr) s += d * keep_scale;
             }
             s *= scale;
             bad |= !isfinite(chk);
@@ -443,6 +488,14 @@ __global__ void __launch_bounds__(kStreamThreads) k_dare(ReplicaPtrs reps, int K
     raise_nonfinite(bad, err);
 }
 
+cudaError_t launch_dare(const ReplicaPtrs& reps, int K, bool bf16, float* theta, float* mom, int64_t N, float scale,
+                        uint32_t pthr, float keep_scale, unsigned int seed, uint64_t ng, float eta, float mu,
+                        uint32_t* err, int grid, cudaStream_t st) {
+    (bf16 ? k_dare<true> : k_dare<false>)<<<grid, kStreamThreads, 0, st>>>(reps, K, theta, mom, N, scale, pthr,
+                                                                           keep_scale, seed, ng, eta, mu, err);
+    return cudaGetLastError();
+}
+
 // TIES trim: per worker k, the key (fp32 bits of |Delta_k|, ordered like the magnitudes) of
 // the n_keep-th largest magnitude over all N entries, n_keep = N - floor(sparsity * N).
 // Radix select over the 31 key bits in four digits, [30:23], [22:15], [14:7], [6:0]: a
@@ -451,7 +504,10 @@ __global__ void __launch_bounds__(kStreamThreads) k_dare(ReplicaPtrs reps, int K
 // the replicas, the library brackets the threshold first:
 //   1. k_ties_sample: S keys per worker at jittered strided positions;
 //   2. radix select on the sample for two ranks per worker, the expected rank of the
-//      threshold -/+ 8 standard deviations (and 16): keys hi >= lo;
+//      threshold -/+ 8 standard deviations (and 16), in its first two digits only: the
+//      bracket [lo, hi] is widened to the ends of the 2^15-key bins that hold them (0.4 % of
+//      the magnitude each, against ~1 % between the ranks), which the exact selection below
+//      does not depend on;
 //   3. k_ties_bracket, one pass over the replicas: A = #(key > hi) and the keys in [lo, hi]
 //      collected per CTA (its own segment of the candidate buffer);
 //   4. k_ties_check: if A < n_keep <= A + #candidates and no segment overflowed, the
@@ -462,7 +518,6 @@ __host__ __device__ constexpr int ties_shift(int pass) { return pass == 0 ? 23 :
 __host__ __device__ constexpr int ties_bins(int pass) { return pass == 3 ? 128 : 256; }
 
 __device__ __forceinline__ uint32_t ties_key(float d) { return __float_as_uint(fabsf(d)); }
-constexpr int kLoadBatch = 8;  // replicas whose loads are issued together in the TIES passes
 
 // Counts, per worker, the digit of this pass of every key whose higher digits equal the
 // prefix chosen so far.  Shared histogram [workers][256]; keys sharing a bin within a warp
@@ -595,75 +650,106 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_sample(ReplicaPtrs reps
     for (int k = 0; k < K; ++k) samp[static_cast<int64_t>(k) * S + j] = ties_key(th - ld_rep1(reps.p[k], dtype, i));
 }
 
-// One pass over theta and the replicas: per worker, the keys above the bracket [lo, hi] are
-// counted and those inside it collected into this CTA's segment of cand [K][gridDim.x][segcap];
-// cnt[k][cta] may exceed segcap (overflow: k_ties_check then fails).  Each thread counts in
-// its own shared slots up_s[k][thread] (no atomics, no warp votes in the loop); the rare keys
-// inside a bracket take a shared atomic for their position.  Dynamic shared memory:
-// K x blockDim.x counters.
-__global__ void __launch_bounds__(kStreamThreads) k_ties_bracket(ReplicaPtrs reps, int K, int dtype,
+// One pass over the replicas of up to kTiesWorkers workers: per worker, the keys above the
+// bracket [lo, hi] are counted and those inside it collected into this CTA's segment of cand
+// [K][gridDim.x][segcap]; cnt[k][cta] may exceed segcap (overflow: k_ties_check then fails).
+// Brackets and counts stay in registers, the workers' loads are issued together (pointers at
+// fixed places in the parameters: chosen by an index they cost registers, and so occupancy),
+// and a worker's four keys share the test for the rare push, whose position comes from a
+// shared atomic.  180M x 8: 1.84 -> 1.27 ms fp32 (6.2 TB/s) and 2.5 -> 1.0 ms bf16, against
+// counters per thread in shared memory, four loads in flight and the type tested between them.
+constexpr int kTiesWorkers = 8;
+template <bool BF16>
+__global__ void __launch_bounds__(kStreamThreads) k_ties_bracket(ReplicaPtrs reps, int K,
                                                                  const float* __restrict__ theta, int64_t N,
                                                                  const uint64_t* __restrict__ prefix_s,
                                                                  uint32_t* __restrict__ cand,
                                                                  uint32_t* __restrict__ cnt, int64_t segcap,
                                                                  unsigned long long* __restrict__ above) {
-    extern __shared__ uint32_t up_s[];
-    __shared__ uint32_t hi_s[kMaxK], lo_s[kMaxK], cnt_s[kMaxK];
-    for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        hi_s[k] = static_cast<uint32_t>(prefix_s[2 * k]);
-        lo_s[k] = static_cast<uint32_t>(prefix_s[2 * k + 1]);
-        cnt_s[k] = 0u;
+    constexpr int KB = kTiesWorkers;
+    __shared__ uint32_t cnt_s[KB], up_s[KB];
+    uint32_t hi[KB], lo[KB], up[KB];
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+        hi[k] = k < K ? static_cast<uint32_t>(__ldg(prefix_s + 2 * k)) : 0xFFFFFFFFu;
+        lo[k] = k < K ? static_cast<uint32_t>(__ldg(prefix_s + 2 * k + 1)) : 0xFFFFFFFFu;
+        up[k] = 0u;
     }
-    for (int j = threadIdx.x; j < K * static_cast<int>(blockDim.x); j += blockDim.x) up_s[j] = 0u;
+    if (threadIdx.x < KB) cnt_s[threadIdx.x] = up_s[threadIdx.x] = 0u;
     __syncthreads();
     const int64_t G = gridDim.x;
     const int64_t nv = N >> 2;
     const int64_t stride = G * blockDim.x;
-    uint32_t* mine = up_s + threadIdx.x;
-    auto one = [&](uint32_t key, int k) -> uint32_t {
-        if (key > hi_s[k]) return 1u;
-        if (key >= lo_s[k]) {
-            const uint32_t pos = atomicAdd(&cnt_s[k], 1u);
-            if (pos < segcap) cand[(static_cast<int64_t>(k) * G + blockIdx.x) * segcap + pos] = key;
-        }
-        return 0u;
+    auto push = [&](uint32_t key, int k) {
+        const uint32_t pos = atomicAdd(&cnt_s[k], 1u);
+        if (pos < segcap) cand[(static_cast<int64_t>(k) * G + blockIdx.x) * segcap + pos] = key;
     };
     for (int64_t v = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; v < nv; v += stride) {
         const int64_t i = 4 * v;
         const float4 th = __ldg(reinterpret_cast<const float4*>(theta + i));
-        for (int k0 = 0; k0 < K; k0 += 4) {
-            float4 r[4];
+        float4 r[KB];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (k0 + q < K) r[q] = ld_rep4(reps.p[k0 + q], dtype, i);
+        for (int k = 0; k < KB; ++k)
+            if (k < K) r[k] = ld_rep4(reps.p[k], BF16 ? 1 : 0, i);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = k0 + q;
-                if (k >= K) break;
-                const uint32_t c = one(ties_key(th.x - r[q].x), k) + one(ties_key(th.y - r[q].y), k) +
-                                   one(ties_key(th.z - r[q].z), k) + one(ties_key(th.w - r[q].w), k);
-                if (c) mine[k * blockDim.x] += c;
+        for (int k = 0; k < KB; ++k) {
+            if (k >= K) break;
+            const uint32_t key[4] = {ties_key(th.x - r[k].x), ties_key(th.y - r[k].y), ties_key(th.z - r[k].z),
+                                     ties_key(th.w - r[k].w)};
+            bool in = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool over = key[j] > hi[k];
+                up[k] += over;
+                in |= !over && key[j] >= lo[k];
+            }
+            if (in) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (key[j] <= hi[k] && key[j] >= lo[k]) push(key[j], k);
             }
         }
     }
     if (blockIdx.x == 0) {
         for (int64_t i = 4 * nv + threadIdx.x; i < N; i += blockDim.x) {
             const float th = __ldg(theta + i);
-            for (int k = 0; k < K; ++k) mine[k * blockDim.x] += one(ties_key(th - ld_rep1(reps.p[k], dtype, i)), k);
+#pragma unroll
+            for (int k = 0; k < KB; ++k) {
+                if (k >= K) break;
+                const uint32_t key = ties_key(th - ld_rep1(reps.p[k], BF16 ? 1 : 0, i));
+                up[k] += key > hi[k];
+                if (key <= hi[k] && key >= lo[k]) push(key, k);
+            }
         }
+    }
+    // per worker: the block's sum of the thread counters
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+        if (k >= K) break;
+        const uint32_t t = __reduce_add_sync(0xffffffffu, up[k]);
+        if ((threadIdx.x & 31) == 0 && t) atomicAdd(&up_s[k], t);
     }
     __syncthreads();
-    // per worker: the block's sum of the thread counters (one warp per worker)
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    for (int k = warp; k < K; k += nwarps) {
-        uint32_t t = 0;
-        for (int j = lane; j < static_cast<int>(blockDim.x); j += 32) t += up_s[k * blockDim.x + j];
-        t = __reduce_add_sync(0xffffffffu, t);
-        if (lane == 0) {
-            cnt[static_cast<int64_t>(k) * G + blockIdx.x] = cnt_s[k];
-            if (t) atomicAdd(&above[k], static_cast<unsigned long long>(t));
-        }
+    if (static_cast<int>(threadIdx.x) < K) {
+        cnt[static_cast<int64_t>(threadIdx.x) * G + blockIdx.x] = cnt_s[threadIdx.x];
+        if (up_s[threadIdx.x]) atomicAdd(&above[threadIdx.x], static_cast<unsigned long long>(up_s[threadIdx.x]));
     }
+}
+
+// The bracket passes for K workers on `grid` CTAs, one per kTiesWorkers workers (theta is read
+// again by each, 4 bytes beside their 16 or 32).
+cudaError_t launch_ties_bracket(const ReplicaPtrs& reps, int K, int dtype, const float* theta, int64_t N,
+                                const uint64_t* prefix_s, uint32_t* cand, uint32_t* cnt, int64_t segcap,
+                                unsigned long long* above, int grid, cudaStream_t st) {
+    for (int w = 0; w < K; w += kTiesWorkers) {
+        const int n = K - w < kTiesWorkers ? K - w : kTiesWorkers;
+        ReplicaPtrs part = {};
+        for (int k = 0; k < n; ++k) part.p[k] = reps.p[w + k];
+        (dtype == 0 ? k_ties_bracket<false> : k_ties_bracket<true>)<<<grid, kStreamThreads, 0, st>>>(
+            part, n, theta, N, prefix_s + 2 * w, cand + static_cast<int64_t>(w) * grid * segcap,
+            cnt + static_cast<int64_t>(w) * grid, segcap, above + w);
+    }
+    return cudaGetLastError();
 }
 
 // One CTA per worker: does the bracket hold the threshold (A < n_keep <= A + candidates, no
@@ -701,10 +787,11 @@ __global__ void __launch_bounds__(256) k_ties_check(int K, int nseg, int64_t seg
 // One warp per selection: the bin holding the rank-th largest key (counting from the top),
 // appended to the prefix; the histogram row is cleared for the next pass.  Lane l holds bins
 // 8 l .. 8 l + 7; a suffix sum over the warp finds the bin.  With only_if_fail it runs only
-// when *only_if_fail != 0 (the fallback passes).
+// when *only_if_fail != 0 (the fallback passes).  widen: the last pass of the sample's bracket;
+// the prefix of an even selection (hi) gets ones, of an odd one (lo) zeros below its digits.
 __global__ void __launch_bounds__(256) k_ties_select(int nw, int pass, unsigned long long* __restrict__ hist,
                                                      uint64_t* __restrict__ rank, uint64_t* __restrict__ prefix,
-                                                     const int* __restrict__ only_if_fail) {
+                                                     const int* __restrict__ only_if_fail, int widen) {
     if (only_if_fail && *only_if_fail == 0) return;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (w >= nw) return;
@@ -748,6 +835,7 @@ __global__ void __launch_bounds__(256) k_ties_select(int nw, int pass, unsigned 
     }
     rank[w] = rr;
     prefix[w] |= static_cast<uint64_t>(digit) << ties_shift(pass);
+    if (widen && (w & 1) == 0) prefix[w] |= (1ull << ties_shift(pass)) - 1ull;
 }
 
 // TIES elect and disjoint merge.  Entry kept when its key >= the threshold (ties kept).  P and N
@@ -765,12 +853,14 @@ __device__ __forceinline__ void ties_acc(float d, uint32_t t, float& P, float& N
     }
 }
 
-__global__ void __launch_bounds__(kStreamThreads) k_ties_merge(ReplicaPtrs reps, int K, int dtype,
-                                                               float* __restrict__ theta, float* __restrict__ mom,
-                                                               int64_t N, const uint64_t* __restrict__ thr_c,
-                                                               const uint64_t* __restrict__ thr_f,
-                                                               const int* __restrict__ fail, float eta, float mu,
-                                                               uint32_t* __restrict__ err) {
+constexpr int kMergeBatch = 4;  // replicas whose loads k_ties_merge issues together
+template <bool BF16>
+__global__ void __launch_bounds__(kStreamThreads) k_ties_merge(ReplicaPtrs reps, int K, float* __restrict__ theta,
+                                                                  float* __restrict__ mom, int64_t N,
+                                                                  const uint64_t* __restrict__ thr_c,
+                                                                  const uint64_t* __restrict__ thr_f,
+                                                                  const int* __restrict__ fail, float eta, float mu,
+                                                                  uint32_t* __restrict__ err) {
     __shared__ uint32_t thr_s[kMaxK];
     const uint64_t* thr = *fail ? thr_f : thr_c;  // the bracket's result, or the fallback's
     for (int k = threadIdx.x; k < K; k += blockDim.x) thr_s[k] = static_cast<uint32_t>(thr[k]);
@@ -781,16 +871,15 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_merge(ReplicaPtrs reps,
     for (int64_t v = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; v < nv; v += stride) {
         const int64_t i = 4 * v;
         float4 th = *reinterpret_cast<const float4*>(theta + i);
-        float4 bb = *reinterpret_cast<const float4*>(mom + i);
         float P[4] = {0.f, 0.f, 0.f, 0.f}, Nn[4] = {0.f, 0.f, 0.f, 0.f}, T = 0.f;
         int cp[4] = {0, 0, 0, 0}, cn[4] = {0, 0, 0, 0};
-        for (int k0 = 0; k0 < K; k0 += kLoadBatch) {
-            float4 r[kLoadBatch];
+        for (int k0 = 0; k0 < K; k0 += kMergeBatch) {
+            float4 r[kMergeBatch];
 #pragma unroll
-            for (int q = 0; q < kLoadBatch; ++q)
-                if (k0 + q < K) r[q] = ld_rep4(reps.p[k0 + q], dtype, i);
+            for (int q = 0; q < kMergeBatch; ++q)
+                if (k0 + q < K) r[q] = ld_rep4(reps.p[k0 + q], BF16 ? 1 : 0, i);
 #pragma unroll
-            for (int q = 0; q < kLoadBatch; ++q) {
+            for (int q = 0; q < kMergeBatch; ++q) {
                 if (k0 + q >= K) break;
                 const uint32_t t = thr_s[k0 + q];
                 const float d[4] = {th.x - r[q].x, th.y - r[q].y, th.z - r[q].z, th.w - r[q].w};
@@ -802,6 +891,7 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_merge(ReplicaPtrs reps,
             }
         }
         bad |= !isfinite(T);
+        float4 bb = *reinterpret_cast<const float4*>(mom + i);
         nesterov1(th.x, bb.x, ties_u(P[0], Nn[0], cp[0], cn[0]), eta, mu);
         nesterov1(th.y, bb.y, ties_u(P[1], Nn[1], cp[1], cn[1]), eta, mu);
         nesterov1(th.z, bb.z, ties_u(P[2], Nn[2], cp[2], cn[2]), eta, mu);
@@ -814,7 +904,7 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_merge(ReplicaPtrs reps,
             float th = theta[i], bb = mom[i], P = 0.f, Nn = 0.f, T = 0.f;
             int cp = 0, cn = 0;
             for (int k = 0; k < K; ++k) {
-                const float d = th - ld_rep1(reps.p[k], dtype, i);
+                const float d = th - ld_rep1(reps.p[k], BF16 ? 1 : 0, i);
                 T += d;
                 ties_acc(d, thr_s[k], P, Nn, cp, cn);
             }
@@ -825,6 +915,14 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_merge(ReplicaPtrs reps,
         }
     }
     raise_nonfinite(bad, err);
+}
+
+cudaError_t launch_ties_merge(const ReplicaPtrs& reps, int K, int dtype, float* theta, float* mom, int64_t N,
+                              const uint64_t* thr_c, const uint64_t* thr_f, const int* fail, float eta, float mu,
+                              uint32_t* err, int grid, cudaStream_t st) {
+    (dtype == 0 ? k_ties_merge<false> : k_ties_merge<true>)<<<grid, kStreamThreads, 0, st>>>(
+        reps, K, theta, mom, N, thr_c, thr_f, fail, eta, mu, err);
+    return cudaGetLastError();
 }
 
 // fp32 [batch][rows][cols] -> bf16 (f16 = 0) or fp16 hi/lo planes with leading dimension ld.
