@@ -100,16 +100,16 @@ constexpr int kDefaultMaxIter = 28;
 constexpr float kDefaultTol = 4e-3f;
 
 // Roles of the tensor maps of one bucket.
-enum MapRole { kRoleKA = 0, kRoleKB = 1, kRoleMN = 2, kRoleST = 3 };
+enum MapRole { kRoleKA = 0, kRoleKB = 1, kRoleMN = 2, kRoleST = 3, kRoleST64 = 4 };
 // 3 sources x 3 roles x 2 planes + G (2x2) + P (2x2) + store maps (X0, X1, G, P) x 2 planes
 // + Y (operand KB, store)
 // + Gram-side buckets: Z in the first n rows of X0 / X1 (operand K-major A, MN-major, store)
 // x 2 planes, A (K-major A), W (MN-major, store) x 2 planes
-constexpr int kMapsPerBucket = 54;
+constexpr int kMapsPerBucket = 58;
 inline int src_map(int src, int role, int plane) { return (src * 3 + role) * 2 + plane; }
 inline int g_map(int role, int plane) { return 18 + role * 2 + plane; }
 inline int p_map(int role, int plane) { return 22 + role * 2 + plane; }
-// store maps (32 x 32 boxes): which 0 = X0, 1 = X1, 2 = G, 3 = P
+// store maps: which 0 = X0, 1 = X1 (64 x 32 boxes), 2 = G, 3 = P (32 x 32 boxes)
 inline int st_map(int which, int plane) { return 26 + which * 2 + plane; }
 // Gram-side maps; Z's roles: 0 K-major A, 1 MN-major, 2 store
 inline int z_map(int buf, int role, int plane) { return 36 + buf * 6 + role * 2 + plane; }
@@ -118,6 +118,8 @@ inline int w_mn_map(int plane) { return 50 + plane; }
 inline int w_st_map(int plane) { return 52 + plane; }
 inline int y_map() { return 34; }     // Y as the B operand (K-major, 256 rows)
 inline int y_st_map() { return 35; }  // Y store map
+// G and P as outputs of an update (64 x 32 boxes; the clip variants): which 0 = G, 1 = P
+inline int gp_st64_map(int which, int plane) { return 54 + which * 2 + plane; }
 
 struct Bucket {
     int rows, cols, ld, n, ld_n, count;
@@ -314,6 +316,8 @@ static bool make_map(CUtensorMap* m, const void* base, int cols, int rows, int c
         box[0] = 64; box[1] = BK; sw = CU_TENSOR_MAP_SWIZZLE_128B;
     } else if (role == kRoleST) {
         box[0] = 32; box[1] = 32; sw = CU_TENSOR_MAP_SWIZZLE_64B;
+    } else if (role == kRoleST64) {
+        box[0] = 64; box[1] = 32; sw = CU_TENSOR_MAP_SWIZZLE_128B;
     } else {
         box[0] = BK; box[1] = (role == kRoleKA) ? BM : kBRows;
         sw = (BK * 2 == 128) ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
@@ -676,13 +680,17 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
                 }
             for (int pl = 0; pl < 2; ++pl) {
                 if (!make_map(&m[st_map(0, pl)], (pl == 0 ? p->xhi[0] : p->xlo[0]) + bk.plane_off, bk.cols, bk.rows,
-                              bk.count, bk.ld, kRoleST) ||
+                              bk.count, bk.ld, kRoleST64) ||
                     !make_map(&m[st_map(1, pl)], (pl == 0 ? p->xhi[1] : p->xlo[1]) + bk.plane_off, bk.cols, bk.rows,
-                              bk.count, bk.ld, kRoleST) ||
+                              bk.count, bk.ld, kRoleST64) ||
                     !make_map(&m[st_map(2, pl)], (pl == 0 ? p->ghi : p->glo) + bk.gplane_off, bk.n, bk.n, bk.count,
                               bk.ld_n, kRoleST) ||
                     !make_map(&m[st_map(3, pl)], (pl == 0 ? p->phi : p->plo) + bk.gplane_off, bk.n, bk.n, bk.count,
-                              bk.ld_n, kRoleST))
+                              bk.ld_n, kRoleST) ||
+                    !make_map(&m[gp_st64_map(0, pl)], (pl == 0 ? p->ghi : p->glo) + bk.gplane_off, bk.n, bk.n, bk.count,
+                              bk.ld_n, kRoleST64) ||
+                    !make_map(&m[gp_st64_map(1, pl)], (pl == 0 ? p->phi : p->plo) + bk.gplane_off, bk.n, bk.n, bk.count,
+                              bk.ld_n, kRoleST64))
                     return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (store maps)");
             }
             if (!make_map(&m[y_map()], p->ypl + bk.gplane_off, bk.n, bk.n, bk.count, bk.ld_n, kRoleKB) ||
@@ -690,7 +698,7 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
                 return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (Y maps)");
             if (bk.gs) {
                 // Z in the first n rows of each matrix's slot of X0 / X1 (tall: ld = ld_n)
-                const int zroles[3] = {kRoleKA, kRoleMN, kRoleST};
+                const int zroles[3] = {kRoleKA, kRoleMN, kRoleST64};
                 for (int buf = 0; buf < 2; ++buf)
                     for (int r = 0; r < 3; ++r)
                         for (int pl = 0; pl < 2; ++pl)
@@ -702,7 +710,7 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
                     const __nv_bfloat16* w = (pl == 0 ? p->whi : p->wlo) + bk.gs_off;
                     if (!make_map(&m[an_map(pl)], a, bk.n, bk.n, bk.count, bk.ld_n, kRoleKA) ||
                         !make_map(&m[w_mn_map(pl)], w, bk.n, bk.n, bk.count, bk.ld_n, kRoleMN) ||
-                        !make_map(&m[w_st_map(pl)], w, bk.n, bk.n, bk.count, bk.ld_n, kRoleST))
+                        !make_map(&m[w_st_map(pl)], w, bk.n, bk.n, bk.count, bk.ld_n, kRoleST64))
                         return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (Gram-side A / W maps)");
                 }
             }
@@ -1574,8 +1582,8 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
                     g.b_lo = m + src_map(0, kRoleKB, 1);
                     g.out_hi = a->ghi + bk.gplane_off;
                     g.out_lo = a->glo + bk.gplane_off;
-                    g.st_hi = m + st_map(2, 0);
-                    g.st_lo = m + st_map(2, 1);
+                    g.st_hi = m + gp_st64_map(0, 0);
+                    g.st_lo = m + gp_st64_map(0, 1);
                 } else {
                     g.a_hi = m + g_map(kRoleKA, 0);
                     g.a_lo = m + g_map(kRoleKA, 1);
@@ -1583,8 +1591,8 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
                     g.b_lo = m + src_map(psrc, kRoleKB, 1);
                     g.out_hi = a->phi + bk.gplane_off;
                     g.out_lo = a->plo + bk.gplane_off;
-                    g.st_hi = m + st_map(3, 0);
-                    g.st_lo = m + st_map(3, 1);
+                    g.st_hi = m + gp_st64_map(1, 0);
+                    g.st_lo = m + gp_st64_map(1, 1);
                 }
                 set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
                 g.bucket = (int)b;

@@ -11,10 +11,10 @@
 // fp16 passes elsewhere (the operand that is not split only perturbs the iterate's
 // spectrum, which later steps correct).
 //
-// Roles (320 threads): warp 0 issues TMA loads into a ring of shared
+// Roles (352 threads): warp 0 issues TMA loads into a ring of shared
 // memory stages; warp 1 owns the tensor-memory accumulator and issues tcgen05.mma
 // from one thread; warps 2..9 drain the accumulator (tcgen05.ld) and run the
-// epilogue.  Stage hand-off uses mbarriers: `full` (TMA bytes landed), `empty`
+// epilogue; warp 10 decodes the tiles for all of them, through a queue in shared memory.  Stage hand-off uses mbarriers: `full` (TMA bytes landed), `empty`
 // (the MMAs reading a stage finished, via tcgen05.commit), `acc` (all MMAs done).
 //
 // Operand layouts: K-major operands (K contiguous in global memory) use swizzled
@@ -66,7 +66,7 @@ __device__ __forceinline__ bool decode_tile(const GemmParams& p, const int* pre,
     return true;
 }
 
-// One tile, decoded by the producer for the other roles (gi < 0: no more tiles).
+// One tile, decoded by the scheduler for the other roles (gi < 0: no more tiles).
 struct GemmTile {
     TileInfo ti;
     int gi;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
         mbar_init(drain, 1);
         for (int q = 0; q < kTileQueue; ++q) {
             mbar_init(&tq_full[q], 1);
-            mbar_init(&tq_empty[q], 1 + kEpiWarps);  // the MMA thread and one lane per epilogue warp
+            mbar_init(&tq_empty[q], kTileReaders);  // the TMA and MMA threads, a lane per epilogue warp
         }
         active_prefix(p, pre);
         *abort_flag = 0;
@@ -145,51 +145,44 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
             RingPos pos = {0, 0u};
             bool wrapped = false;  // the ring has been filled once
             int prefetched = -1;
-            const int T = pre[p.num_groups];
             int q = 0;
             uint32_t qphase = 0;
-            // cluster c takes tiles c, c + clusters, ... (both CTAs of the pair agree)
-            const int tile_stride = static_cast<int>(gridDim.x >> 1);
-            for (int t = static_cast<int>(blockIdx.x >> 1);; t += tile_stride) {
-                // decode the next tile with work (gi < 0: no more) and hand it to the MMA and
-                // epilogue warps
-                TileInfo ti;
-                int gi = -1;
-                while (t < T && !decode_tile<EPI>(p, pre, t, crank, gi, ti)) t += tile_stride;
-                if (t >= T || *abort_flag) gi = -1;
-                if (!mbar_wait(&tq_empty[q], qphase ^ 1u)) {
+            for (;;) {
+                if (!mbar_wait(&tq_full[q], qphase)) {
                     *abort_flag = 1;
                     atomicOr(p.err, kErrTimeout);
                     break;
                 }
-                tq[q].ti = ti;
-                tq[q].gi = gi;
-                mbar_arrive(&tq_full[q]);
+                const TileInfo& ti = tq[q].ti;
+                const int gi = tq[q].gi;
+                if (gi < 0) break;
+                // (after a timeout the queue only drains)
+                if (ti.run_mma && !*abort_flag) {
+                    const GemmGroup& g = p.g[gi];
+                    if (prefetched != gi) {
+                        tma_prefetch_desc(g.a_hi);
+                        tma_prefetch_desc(g.b_hi);
+                        if (ti.a_split) tma_prefetch_desc(g.a_lo);
+                        if (ti.b_split) tma_prefetch_desc(g.b_lo);
+                        prefetched = gi;
+                    }
+                    bool ok;
+                    if (g.a_mn)
+                        ok = g.b_mn ? load_tile<true, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
+                                    : load_tile<true, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
+                    else
+                        ok = g.b_mn ? load_tile<false, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
+                                    : load_tile<false, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
+                    wrapped |= pos.phase != 0u || ti.kb_end - ti.kb_begin >= nstages;
+                    if (!ok) {
+                        *abort_flag = 1;
+                        atomicOr(p.err, kErrTimeout);
+                    }
+                }
+                mbar_arrive(&tq_empty[q]);
                 if (++q == kTileQueue) {
                     q = 0;
                     qphase ^= 1u;
-                }
-                if (gi < 0) break;
-                if (!ti.run_mma) continue;
-                const GemmGroup& g = p.g[gi];
-                if (prefetched != gi) {
-                    tma_prefetch_desc(g.a_hi);
-                    tma_prefetch_desc(g.b_hi);
-                    if (ti.a_split) tma_prefetch_desc(g.a_lo);
-                    if (ti.b_split) tma_prefetch_desc(g.b_lo);
-                    prefetched = gi;
-                }
-                bool ok;
-                if (g.a_mn)
-                    ok = g.b_mn ? load_tile<true, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
-                                : load_tile<true, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
-                else
-                    ok = g.b_mn ? load_tile<false, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
-                                : load_tile<false, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
-                wrapped |= pos.phase != 0u || ti.kb_end - ti.kb_begin >= nstages;
-                if (!ok) {
-                    *abort_flag = 1;
-                    atomicOr(p.err, kErrTimeout);
                 }
             }
             if (*abort_flag) {
@@ -206,6 +199,37 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     while (globaltimer_ns() - t0 < 100000ull) {
                     }
                 }
+            }
+        }
+    } else if (warp == kSchedWarp) {
+        // ================= scheduler (one thread): decodes the cluster's tiles ahead of the other
+        // roles.  In the TMA thread the decoding of a tile (~2.5 us: cold code, one thread) came
+        // between two tiles' loads and left the MMAs waiting.
+        if (elect_one()) {
+            const int T = pre[p.num_groups];
+            int q = 0;
+            uint32_t qphase = 0;
+            // cluster c takes tiles c, c + clusters, ... (both CTAs of the pair agree)
+            const int tile_stride = static_cast<int>(gridDim.x >> 1);
+            for (int t = static_cast<int>(blockIdx.x >> 1);; t += tile_stride) {
+                // the next tile with work (gi < 0: no more)
+                TileInfo ti = {};
+                int gi = -1;
+                while (t < T && !decode_tile<EPI>(p, pre, t, crank, gi, ti)) t += tile_stride;
+                if (t >= T || *abort_flag) gi = -1;
+                if (!mbar_wait(&tq_empty[q], qphase ^ 1u)) {
+                    *abort_flag = 1;
+                    atomicOr(p.err, kErrTimeout);
+                    break;
+                }
+                tq[q].ti = ti;
+                tq[q].gi = gi;
+                mbar_arrive(&tq_full[q]);
+                if (++q == kTileQueue) {
+                    q = 0;
+                    qphase ^= 1u;
+                }
+                if (gi < 0) break;
             }
         }
     } else if (warp == 1) {

@@ -190,6 +190,116 @@ __device__ __forceinline__ void stage_store_block(const uint32_t (&w)[16], const
     }
 }
 
+// A row's share of tr(Q^T Delta) in 32 columns from c0, added to s: Q in fp32 as stored (before
+// its split into planes), Delta from its bf16 hi/lo planes.
+__device__ __forceinline__ float trace_share(const GemmGroup& g, const TileInfo& ti, const float (&v)[32], int row,
+                                             int c0, float s) {
+    const int64_t doff = ti.b * g.bf_batch_stride + static_cast<int64_t>(row) * g.ld_bf + c0;
+    const uint16_t* dh = reinterpret_cast<const uint16_t*>(g.d_hi) + doff;
+    const uint16_t* dl = reinterpret_cast<const uint16_t*>(g.d_lo) + doff;
+    if (g.N - c0 >= 32) {
+        const uint4* h4 = reinterpret_cast<const uint4*>(dh);
+        const uint4* l4 = reinterpret_cast<const uint4*>(dl);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint4 hh = h4[q], ll = l4[q];
+            const uint32_t hw[4] = {hh.x, hh.y, hh.z, hh.w};
+            const uint32_t lw[4] = {ll.x, ll.y, ll.z, ll.w};
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const float d0 = __uint_as_float(hw[w] << 16) + __uint_as_float(lw[w] << 16);
+                const float d1 = __uint_as_float(hw[w] & 0xFFFF0000u) + __uint_as_float(lw[w] & 0xFFFF0000u);
+                s = fmaf(v[8 * q + 2 * w], d0, s);
+                s = fmaf(v[8 * q + 2 * w + 1], d1, s);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            if (j < g.N - c0)
+                s = fmaf(v[j], __uint_as_float(static_cast<uint32_t>(dh[j]) << 16) +
+                                   __uint_as_float(static_cast<uint32_t>(dl[j]) << 16), s);
+    }
+    return s;
+}
+
+// Fixed-order warp reduction into this warp's slot of the tile (every slot of every tile of the
+// matrix is written by the launch that writes its Q).
+__device__ __forceinline__ void trace_store(const GemmGroup& g, const TileInfo& ti, float s, int eg, int half, int lane,
+                                            uint32_t crank) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0)
+        g.tf_part[(static_cast<int64_t>(ti.b) * (g.tiles_m * g.tiles_n) + ti.tile) * kPartSlots +
+                  static_cast<int>(crank) * kEpiWarps + half * 4 + eg] = static_cast<double>(s);
+}
+
+// Epilogue of an update tile (kEpiXSplit: X = xs acc as hi or hi and lo planes), for one warp's 32
+// rows and 128 columns.  A plane leaves 64 columns at a time through the warp's whole staging (32
+// rows of 128 bytes, 128-byte swizzle) and one TMA store: the TMA unit, which also brings the
+// operands, takes a row of up to 128 bytes every ~2 cycles, so 64-byte rows cost it twice.
+// The accumulator is read again for the second plane.  (A tile alone in a launch 16.2 -> 13.6 us,
+// 1016-wide updates 238 -> 219 us; 1024-wide ones are bound elsewhere and level.)
+template <bool ROLLED>
+__device__ __forceinline__ void update_epilogue(const TileFlags& p, const GemmGroup& g, const TileInfo& ti,
+                                                uint32_t tacc, bool ok, int eg, int half, int lane, uint32_t crank,
+                                                uint32_t stg) {
+    const int b = ti.b, row_base = ti.m0 + eg * 32, row = row_base + lane;
+    const bool row_ok = row < g.M, of16 = p.out_f16 != 0;
+    const bool have = ti.run_mma && ok;
+    const float xs = ti.xs;
+    const int nplanes = (ti.hi_only || g.st_lo == nullptr) ? 1 : 2;
+    const uint32_t row_addr = stg + lane * 128 + ((lane & 7) << 4);
+    float s_tq = 0.f;  // share of tr(Q^T Delta) (ti.trace)
+#pragma unroll 1
+    for (int c64 = half * (BN / 128); c64 < (half + 1) * (BN / 128); ++c64) {
+        const int col0 = ti.n0 + c64 * 64;
+        if (col0 >= g.N || row_base >= g.M) break;
+        constexpr int kUnroll = ROLLED ? 1 : 2;
+#pragma unroll kUnroll
+        for (int pl = 0; pl < nplanes; ++pl) {
+            if (elect_one()) bulk_wait_read0();
+            __syncwarp();
+#pragma unroll kUnroll
+            for (int h = 0; h < 2; ++h) {
+                float v[32];
+                if (have) {
+                    uint32_t r[32];
+                    tmem_ld32(tacc + (static_cast<uint32_t>(eg * 32) << 16) + c64 * 64 + h * 32, r);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * xs;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = 0.f;
+                }
+                const int c0 = col0 + h * 32;
+                if (ti.trace && pl == 0 && row_ok && c0 < g.N) s_tq = trace_share(g, ti, v, row, c0, s_tq);
+                uint32_t w[16];
+                if (pl == 0) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) w[j] = round16x2(v[2 * j], v[2 * j + 1], of16);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        uint32_t hi;
+                        split16x2(v[2 * j], v[2 * j + 1], of16, hi, w[j]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    st_shared4(row_addr ^ ((h * 4 + q) << 4), w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (elect_one()) {
+                tma_store_3d(pl == 0 ? g.st_hi : g.st_lo, stg, col0, row_base, b);
+                bulk_commit();
+            }
+        }
+    }
+    if (ti.trace) trace_store(g, ti, s_tq, eg, half, lane, crank);
+}
+
 // Epilogue of one tile's column half, run by four warps (thread (eg, lane) owns
 // output row m0 + 32 eg + lane).  `tacc` is the tensor-memory accumulator of the tile.
 // 16-bit outputs leave through the warp's shared-memory staging blocks `stg` and TMA
@@ -201,8 +311,12 @@ template <int EPI, bool ROLLED>
 __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGroup& g, const TileInfo& ti, uint32_t tacc, bool ok,
                                               int eg, int half, int lane, uint32_t crank, uint32_t stg,
                                               uint32_t& sseq) {
+    if (EPI == kEpiXSplit) {
+        update_epilogue<ROLLED>(p, g, ti, tacc, ok, eg, half, lane, crank, stg);
+        return;
+    }
     const int b = ti.b, m0 = ti.m0, n0 = ti.n0, split = ti.split;
-    const float ca = ti.ca, cb = ti.cb, cc = ti.cc, xs = ti.xs;
+    const float ca = ti.ca, cb = ti.cb, cc = ti.cc;
     const int row_base = m0 + eg * 32;
     const int row = row_base + lane;
     const bool row_ok = row < g.M;
@@ -215,7 +329,6 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
     const int lo_plane = (ti.horner || ti.hi_only || g.st_lo == nullptr) ? 0 : 1;
     const int nplanes = 1 + lo_plane + ((EPI == kEpiGram && p.gram_y) ? 1 : 0);
     float s_sq = 0.f, s_tr = 0.f, s_dev = 0.f;
-    float s_tq = 0.f;  // share of tr(Q^T Delta) (ti.trace)
     for (int c32 = half * (BN / 64); c32 < (half + 1) * (BN / 64); ++c32) {
         const int col0 = n0 + c32 * 32;
         if (col0 >= g.N || row_base >= g.M) break;
@@ -268,39 +381,6 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
 #pragma unroll
             for (int j = 0; j < 32; ++j)
                 if (j == d) v[j] += ca;
-        } else if (EPI == kEpiXSplit) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] *= xs;
-            if (ti.trace && row_ok) {
-                // this row's share of tr(Q^T Delta): Q in fp32 as stored (before its split
-                // into planes), Delta from its bf16 hi/lo planes
-                const int64_t doff = b * g.bf_batch_stride + static_cast<int64_t>(row) * g.ld_bf + col0;
-                const uint16_t* dh = reinterpret_cast<const uint16_t*>(g.d_hi) + doff;
-                const uint16_t* dl = reinterpret_cast<const uint16_t*>(g.d_lo) + doff;
-                if (nvalid == 32) {
-                    const uint4* h4 = reinterpret_cast<const uint4*>(dh);
-                    const uint4* l4 = reinterpret_cast<const uint4*>(dl);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const uint4 hh = h4[q], ll = l4[q];
-                        const uint32_t hw[4] = {hh.x, hh.y, hh.z, hh.w};
-                        const uint32_t lw[4] = {ll.x, ll.y, ll.z, ll.w};
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            const float d0 = __uint_as_float(hw[w] << 16) + __uint_as_float(lw[w] << 16);
-                            const float d1 = __uint_as_float(hw[w] & 0xFFFF0000u) + __uint_as_float(lw[w] & 0xFFFF0000u);
-                            s_tq = fmaf(v[8 * q + 2 * w], d0, s_tq);
-                            s_tq = fmaf(v[8 * q + 2 * w + 1], d1, s_tq);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (j < nvalid)
-                            s_tq = fmaf(v[j], __uint_as_float(static_cast<uint32_t>(dh[j]) << 16) +
-                                                  __uint_as_float(static_cast<uint32_t>(dl[j]) << 16), s_tq);
-                }
-            }
         }
         if (gram_fused && row_ok && sym && !diag && nvalid == 32) {
             // block strictly above the diagonal: every entry counts twice and (G - I) = G
@@ -376,15 +456,6 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
             }
             stage_store_block(w, map, stg, sseq, diag, sym, lane, col0, row_base, b);
         }
-    }
-    if (ti.trace) {
-        // fixed-order warp reduction into this warp's slot of the tile (every slot of every
-        // tile of the matrix is written by the launch that writes its Q)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s_tq += __shfl_xor_sync(0xffffffffu, s_tq, o);
-        if (lane == 0)
-            g.tf_part[(static_cast<int64_t>(b) * (g.tiles_m * g.tiles_n) + ti.tile) * kPartSlots +
-                      static_cast<int>(crank) * kEpiWarps + half * 4 + eg] = static_cast<double>(s_tq);
     }
     if (gram_fused) {
         // fixed-order warp reduction; each epilogue warp owns one of the tile's kEpiWarps slots

@@ -14,16 +14,18 @@
 // to tiles earlier in the sequence and all clusters are resident at once (cooperative launch),
 // so the walk cannot lock up; every wait is bounded all the same.
 //
-// Roles per CTA as in gemm.cu: warp 0 walks the sequence (all lanes: 32 matrices' control words
-// and states at a time), waits for operands and issues the TMA loads (one lane); warp 1 issues
-// the MMAs; warps 2..9 run the epilogues.  The ring of shared memory is cut into 16 KB slots,
+// Roles per CTA as in gemm.cu: warp 10 walks the sequence (all lanes: 32 matrices' control words
+// and states at a time) and queues this cluster's tiles; warp 0 waits for a tile's operands and
+// issues its TMA loads; warp 1 issues the MMAs; warps 2..9 run the epilogues.  The ring of shared memory is cut into 16 KB slots,
 // one operand plane each, so that single-, two- and three-pass tiles can follow one another:
 // a k-block takes two to four consecutive slots and one of kKb barrier pairs.
 //
 // Measured (GB300, whole outer step against the same kernels as a graph of launches): eight
 // matrices of 64 to 256 (K = 2) 586 -> 399 us, ragged 515-wide set (K = 3) 2052 -> 1546, the 180M set
 // (K = 8) 10.70 -> 10.12 ms; 2048- and 3072-wide sets, whose phases are hundreds of waves long,
-// are level.  A phase of a few tiles takes 7 to 13 us: operands' arrival seen ~0.4, decode and
+// are level.  A scheduler warp of its own (the TMA thread used to walk: 5,800 cycles between two
+// tiles' loads, the MMAs idle for most of them): 180M 10.23 -> 9.59 ms, 2048-wide 31.0 -> 28.6,
+// 3072-wide 21.0 -> 19.8.  A phase of a few tiles takes 7 to 13 us: operands' arrival seen ~0.4, decode and
 // loads ~1, MMAs, epilogue ~3 (its code is cold every time: ~12 cycles per instruction),
 // arrival ~1, control ~2.5.
 #include "control.cuh"
@@ -41,13 +43,16 @@ constexpr int kLoopQueue = 6;
 static_assert(kTileABytes == kTileBBytes && kSlots / 2 <= kKb, "slot ring");
 static_assert(kKb * 4 <= 32, "slot counts of the k-blocks in flight packed in 4 bits each");
 
-// One tile, decoded by warp 0 for the other roles.
+// One tile, decoded by the scheduler for the other roles.
 struct LoopTile {
     TileInfo ti;
     TileFlags f;
     int group;    // index in LoopParams::groups
     int kind;     // LoopKind, or -1: no more tiles
     int t;        // iteration
+    uint32_t want;        // arrivals at *dep that the tile's operands wait for (dep null: none)
+    const uint32_t* dep;
+    int first;    // the matrix's first tile here in this phase: its operands come from other SMs
 };
 
 // What the walk needs of a matrix's state.
@@ -251,7 +256,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
         mbar_init(drain, 1);
         for (int q = 0; q < kLoopQueue; ++q) {
             mbar_init(&tq_full[q], 1);
-            mbar_init(&tq_empty[q], 1 + kEpiWarps);
+            mbar_init(&tq_empty[q], kTileReaders);
         }
         *abort_flag = 0;
         for (int i = 0; i < 4; ++i) epi_done[i] = 0u;
@@ -268,10 +273,72 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp == 0) {
-        // ================= the walk, and the TMA loads
-        const uint32_t sbase = smem_u32(smem);
-        const uint32_t fbar0 = mapa_shared(smem_u32(full), 0);
-        SlotRing ring;
+        // ================= TMA producer (one thread)
+        if (elect_one()) {
+            const uint32_t sbase = smem_u32(smem);
+            const uint32_t fbar0 = mapa_shared(smem_u32(full), 0);
+            SlotRing ring;
+            int q = 0;
+            uint32_t qphase = 0;
+            for (;;) {
+                // (a wait for another cluster's decisions ends in the scheduler, which then says so
+                // here: longer than its limit)
+                if (!mbar_wait(&tq_full[q], qphase, 3 * kWaitTimeoutNs)) {
+                    *abort_flag = 1;
+                    atomicOr(p.err, kErrTimeout);
+                    break;
+                }
+                const LoopTile& lt = tq[q];
+                if (lt.kind < 0) break;
+                const TileInfo& ti = lt.ti;
+                if (!*abort_flag) {  // after a timeout the queue only drains
+                    bool good = true;
+                    if (lt.first) {
+                        if (lt.dep) good = wait_count(lt.dep, lt.want, p.err);
+                        fence_proxy_async_all();  // operands written by other SMs, read by TMA
+                    }
+                    if (good && ti.run_mma) {
+                        const GemmGroup& g = p.groups[lt.group].g;
+                        if (g.a_mn)
+                            good = g.b_mn ? loop_load<true, true>(g, ti, sbase, full, empty, fbar0, crank, ring)
+                                          : loop_load<true, false>(g, ti, sbase, full, empty, fbar0, crank, ring);
+                        else
+                            good = g.b_mn ? loop_load<false, true>(g, ti, sbase, full, empty, fbar0, crank, ring)
+                                          : loop_load<false, false>(g, ti, sbase, full, empty, fbar0, crank, ring);
+                    }
+                    if (!good) {
+                        *abort_flag = 1;
+                        atomicOr(p.err, kErrTimeout);
+                    }
+                }
+                mbar_arrive(&tq_empty[q]);
+                if (++q == kLoopQueue) {
+                    q = 0;
+                    qphase ^= 1u;
+                }
+            }
+            if (*abort_flag) {
+                // let the copies in flight land before the CTA exits (rank 0's barriers also
+                // count rank 1's copies; rank 1 cannot observe its own, so it leaves a margin)
+                if (leader) {
+                    int k = ring.tail;
+                    uint32_t ph = ring.tphase;
+                    for (int i = 0; i < ring.inflight; ++i) {
+                        (void)mbar_wait(&full[k], ph);
+                        if (++k == kKb) {
+                            k = 0;
+                            ph ^= 1u;
+                        }
+                    }
+                } else {
+                    const uint64_t t0 = globaltimer_ns();
+                    while (globaltimer_ns() - t0 < 100000ull) {
+                    }
+                }
+            }
+        }
+    } else if (warp == kSchedWarp) {
+        // ================= scheduler: the walk
         int q = 0;
         uint32_t qphase = 0;
         int off = 0;      // tiles handed out so far, modulo C
@@ -358,6 +425,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                         const bool has = j0 < tiles;
                         off = (off + total) % C;
                         // this cluster's matrices: their states, and whether their operands are there
+                        // (if not, the TMA thread waits for them)
                         TileState st = {};
                         bool there = true;
                         if (has) {
@@ -388,9 +456,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                             if (elect_one()) {
                                 const GemmGroup& g = p.groups[mgrp].g;
                                 const TileFlags f = L.f;
-                                bool fenced = false;
-                                for (int j = js; good && j < mt; j += C) {
-                                    if (!mbar_wait(&tq_empty[q], qphase ^ 1u) || *abort_flag) {
+                                for (int j = js; j < mt; j += C) {
+                                    if (!mbar_wait(&tq_empty[q], qphase ^ 1u, 2 * kWaitTimeoutNs) || *abort_flag) {
                                         good = false;
                                         break;
                                     }
@@ -407,26 +474,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                                     lt.group = mgrp;
                                     lt.kind = kind;
                                     lt.t = t;
+                                    lt.first = j == js;
+                                    lt.want = mwant;
+                                    lt.dep = (j == js && !ready) ? p.arr + static_cast<int64_t>(mmat) * kArrKinds + dep : nullptr;
                                     mbar_arrive(&tq_full[q]);
                                     if (++q == kLoopQueue) {
                                         q = 0;
                                         qphase ^= 1u;
                                     }
-                                    // the operands (of the first tile: the others read the same matrix)
-                                    if (!fenced) {
-                                        if (!ready)
-                                            good = wait_count(p.arr + static_cast<int64_t>(mmat) * kArrKinds + dep, mwant, p.err);
-                                        fence_proxy_async_all();  // written by other SMs, read by TMA
-                                        fenced = true;
-                                        if (!good) break;
-                                    }
-                                    if (!ti.run_mma) continue;
-                                    if (g.a_mn)
-                                        good = g.b_mn ? loop_load<true, true>(g, ti, sbase, full, empty, fbar0, crank, ring)
-                                                      : loop_load<true, false>(g, ti, sbase, full, empty, fbar0, crank, ring);
-                                    else
-                                        good = g.b_mn ? loop_load<false, true>(g, ti, sbase, full, empty, fbar0, crank, ring)
-                                                      : loop_load<false, false>(g, ti, sbase, full, empty, fbar0, crank, ring);
                                 }
                             }
                             ok = __all_sync(0xffffffffu, good);
@@ -455,25 +510,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                 tq[q].kind = -1;
                 mbar_arrive(&tq_full[q]);
             }
-            if (!ok) {
-                // let the copies in flight land before the CTA exits (rank 0's barriers also
-                // count rank 1's copies; rank 1 cannot observe its own, so it leaves a margin)
-                if (leader) {
-                    int k = ring.tail;
-                    uint32_t ph = ring.tphase;
-                    for (int i = 0; i < ring.inflight; ++i) {
-                        (void)mbar_wait(&full[k], ph);
-                        if (++k == kKb) {
-                            k = 0;
-                            ph ^= 1u;
-                        }
-                    }
-                } else {
-                    const uint64_t t0 = globaltimer_ns();
-                    while (globaltimer_ns() - t0 < 100000ull) {
-                    }
-                }
-            }
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -485,9 +521,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
             int q = 0;
             uint32_t qphase = 0;
             for (;;) {
-                // (a wait for another cluster's tiles ends in warp 0, which then says so here:
-                // twice its limit)
-                if (!mbar_wait(&tq_full[q], qphase, 2 * kWaitTimeoutNs)) {
+                if (!mbar_wait(&tq_full[q], qphase, 3 * kWaitTimeoutNs)) {
                     *abort_flag = 1;
                     atomicOr(p.err, kErrTimeout);
                     break;
@@ -506,7 +540,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                 if (!leader) continue;
                 const uint32_t buf = n & 1u, use = n >> 1;
                 ++n;
-                if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u)) {
+                if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u, 2 * kWaitTimeoutNs)) {
                     *abort_flag = 1;
                     atomicOr(p.err, kErrTimeout);
                     break;
@@ -548,7 +582,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
         int q = 0;
         uint32_t qphase = 0;
         for (;;) {
-            const bool got = __all_sync(0xffffffffu, mbar_wait(&tq_full[q], qphase, 2 * kWaitTimeoutNs));
+            const bool got = __all_sync(0xffffffffu, mbar_wait(&tq_full[q], qphase, 3 * kWaitTimeoutNs));
             if (!got) {
                 if (lane == 0) {
                     *abort_flag = 1;
@@ -567,7 +601,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
             const uint32_t buf = n & 1u, use = n >> 1;
             unsigned* through = epi_done + (n & 3u);
             ++n;
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], use & 1u));
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(&tfull[buf], use & 1u, 2 * kWaitTimeoutNs));
             if (!ok) {
                 if (lane == 0) {
                     *abort_flag = 1;

@@ -31,7 +31,8 @@ constexpr int kTileBBytes = kBRows * BK * 2;                   // one bf16 plane
 
 constexpr int kEpiWarps = 8;       // two warps per tensor-memory lane quarter
 constexpr int kPartSlots = kEpiWarps * 2;  // Gram partial sums per output tile
-constexpr int kGemmThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 MMA, warps 2.. epilogue
+constexpr int kSchedWarp = 2 + kEpiWarps;
+constexpr int kGemmThreads = 32 * (kSchedWarp + 1);  // warp 0 TMA, 1 MMA, 2.. epilogue, last the scheduler
 constexpr int kTmemCols = 256;     // one accumulator; the kernel double-buffers (512 columns)
 constexpr int kMaxGroups = 8;
 constexpr int kControlThreads = 256;  // k_control block: one warp per matrix
@@ -51,7 +52,8 @@ constexpr float kOnePassGramResid = 0.5f;
 constexpr int kStageBlockBytes = 32 * 32 * 2;
 constexpr int kStageBlocks = 2;
 constexpr int kEpiStagingBytes = kEpiWarps * kStageBlocks * kStageBlockBytes;
-constexpr int kTileQueue = 8;  // tiles handed from the producer warp to the MMA and epilogue warps
+constexpr int kTileQueue = 8;  // tiles handed from the scheduler to the other warps
+constexpr int kTileReaders = 2 + kEpiWarps;  // arrivals that give a queue slot back
 constexpr int kGemmTailBytes = 1280;  // barriers, tile queue
 constexpr int kGemmSmemBytes = kRingBytes + kEpiStagingBytes + 1024 /*align*/ + kGemmTailBytes;
 
@@ -101,7 +103,8 @@ struct GemmGroup {
     int64_t f32_split_stride, f32_batch_stride;
     int ld_f32;
     // 16-bit hi/lo output planes (kEpiGram, kEpiPoly, kEpiXSplit) and their TMA store maps
-    // (32 x 32 boxes, 64-byte swizzle); out_lo/st_lo may be null when no lo plane is kept
+    // (kEpiXSplit: boxes of 64 columns x 32 rows, 128-byte swizzle; else 32 x 32, 64-byte
+    // swizzle); out_lo/st_lo may be null when no lo plane is kept
     __nv_bfloat16* out_hi;
     __nv_bfloat16* out_lo;
     const CUtensorMap* st_hi;
