@@ -101,25 +101,27 @@ constexpr float kDefaultTol = 4e-3f;
 
 // Roles of the tensor maps of one bucket.
 enum MapRole { kRoleKA = 0, kRoleKB = 1, kRoleMN = 2, kRoleST = 3, kRoleST64 = 4 };
-// 3 sources x 3 roles x 2 planes + G (2x2) + P (2x2) + store maps (X0, X1, G, P) x 2 planes
-// + Y (operand KB, store)
-// + Gram-side buckets: Z in the first n rows of X0 / X1 (operand K-major A, MN-major, store)
-// x 2 planes, A (K-major A), W (MN-major, store) x 2 planes
-constexpr int kMapsPerBucket = 58;
+// The lo plane's map follows the hi plane's (GEMM operands count on it).
+// 3 sources x 3 roles x 2 planes; G and P (3 roles x 2); store maps: X0, X1 (64 x 32 boxes), G and
+// P (32 x 32 boxes, then 64 x 32) x 2 planes; Y: operand K-major and MN-major, store 32 x 32 and
+// 64 x 32; Gram-side buckets: Z in the first n rows of X0 / X1 (operand K-major A, MN-major,
+// store) x 2 planes, A (K-major A), W (MN-major, store) x 2 planes
+constexpr int kMapsPerBucket = 64;
 inline int src_map(int src, int role, int plane) { return (src * 3 + role) * 2 + plane; }
 inline int g_map(int role, int plane) { return 18 + role * 2 + plane; }
-inline int p_map(int role, int plane) { return 22 + role * 2 + plane; }
-// store maps: which 0 = X0, 1 = X1 (64 x 32 boxes), 2 = G, 3 = P (32 x 32 boxes)
-inline int st_map(int which, int plane) { return 26 + which * 2 + plane; }
+inline int p_map(int role, int plane) { return 24 + role * 2 + plane; }
+// from an operand's map to the MN-major one of the same matrix (GemmGroup::a_tri, b_tri)
+constexpr int kTriA = 2 * (kRoleMN - kRoleKA), kTriB = 2 * (kRoleMN - kRoleKB), kTriY = 1;
+inline int x_st_map(int buf, int plane) { return 30 + buf * 2 + plane; }
+// which: 0 = G, 1 = P; the 64 x 32 box's map kSt64 further
+inline int gp_st_map(int which, int plane) { return 34 + which * 4 + plane; }
+inline int y_map() { return 42; }     // Y as the B operand (K-major), MN-major kTriY further
+inline int y_st_map() { return 44; }  // kStY64 further: 64 x 32 boxes
 // Gram-side maps; Z's roles: 0 K-major A, 1 MN-major, 2 store
-inline int z_map(int buf, int role, int plane) { return 36 + buf * 6 + role * 2 + plane; }
-inline int an_map(int plane) { return 48 + plane; }
-inline int w_mn_map(int plane) { return 50 + plane; }
-inline int w_st_map(int plane) { return 52 + plane; }
-inline int y_map() { return 34; }     // Y as the B operand (K-major, 256 rows)
-inline int y_st_map() { return 35; }  // Y store map
-// G and P as outputs of an update (64 x 32 boxes; the clip variants): which 0 = G, 1 = P
-inline int gp_st64_map(int which, int plane) { return 54 + which * 2 + plane; }
+inline int z_map(int buf, int role, int plane) { return 46 + buf * 6 + role * 2 + plane; }
+inline int an_map(int plane) { return 58 + plane; }
+inline int w_mn_map(int plane) { return 60 + plane; }
+inline int w_st_map(int plane) { return 62 + plane; }
 
 struct Bucket {
     int rows, cols, ld, n, ld_n, count;
@@ -670,7 +672,7 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
                         if (!make_map(&m[src_map(s, role, pl)], base, bk.cols, bk.rows, bk.count, bk.ld, role))
                             return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (iterate planes)");
                     }
-            for (int role = 0; role < 2; ++role)
+            for (int role = 0; role < 3; ++role)
                 for (int pl = 0; pl < 2; ++pl) {
                     if (!make_map(&m[g_map(role, pl)], (pl == 0 ? p->ghi : p->glo) + bk.gplane_off, bk.n, bk.n,
                                   bk.count, bk.ld_n, role) ||
@@ -679,22 +681,23 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
                         return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (Gram planes)");
                 }
             for (int pl = 0; pl < 2; ++pl) {
-                if (!make_map(&m[st_map(0, pl)], (pl == 0 ? p->xhi[0] : p->xlo[0]) + bk.plane_off, bk.cols, bk.rows,
-                              bk.count, bk.ld, kRoleST64) ||
-                    !make_map(&m[st_map(1, pl)], (pl == 0 ? p->xhi[1] : p->xlo[1]) + bk.plane_off, bk.cols, bk.rows,
-                              bk.count, bk.ld, kRoleST64) ||
-                    !make_map(&m[st_map(2, pl)], (pl == 0 ? p->ghi : p->glo) + bk.gplane_off, bk.n, bk.n, bk.count,
-                              bk.ld_n, kRoleST) ||
-                    !make_map(&m[st_map(3, pl)], (pl == 0 ? p->phi : p->plo) + bk.gplane_off, bk.n, bk.n, bk.count,
-                              bk.ld_n, kRoleST) ||
-                    !make_map(&m[gp_st64_map(0, pl)], (pl == 0 ? p->ghi : p->glo) + bk.gplane_off, bk.n, bk.n, bk.count,
-                              bk.ld_n, kRoleST64) ||
-                    !make_map(&m[gp_st64_map(1, pl)], (pl == 0 ? p->phi : p->plo) + bk.gplane_off, bk.n, bk.n, bk.count,
-                              bk.ld_n, kRoleST64))
-                    return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (store maps)");
+                for (int buf = 0; buf < 2; ++buf)
+                    if (!make_map(&m[x_st_map(buf, pl)], (pl == 0 ? p->xhi[buf] : p->xlo[buf]) + bk.plane_off, bk.cols,
+                                  bk.rows, bk.count, bk.ld, kRoleST64))
+                        return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (store maps)");
+                for (int which = 0; which < 2; ++which) {
+                    const __nv_bfloat16* base = which == 0 ? (pl == 0 ? p->ghi : p->glo) : (pl == 0 ? p->phi : p->plo);
+                    for (int wide = 0; wide < 2; ++wide)
+                        if (!make_map(&m[gp_st_map(which, pl) + (wide ? kSt64 : 0)], base + bk.gplane_off, bk.n, bk.n,
+                                      bk.count, bk.ld_n, wide ? kRoleST64 : kRoleST))
+                            return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (store maps)");
+                }
             }
-            if (!make_map(&m[y_map()], p->ypl + bk.gplane_off, bk.n, bk.n, bk.count, bk.ld_n, kRoleKB) ||
-                !make_map(&m[y_st_map()], p->ypl + bk.gplane_off, bk.n, bk.n, bk.count, bk.ld_n, kRoleST))
+            const __nv_bfloat16* y = p->ypl + bk.gplane_off;
+            if (!make_map(&m[y_map()], y, bk.n, bk.n, bk.count, bk.ld_n, kRoleKB) ||
+                !make_map(&m[y_map() + kTriY], y, bk.n, bk.n, bk.count, bk.ld_n, kRoleMN) ||
+                !make_map(&m[y_st_map()], y, bk.n, bk.n, bk.count, bk.ld_n, kRoleST) ||
+                !make_map(&m[y_st_map() + kStY64], y, bk.n, bk.n, bk.count, bk.ld_n, kRoleST64))
                 return fail(ISOLOCO_ERR_CUDA, "cuTensorMapEncodeTiled failed (Y maps)");
             if (bk.gs) {
                 // Z in the first n rows of each matrix's slot of X0 / X1 (tall: ld = ld_n)
@@ -908,9 +911,7 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
             const int zb = t & 1;  // ping-pong buffer holding Z_t
             GemmGroup w{};
             w.a_hi = m + an_map(0);
-            w.a_lo = m + an_map(1);
             w.b_hi = m + z_map(zb, 1, 0);
-            w.b_lo = m + z_map(zb, 1, 1);
             set_group_common(w, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
             w.bucket = (int)b;
             w.out_hi = p->whi + bk.gs_off;
@@ -921,15 +922,13 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
             w.ld_bf = bk.ld_n;
             wset.add(w, false, true);
             g.a_hi = m + z_map(zb, 1, 0);
-            g.a_lo = m + z_map(zb, 1, 1);
             g.b_hi = m + w_mn_map(0);
-            g.b_lo = m + w_mn_map(1);
             set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
             g.out_hi = p->ghi + bk.gplane_off;
             g.out_lo = p->glo + bk.gplane_off;
-            g.st_hi = m + st_map(2, 0);
-            g.st_lo = m + st_map(2, 1);
+            g.st_hi = m + gp_st_map(0, 0);
+            g.st_lo = m + gp_st_map(0, 1);
             g.st_y = m + y_st_map();
             g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
             g.ld_bf = bk.ld_n;
@@ -942,9 +941,7 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
         const int role_a = bk.tall ? kRoleMN : kRoleKA;
         const int role_b = bk.tall ? kRoleMN : kRoleKB;
         g.a_hi = m + src_map(src, role_a, 0);
-        g.a_lo = m + src_map(src, role_a, 1);
         g.b_hi = m + src_map(src, role_b, 0);
-        g.b_lo = m + src_map(src, role_b, 1);
         set_group_common(g, bk.n, bk.n, bk.tall ? bk.rows : bk.cols, bk.count, bk.splits, bk.mat_base);
         g.bucket = (int)b;
         g.out_f32 = p->gpart + bk.gpart_off;
@@ -953,8 +950,8 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
         g.ld_f32 = bk.ld_n;
         g.out_hi = p->ghi + bk.gplane_off;
         g.out_lo = p->glo + bk.gplane_off;
-        g.st_hi = m + st_map(2, 0);
-        g.st_lo = m + st_map(2, 1);
+        g.st_hi = m + gp_st_map(0, 0);
+        g.st_lo = m + gp_st_map(0, 1);
         g.st_y = m + y_st_map();
         g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
         g.ld_bf = bk.ld_n;
@@ -974,15 +971,15 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
         const CUtensorMap* m = maps + b * kMapsPerBucket;
         GemmGroup g{};
         g.a_hi = m + g_map(kRoleKA, 0);
-        g.a_lo = m + g_map(kRoleKA, 1);
         g.b_hi = (first || full) ? m + g_map(kRoleKB, 0) : m + y_map();  // G G or G Y (Horner)
-        g.b_lo = m + g_map(kRoleKB, 1);
+        g.a_tri = kTriA;
+        g.b_tri = (first || full) ? kTriB : kTriY;
         set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
         g.bucket = (int)b;
         g.out_hi = p->phi + bk.gplane_off;
         g.out_lo = p->plo + bk.gplane_off;
-        g.st_hi = m + st_map(3, 0);
-        g.st_lo = m + st_map(3, 1);
+        g.st_hi = m + gp_st_map(1, 0);
+        g.st_lo = m + gp_st_map(1, 1);
         g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
         g.ld_bf = bk.ld_n;
         g.g_hi = p->ghi + bk.gplane_off;
@@ -1007,9 +1004,8 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
             if (first) continue;  // Z_1 = P_0: k_gs_init below
             // Z_{t+1} = Z_t P_t in the first n rows of the other buffer
             g.a_hi = m + z_map(t & 1, 0, 0);
-            g.a_lo = m + z_map(t & 1, 0, 1);
             g.b_hi = m + p_map(kRoleKB, 0);
-            g.b_lo = m + p_map(kRoleKB, 1);
+            g.b_tri = kTriB;
             set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
             g.out_hi = p->xhi[dst] + bk.plane_off;
@@ -1023,21 +1019,19 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
         }
         if (bk.tall) {
             g.a_hi = m + src_map(src, kRoleKA, 0);
-            g.a_lo = m + src_map(src, kRoleKA, 1);
             g.b_hi = m + p_map(kRoleKB, 0);
-            g.b_lo = m + p_map(kRoleKB, 1);
+            g.b_tri = kTriB;
         } else {
             g.a_hi = m + p_map(kRoleKA, 0);
-            g.a_lo = m + p_map(kRoleKA, 1);
+            g.a_tri = kTriA;
             g.b_hi = m + src_map(src, kRoleMN, 0);
-            g.b_lo = m + src_map(src, kRoleMN, 1);
         }
         set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
         g.bucket = (int)b;
         g.out_hi = p->xhi[dst] + bk.plane_off;
         g.out_lo = p->xlo[dst] + bk.plane_off;
-        g.st_hi = m + st_map(dst, 0);
-        g.st_lo = m + st_map(dst, 1);
+        g.st_hi = m + x_st_map(dst, 0);
+        g.st_lo = m + x_st_map(dst, 1);
         g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
         g.ld_bf = bk.ld;
         set_one_pass(p, g, bk, true);
@@ -1265,16 +1259,14 @@ static int gs_final(isoloco_plan* p, cudaStream_t st) {
         for (int fb = 0; fb < 2; ++fb) {
             GemmGroup g{};
             g.a_hi = m + src_map(0, kRoleKA, 0);
-            g.a_lo = m + src_map(0, kRoleKA, 1);
             g.b_hi = m + w_mn_map(0);
-            g.b_lo = m + w_mn_map(1);
             set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
             g.gate_fb = fb + 1;
             g.out_hi = p->xhi[1 - fb] + bk.plane_off;
             g.out_lo = p->xlo[1 - fb] + bk.plane_off;
-            g.st_hi = m + st_map(1 - fb, 0);
-            g.st_lo = m + st_map(1 - fb, 1);
+            g.st_hi = m + x_st_map(1 - fb, 0);
+            g.st_lo = m + x_st_map(1 - fb, 1);
             g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
             g.ld_bf = bk.ld;
             g.d_hi = p->dhi + bk.plane_off;  // Q is final: tr(Q^T Delta) in the epilogue
@@ -1456,14 +1448,10 @@ static int form_h(isoloco_plan* p, cudaStream_t st) {
             GemmGroup g{};
             if (bk.tall) {
                 g.a_hi = m + src_map(qsrc, kRoleMN, 0);
-                g.a_lo = m + src_map(qsrc, kRoleMN, 1);
                 g.b_hi = m + src_map(0, kRoleMN, 0);
-                g.b_lo = m + src_map(0, kRoleMN, 1);
             } else {
                 g.a_hi = m + src_map(0, kRoleKA, 0);
-                g.a_lo = m + src_map(0, kRoleKA, 1);
                 g.b_hi = m + src_map(qsrc, kRoleKB, 0);
-                g.b_lo = m + src_map(qsrc, kRoleKB, 1);
             }
             set_group_common(g, bk.n, bk.n, bk.tall ? bk.rows : bk.cols, bk.count, bk.splits, bk.mat_base);
             g.bucket = (int)b;
@@ -1577,22 +1565,18 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
                 GemmGroup g{};
                 if (step == 0) {
                     g.a_hi = m + src_map(psrc, kRoleKA, 0);
-                    g.a_lo = m + src_map(psrc, kRoleKA, 1);
                     g.b_hi = m + src_map(0, kRoleKB, 0);
-                    g.b_lo = m + src_map(0, kRoleKB, 1);
                     g.out_hi = a->ghi + bk.gplane_off;
                     g.out_lo = a->glo + bk.gplane_off;
-                    g.st_hi = m + gp_st64_map(0, 0);
-                    g.st_lo = m + gp_st64_map(0, 1);
+                    g.st_hi = m + gp_st_map(0, 0) + kSt64;
+                    g.st_lo = m + gp_st_map(0, 1) + kSt64;
                 } else {
                     g.a_hi = m + g_map(kRoleKA, 0);
-                    g.a_lo = m + g_map(kRoleKA, 1);
                     g.b_hi = m + src_map(psrc, kRoleKB, 0);
-                    g.b_lo = m + src_map(psrc, kRoleKB, 1);
                     g.out_hi = a->phi + bk.gplane_off;
                     g.out_lo = a->plo + bk.gplane_off;
-                    g.st_hi = m + gp_st64_map(1, 0);
-                    g.st_lo = m + gp_st64_map(1, 1);
+                    g.st_hi = m + gp_st_map(1, 0) + kSt64;
+                    g.st_lo = m + gp_st_map(1, 1) + kSt64;
                 }
                 set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
                 g.bucket = (int)b;
@@ -1622,22 +1606,18 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
             GemmGroup g{};
             if (bk.tall) {
                 g.a_hi = m + src_map(src, kRoleKA, 0);
-                g.a_lo = m + src_map(src, kRoleKA, 1);
                 g.b_hi = m + p_map(kRoleKB, 0);
-                g.b_lo = m + p_map(kRoleKB, 1);
             } else {
                 g.a_hi = m + p_map(kRoleKA, 0);
-                g.a_lo = m + p_map(kRoleKA, 1);
                 g.b_hi = m + src_map(src, kRoleMN, 0);
-                g.b_lo = m + src_map(src, kRoleMN, 1);
             }
             set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
             g.gate_fb = fb + 1;
             g.out_hi = p->xhi[dst] + bk.plane_off;
             g.out_lo = p->xlo[dst] + bk.plane_off;
-            g.st_hi = m + st_map(dst, 0);
-            g.st_lo = m + st_map(dst, 1);
+            g.st_hi = m + x_st_map(dst, 0);
+            g.st_lo = m + x_st_map(dst, 1);
             g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
             g.ld_bf = bk.ld;
             us.add(g, false, !bk.tall);
@@ -2227,7 +2207,8 @@ int isoloco_debug_gemm(int a_mn, int b_mn, int precision, int batch, int M, int 
     gp.b_split = (precision == 0 || precision == 2 || precision == 3) ? 1 : 0;
     gp.err = err;
     GemmGroup& g = gp.g[0];
-    g.a_hi = maps_d; g.a_lo = maps_d + 1; g.b_hi = maps_d + 2; g.b_lo = maps_d + 3;
+    g.a_hi = maps_d;
+    g.b_hi = maps_d + 2;
     g.a_mn = a_mn != 0 ? 1 : 0;
     g.b_mn = b_mn != 0 ? 1 : 0;
     g.a_split = gp.a_split;
@@ -2345,7 +2326,8 @@ int isoloco_debug_gemm_noalloc(int a_mn, int b_mn, int precision, int batch, int
     gp.b_split = (precision == 0 || precision == 2 || precision == 3) ? 1 : 0;
     gp.err = err;
     GemmGroup& g = gp.g[0];
-    g.a_hi = maps_d; g.a_lo = maps_d + 1; g.b_hi = maps_d + 2; g.b_lo = maps_d + 3;
+    g.a_hi = maps_d;
+    g.b_hi = maps_d + 2;
     g.a_mn = a_mn != 0 ? 1 : 0;
     g.b_mn = b_mn != 0 ? 1 : 0;
     g.a_split = gp.a_split;

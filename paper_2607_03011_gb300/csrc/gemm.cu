@@ -162,17 +162,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     if (prefetched != gi) {
                         tma_prefetch_desc(g.a_hi);
                         tma_prefetch_desc(g.b_hi);
-                        if (ti.a_split) tma_prefetch_desc(g.a_lo);
-                        if (ti.b_split) tma_prefetch_desc(g.b_lo);
+                        if (ti.a_split) tma_prefetch_desc(g.a_hi + 1);
+                        if (ti.b_split) tma_prefetch_desc(g.b_hi + 1);
                         prefetched = gi;
                     }
-                    bool ok;
-                    if (g.a_mn)
-                        ok = g.b_mn ? load_tile<true, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
-                                    : load_tile<true, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
-                    else
-                        ok = g.b_mn ? load_tile<false, true>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos)
-                                    : load_tile<false, false>(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
+                    const bool ok = load_tile(g, ti, sbase, stage_stride, nstages, full, empty, fbar0, crank, pos);
                     wrapped |= pos.phase != 0u || ti.kb_end - ti.kb_begin >= nstages;
                     if (!ok) {
                         *abort_flag = 1;
@@ -246,8 +240,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     atomicOr(p.err, kErrTimeout);
                     break;
                 }
-                const int gi = tq[q].gi, nkb = tq[q].ti.kb_end - tq[q].ti.kb_begin;
-                const bool run = tq[q].ti.run_mma, as = tq[q].ti.a_split, bs = tq[q].ti.b_split;
+                const int gi = tq[q].gi;
+                const TileInfo ti = tq[q].ti;
                 mbar_arrive(&tq_empty[q]);
                 if (++q == kTileQueue) {
                     q = 0;
@@ -263,23 +257,26 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     break;
                 }
                 tc_fence_after();
-                if (run) {
-                    // instruction and operand descriptors for the layouts of this tile's group
-                    const bool a_mn = p.g[gi].a_mn != 0, b_mn = p.g[gi].b_mn != 0;
-                    const uint32_t tacc = tmem_base + buf * kTmemCols;
-                    const uint32_t idesc = make_idesc_16bit(kTileM, BN, a_mn, b_mn, p.in_f16 != 0);
-                    const uint64_t da = operand_desc(sbase, a_mn);
-                    const uint64_t db = operand_desc(sbase + kTileABytes * (as ? 2u : 1u), b_mn);
-                    const uint32_t a_lo = static_cast<uint32_t>(da), a_hi = static_cast<uint32_t>(da >> 32);
-                    const uint32_t b_lo = static_cast<uint32_t>(db), b_hi = static_cast<uint32_t>(db >> 32);
-                    const uint32_t sa = slice_step(a_mn), sb = slice_step(b_mn), st16 = stage_stride >> 4;
-                    bool ok;
-                    if (as)
-                        ok = bs ? issue_tile<true, true>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos)
-                                : issue_tile<true, false>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos);
-                    else
-                        ok = bs ? issue_tile<false, true>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos)
-                                : issue_tile<false, false>(full, empty, nstages, st16, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos);
+                if (ti.run_mma) {
+                    const bool as = ti.a_split, bs = ti.b_split;
+                    const uint32_t tacc = tmem_base + buf * kTmemCols, st16 = stage_stride >> 4;
+                    uint32_t acc = 0u;
+                    const bool ok = for_k_runs(ti, [&](int from, int to, bool at, bool bt) {
+                        // instruction and operand descriptors for the layouts of this run
+                        const bool a_mn = p.g[gi].a_mn || at, b_mn = p.g[gi].b_mn || bt;
+                        const uint32_t idesc = make_idesc_16bit(kTileM, BN, a_mn, b_mn, p.in_f16 != 0);
+                        const uint64_t da = operand_desc(sbase, a_mn);
+                        const uint64_t db = operand_desc(sbase + kTileABytes * (as ? 2u : 1u), b_mn);
+                        const uint32_t a_lo = static_cast<uint32_t>(da), a_hi = static_cast<uint32_t>(da >> 32);
+                        const uint32_t b_lo = static_cast<uint32_t>(db), b_hi = static_cast<uint32_t>(db >> 32);
+                        const uint32_t sa = slice_step(a_mn), sb = slice_step(b_mn);
+                        const int n = to - from;
+                        if (as)
+                            return bs ? issue_tile<true, true>(full, empty, nstages, st16, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc)
+                                      : issue_tile<true, false>(full, empty, nstages, st16, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc);
+                        return bs ? issue_tile<false, true>(full, empty, nstages, st16, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc)
+                                  : issue_tile<false, false>(full, empty, nstages, st16, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc);
+                    });
                     if (!ok) {
                         *abort_flag = 1;
                         atomicOr(p.err, kErrTimeout);
@@ -299,7 +296,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
         const int eg = warp & 3;  // tensor-memory lane quarter this warp may access
         const int half = (warp - 2) >> 2;
         uint32_t n = 0;
-        uint32_t sseq = 0;  // this warp's staged stores so far (staging block rotation)
         int q = 0;
         uint32_t qphase = 0;
         for (;;) {
@@ -322,7 +318,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
             __syncwarp();
             tc_fence_after();
             tile_epilogue<EPI, false>(tile_flags(p), p.g[gi], ti, tmem_base + buf * kTmemCols, ok, eg, half, lane, crank,
-                          smem_u32(staging) + (warp - 2) * kStageBlocks * kStageBlockBytes, sseq);
+                          smem_u32(staging) + (warp - 2) * kStageBlocks * kStageBlockBytes);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {

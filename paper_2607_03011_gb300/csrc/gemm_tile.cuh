@@ -41,6 +41,7 @@ __device__ __forceinline__ void sym_tile(int t, int tiles_m, int tiles_n, int& t
 // Everything a role needs to know about one output tile of a group.
 struct TileInfo {
     int b, tile, split, m0, n0, mat, kb_begin, kb_end;
+    int a_sw, b_sw;  // k-blocks below these come from the transposed tile (GemmGroup::a_tri, b_tri)
     bool run_mma, a_split, b_split;
     bool horner;     // kEpiPoly: P = acc + a I (the MMA computed G Y); else P = a I + b G + c acc
     bool hi_only;    // write the hi plane only (a single-pass Gram's G; an update's X whose lo
@@ -109,6 +110,27 @@ __device__ __forceinline__ void setup_tile(const TileFlags& f, const GemmGroup& 
     ti.kb_begin = split * g.kblocks_per_split;
     ti.kb_end = min(total_kb, ti.kb_begin + g.kblocks_per_split);
     if (ti.kb_begin >= ti.kb_end) ti.run_mma = false;
+    ti.a_sw = g.a_tri ? tm * (kTileM / BK) : 0;
+    ti.b_sw = g.b_tri ? tn * (BN / BK) : 0;
+}
+
+// (Symmetric G, Y, P with only the tiles on and above the diagonal stored: mirroring each tile
+// cost the Gram's epilogue, which bounds its phase, half of its 20,000 cycles per tile, and 40 %
+// of the planes' writes.  A step on 12 layers of 1024 x 2816, 8 replicas: 10.01 -> 9.71 ms.)
+// Calls f(from, to, a transposed, b transposed) for the runs of a tile's k-blocks that read both
+// operands in one layout; stops when f returns false.
+template <class F>
+__device__ __forceinline__ bool for_k_runs(const TileInfo& ti, F f) {
+    const int end = ti.kb_end;
+    for (int k = ti.kb_begin; k < end;) {
+        const bool at = k < ti.a_sw, bt = k < ti.b_sw;
+        int to = end;
+        if (at) to = min(to, ti.a_sw);
+        if (bt) to = min(to, ti.b_sw);
+        if (!f(k, to, at, bt)) return false;
+        k = to;
+    }
+    return true;
 }
 
 // Staging of an epilogue warp: blocks of 32 x 32 16-bit values with 64-byte rows whose 16-byte
@@ -140,29 +162,19 @@ __device__ __forceinline__ void stage_transposed(const uint32_t (&w)[16], uint32
     }
 }
 
-// One warp writes a 32 x 32 block of 16-bit values (lane = row, w = the lane's 32 values
-// packed in pairs) to staging and stores it with TMA at (col0, row_base, b): the diagonal
-// block is made symmetric (each row takes what lies left of the diagonal from the transpose);
-// an off-diagonal block of a symmetric output is also stored transposed at (row_base, col0, b).
-// `stg` is the warp's two blocks and `seq` counts its stores (one bulk group each): a
-// symmetric store takes both once the store before it has read them, any other store
-// alternates them.
+// One warp writes a 32 x 32 block of a diagonal tile (16-bit values, lane = row, w = the lane's 32
+// values packed in pairs) to staging and stores it with TMA at (col0, row_base, b).  The block
+// on the diagonal (diag) is made symmetric (each row takes what lies left of the diagonal from
+// the transpose); another is also stored transposed at (row_base, col0, b).  `stg` is the
+// warp's two blocks, taken once the store before has read them.
 __device__ __forceinline__ void stage_store_block(const uint32_t (&w)[16], const CUtensorMap* map, uint32_t stg,
-                                                  uint32_t& seq, bool diag, bool sym, int lane, int col0,
-                                                  int row_base, int b) {
-    static_assert(kStageBlocks == 2, "block rotation below handles two blocks");
-    const uint32_t sd = sym ? stg : stg + (seq & 1u) * kStageBlockBytes;
-    const uint32_t sm = stg + kStageBlockBytes;  // transposed block (symmetric outputs only)
-    if (elect_one()) {
-        if (sym)
-            bulk_wait_read0();
-        else
-            bulk_wait_read1();
-    }
-    ++seq;
+                                                  bool diag, int lane, int col0, int row_base, int b) {
+    static_assert(kStageBlocks == 2, "a block and its transpose");
+    const uint32_t sm = stg + kStageBlockBytes;  // the transpose
+    if (elect_one()) bulk_wait_read0();
     __syncwarp();
-    if (sym) stage_transposed(w, sm, lane);
-    const uint32_t row = stage_row_addr(sd, lane);
+    stage_transposed(w, sm, lane);
+    const uint32_t row = stage_row_addr(stg, lane);
     if (diag) {
         __syncwarp();
         const uint32_t trow = stage_row_addr(sm, lane);
@@ -184,8 +196,8 @@ __device__ __forceinline__ void stage_store_block(const uint32_t (&w)[16], const
     fence_proxy_async_smem();
     __syncwarp();
     if (elect_one()) {
-        tma_store_3d(map, sd, col0, row_base, b);
-        if (sym && !diag) tma_store_3d(map, sm, row_base, col0, b);
+        tma_store_3d(map, stg, col0, row_base, b);
+        if (!diag) tma_store_3d(map, sm, row_base, col0, b);
         bulk_commit();
     }
 }
@@ -234,57 +246,144 @@ __device__ __forceinline__ void trace_store(const GemmGroup& g, const TileInfo& 
                   static_cast<int>(crank) * kEpiWarps + half * 4 + eg] = static_cast<double>(s);
 }
 
-// Epilogue of an update tile (kEpiXSplit: X = xs acc as hi or hi and lo planes), for one warp's 32
-// rows and 128 columns.  A plane leaves 64 columns at a time through the warp's whole staging (32
-// rows of 128 bytes, 128-byte swizzle) and one TMA store: the TMA unit, which also brings the
-// operands, takes a row of up to 128 bytes every ~2 cycles, so 64-byte rows cost it twice.
-// The accumulator is read again for the second plane.  (A tile alone in a launch 16.2 -> 13.6 us,
-// 1016-wide updates 238 -> 219 us; 1024-wide ones are bound elsewhere and level.)
-template <bool ROLLED>
-__device__ __forceinline__ void update_epilogue(const TileFlags& p, const GemmGroup& g, const TileInfo& ti,
-                                                uint32_t tacc, bool ok, int eg, int half, int lane, uint32_t crank,
-                                                uint32_t stg) {
+// The 16-bit words of one plane of 32 values: kind 0 hi, 1 lo, 2 Y = yb I + yc G (hi plane only,
+// it is the single operand of G Y), its diagonal at column d if diag.
+__device__ __forceinline__ void plane_words(const float (&v)[32], int kind, bool of16, float yb, float yc, bool diag,
+                                            int d, uint32_t (&w)[16]) {
+    if (kind == 0) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) w[j] = round16x2(v[2 * j], v[2 * j + 1], of16);
+    } else if (kind == 1) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            uint32_t hi;
+            split16x2(v[2 * j], v[2 * j + 1], of16, hi, w[j]);
+        }
+    } else if (diag) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            w[j] = round16x2(yc * v[2 * j] + (2 * j == d ? yb : 0.f), yc * v[2 * j + 1] + (2 * j + 1 == d ? yb : 0.f), of16);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) w[j] = round16x2(yc * v[2 * j], yc * v[2 * j + 1], of16);
+    }
+}
+
+// kEpiPoly without Horner's form: v = cc v + cb G for this lane's row and 32 columns from c0 (G past
+// L1: within the polar loop other SMs rewrite it in every iteration).
+__device__ __forceinline__ void add_gram(const GemmGroup& g, const TileInfo& ti, bool f16, int row, int c0,
+                                         float (&v)[32]) {
+    const int64_t goff = ti.b * g.bf_batch_stride + static_cast<int64_t>(row) * g.ld_bf + c0;
+    const uint16_t* gh = reinterpret_cast<const uint16_t*>(g.g_hi) + goff;
+    const uint16_t* gl = reinterpret_cast<const uint16_t*>(g.g_lo) + goff;
+    const float cb = ti.cb, cc = ti.cc;
+    if (g.N - c0 >= 32) {
+        const uint4* h4 = reinterpret_cast<const uint4*>(gh);
+        const uint4* l4 = reinterpret_cast<const uint4*>(gl);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint4 hh = __ldcg(h4 + q), ll = __ldcg(l4 + q);
+            const uint32_t hw[4] = {hh.x, hh.y, hh.z, hh.w};
+            const uint32_t lw[4] = {ll.x, ll.y, ll.z, ll.w};
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const float g0 = dec16(hw[w] & 0xFFFFu, f16) + dec16(lw[w] & 0xFFFFu, f16);
+                const float g1 = dec16(hw[w] >> 16, f16) + dec16(lw[w] >> 16, f16);
+                v[8 * q + 2 * w] = cc * v[8 * q + 2 * w] + cb * g0;
+                v[8 * q + 2 * w + 1] = cc * v[8 * q + 2 * w + 1] + cb * g1;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            if (j < g.N - c0) v[j] = cc * v[j] + cb * (dec16(__ldcg(gh + j), f16) + dec16(__ldcg(gl + j), f16));
+    }
+}
+
+// A Gram tile's partial sums (sum of squares, trace, squared distance from I; an entry off the
+// diagonal counts for its mirror too): fixed-order warp reduction into this warp's slot.
+__device__ __forceinline__ void gram_sums_store(const GemmGroup& g, const TileInfo& ti, float sq, float tr, float dev,
+                                                int eg, int half, int lane, uint32_t crank) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        tr += __shfl_xor_sync(0xffffffffu, tr, o);
+        dev += __shfl_xor_sync(0xffffffffu, dev, o);
+    }
+    if (lane == 0) {
+        const int ntiles = g.sym ? g.tiles_sym : g.tiles_m * g.tiles_n;
+        float* slot = g.part + ((g.part_base + static_cast<int64_t>(ti.b) * ntiles + ti.tile) * kPartSlots +
+                                static_cast<int>(crank) * kEpiWarps + half * 4 + eg) * 3;
+        slot[0] = sq;
+        slot[1] = tr;
+        slot[2] = dev;
+    }
+}
+
+// Epilogue of an update tile (kEpiXSplit: X = xs acc) or of a tile above the diagonal of a
+// symmetric output (Gram, polynomial), for one warp's 32 rows and 128 columns.  A plane leaves
+// 64 columns at a time through the warp's whole staging (32 rows of 128 bytes, 128-byte
+// swizzle) and one TMA store: the TMA unit, which also brings the operands, takes a row of up
+// to 128 bytes every ~2 cycles, so 64-byte rows cost it twice.  The accumulator is read again
+// for each plane.  (A tile alone in a launch 16.2 -> 13.6 us, 1016-wide updates 238 -> 219 us;
+// 1024-wide ones are bound elsewhere and level.)
+template <int EPI, bool ROLLED>
+__device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGroup& g, const TileInfo& ti,
+                                              uint32_t tacc, bool ok, int eg, int half, int lane, uint32_t crank,
+                                              uint32_t stg) {
     const int b = ti.b, row_base = ti.m0 + eg * 32, row = row_base + lane;
     const bool row_ok = row < g.M, of16 = p.out_f16 != 0;
     const bool have = ti.run_mma && ok;
-    const float xs = ti.xs;
-    const int nplanes = (ti.hi_only || g.st_lo == nullptr) ? 1 : 2;
+    const float xs = EPI == kEpiXSplit ? ti.xs : 1.f;
+    const int lo_plane = (ti.horner || ti.hi_only || g.st_lo == nullptr) ? 0 : 1;
+    const int nplanes = 1 + lo_plane + ((EPI == kEpiGram && p.gram_y) ? 1 : 0);
+    const int st64 = EPI == kEpiXSplit ? 0 : kSt64;
     const uint32_t row_addr = stg + lane * 128 + ((lane & 7) << 4);
-    float s_tq = 0.f;  // share of tr(Q^T Delta) (ti.trace)
+    float s_tq = 0.f, s_sq = 0.f;  // shares of tr(Q^T Delta) (ti.trace), of the sum of G^2
 #pragma unroll 1
     for (int c64 = half * (BN / 128); c64 < (half + 1) * (BN / 128); ++c64) {
         const int col0 = ti.n0 + c64 * 64;
         if (col0 >= g.N || row_base >= g.M) break;
-        constexpr int kUnroll = ROLLED ? 1 : 2;
+        constexpr int kUnroll = ROLLED ? 1 : EPI == kEpiGram ? 3 : 2;
 #pragma unroll kUnroll
         for (int pl = 0; pl < nplanes; ++pl) {
+            const int kind = pl == 0 ? 0 : pl == lo_plane ? 1 : 2;
             if (elect_one()) bulk_wait_read0();
             __syncwarp();
-#pragma unroll kUnroll
+            constexpr int kUnrollH = ROLLED ? 1 : 2;
+#pragma unroll kUnrollH
             for (int h = 0; h < 2; ++h) {
                 float v[32];
                 if (have) {
                     uint32_t r[32];
                     tmem_ld32(tacc + (static_cast<uint32_t>(eg * 32) << 16) + c64 * 64 + h * 32, r);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * xs;
+                    for (int j = 0; j < 32; ++j)
+                        v[j] = EPI == kEpiXSplit ? __uint_as_float(r[j]) * xs : __uint_as_float(r[j]);
                 } else {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = 0.f;
                 }
-                const int c0 = col0 + h * 32;
-                if (ti.trace && pl == 0 && row_ok && c0 < g.N) s_tq = trace_share(g, ti, v, row, c0, s_tq);
-                uint32_t w[16];
-                if (pl == 0) {
+                const int c0 = col0 + h * 32, nvalid = g.N - c0;
+                if (row_ok && nvalid > 0) {
+                    if (EPI == kEpiPoly && !ti.horner) add_gram(g, ti, p.in_f16 != 0, row, c0, v);
+                    if (EPI == kEpiXSplit && ti.trace && pl == 0) s_tq = trace_share(g, ti, v, row, c0, s_tq);
+                    if (EPI == kEpiGram && pl == 0) {
+                        // every entry counts twice, and (G - I) = G here
+                        if (nvalid >= 32) {
+                            float ss = 0.f;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) w[j] = round16x2(v[2 * j], v[2 * j + 1], of16);
-                } else {
+                            for (int j = 0; j < 32; ++j) ss = fmaf(v[j], v[j], ss);
+                            s_sq = fmaf(2.f, ss, s_sq);
+                        } else {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        uint32_t hi;
-                        split16x2(v[2 * j], v[2 * j + 1], of16, hi, w[j]);
+                            for (int j = 0; j < 32; ++j)
+                                if (j < nvalid) s_sq = fmaf(2.f * v[j], v[j], s_sq);
+                        }
                     }
                 }
+                uint32_t w[16];
+                plane_words(v, kind, of16, 0.f, ti.yc, false, 0, w);
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     st_shared4(row_addr ^ ((h * 4 + q) << 4), w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
@@ -292,43 +391,45 @@ __device__ __forceinline__ void update_epilogue(const TileFlags& p, const GemmGr
             fence_proxy_async_smem();
             __syncwarp();
             if (elect_one()) {
-                tma_store_3d(pl == 0 ? g.st_hi : g.st_lo, stg, col0, row_base, b);
+                tma_store_3d(kind == 0 ? g.st_hi + st64 : kind == 1 ? g.st_lo + st64 : g.st_y + kStY64, stg, col0,
+                             row_base, b);
                 bulk_commit();
             }
         }
     }
-    if (ti.trace) trace_store(g, ti, s_tq, eg, half, lane, crank);
+    if (EPI == kEpiXSplit && ti.trace) trace_store(g, ti, s_tq, eg, half, lane, crank);
+    if (EPI == kEpiGram) gram_sums_store(g, ti, s_sq, 0.f, s_sq, eg, half, lane, crank);
 }
 
 // Epilogue of one tile's column half, run by four warps (thread (eg, lane) owns
 // output row m0 + 32 eg + lane).  `tacc` is the tensor-memory accumulator of the tile.
-// 16-bit outputs leave through the warp's shared-memory staging blocks `stg` and TMA
-// stores, one 32 x 32 block at a time.  In symmetric mode (Gram, G^2) blocks below the
-// diagonal are skipped, a block above it is also stored transposed at (col, row), and the
-// diagonal block is made symmetric in shared memory (its upper half mirrored) before its
-// single store, so every entry is written once and the matrix is bitwise symmetric.
+// Of a symmetric 16-bit output (Gram, polynomial) only the tiles on and above the diagonal are
+// stored.  A diagonal tile goes one 32 x 32 block at a time: blocks below the diagonal are
+// skipped, a block above it is also stored transposed, and the diagonal block is made
+// symmetric in shared memory (its upper half mirrored) before its single store, so every
+// entry is written once and the matrix is bitwise symmetric.
 template <int EPI, bool ROLLED>
-__device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGroup& g, const TileInfo& ti, uint32_t tacc, bool ok,
-                                              int eg, int half, int lane, uint32_t crank, uint32_t stg,
-                                              uint32_t& sseq) {
-    if (EPI == kEpiXSplit) {
-        update_epilogue<ROLLED>(p, g, ti, tacc, ok, eg, half, lane, crank, stg);
+__device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGroup& g, const TileInfo& ti, uint32_t tacc,
+                                              bool ok, int eg, int half, int lane, uint32_t crank, uint32_t stg) {
+    const int b = ti.b, m0 = ti.m0, n0 = ti.n0, split = ti.split;
+    // (the polar loop's tiles, ROLLED, are never split over K, and symmetric here)
+    const bool f32_out = (EPI == kEpiF32) || (!ROLLED && EPI == kEpiGram && g.splits > 1);
+    if (EPI == kEpiXSplit || (!f32_out && n0 != (m0 & ~(kTileM - 1)))) {
+        wide_epilogue<EPI, ROLLED>(p, g, ti, tacc, ok, eg, half, lane, crank, stg);
         return;
     }
-    const int b = ti.b, m0 = ti.m0, n0 = ti.n0, split = ti.split;
-    const float ca = ti.ca, cb = ti.cb, cc = ti.cc;
     const int row_base = m0 + eg * 32;
     const int row = row_base + lane;
     const bool row_ok = row < g.M;
-    const bool sym = g.sym != 0;
-    const bool f32_out = (EPI == kEpiF32) || (EPI == kEpiGram && g.splits > 1);
-    const bool gram_fused = (EPI == kEpiGram && g.splits == 1);
+    const bool sym = ROLLED || g.sym != 0;
+    const bool gram_fused = EPI == kEpiGram && !f32_out;
     const bool of16 = p.out_f16 != 0;
     // planes written: hi, lo (if kept; not for a Horner-form P, whose lo plane nobody reads),
     // and for the Gram with p.gram_y the plane Y = yb I + yc G (hi only)
     const int lo_plane = (ti.horner || ti.hi_only || g.st_lo == nullptr) ? 0 : 1;
     const int nplanes = 1 + lo_plane + ((EPI == kEpiGram && p.gram_y) ? 1 : 0);
     float s_sq = 0.f, s_tr = 0.f, s_dev = 0.f;
+#pragma unroll 1
     for (int c32 = half * (BN / 64); c32 < (half + 1) * (BN / 64); ++c32) {
         const int col0 = n0 + c32 * 32;
         if (col0 >= g.N || row_base >= g.M) break;
@@ -347,37 +448,9 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
         }
         const int nvalid = min(32, g.N - col0);
         const int d = row - col0;  // column index of this lane's diagonal entry in the block
-        if (ti.horner) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (j == d) v[j] += ca;
-        } else if (EPI == kEpiPoly && row_ok) {
-            // (past L1: within the polar loop other SMs rewrite G in every iteration)
-            const int64_t goff = b * g.bf_batch_stride + static_cast<int64_t>(row) * g.ld_bf + col0;
-            const uint16_t* gh = reinterpret_cast<const uint16_t*>(g.g_hi) + goff;
-            const uint16_t* gl = reinterpret_cast<const uint16_t*>(g.g_lo) + goff;
-            const bool gf16 = p.in_f16 != 0;
-            if (nvalid == 32) {
-                const uint4* h4 = reinterpret_cast<const uint4*>(gh);
-                const uint4* l4 = reinterpret_cast<const uint4*>(gl);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint4 hh = __ldcg(h4 + q), ll = __ldcg(l4 + q);
-                    const uint32_t hw[4] = {hh.x, hh.y, hh.z, hh.w};
-                    const uint32_t lw[4] = {ll.x, ll.y, ll.z, ll.w};
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        const float g0 = dec16(hw[w] & 0xFFFFu, gf16) + dec16(lw[w] & 0xFFFFu, gf16);
-                        const float g1 = dec16(hw[w] >> 16, gf16) + dec16(lw[w] >> 16, gf16);
-                        v[8 * q + 2 * w] = cc * v[8 * q + 2 * w] + cb * g0;
-                        v[8 * q + 2 * w + 1] = cc * v[8 * q + 2 * w + 1] + cb * g1;
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (j < nvalid) v[j] = cc * v[j] + cb * (dec16(__ldcg(gh + j), gf16) + dec16(__ldcg(gl + j), gf16));
-            }
+        if (EPI == kEpiPoly) {
+            if (!ti.horner && row_ok) add_gram(g, ti, p.in_f16 != 0, row, col0, v);
+            const float ca = ti.ca;
 #pragma unroll
             for (int j = 0; j < 32; ++j)
                 if (j == d) v[j] += ca;
@@ -428,52 +501,13 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
         constexpr int kUnroll = ROLLED ? 1 : 3;
 #pragma unroll kUnroll
         for (int pl = 0; pl < nplanes; ++pl) {
+            const int kind = pl == 0 ? 0 : pl == lo_plane ? 1 : 2;
             uint32_t w[16];
-            const CUtensorMap* map = g.st_hi;
-            if (pl == 0) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) w[j] = round16x2(v[2 * j], v[2 * j + 1], of16);
-            } else if (pl == lo_plane) {
-                map = g.st_lo;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    uint32_t hi;
-                    split16x2(v[2 * j], v[2 * j + 1], of16, hi, w[j]);
-                }
-            } else {
-                // Y = yb I + yc G, hi plane only (it is the single operand of G Y)
-                map = g.st_y;
-                const float yb = ti.yb, yc = ti.yc;
-                if (diag) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        w[j] = round16x2(yc * v[2 * j] + (2 * j == d ? yb : 0.f),
-                                         yc * v[2 * j + 1] + (2 * j + 1 == d ? yb : 0.f), of16);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) w[j] = round16x2(yc * v[2 * j], yc * v[2 * j + 1], of16);
-                }
-            }
-            stage_store_block(w, map, stg, sseq, diag, sym, lane, col0, row_base, b);
+            plane_words(v, kind, of16, ti.yb, ti.yc, diag, d, w);
+            stage_store_block(w, kind == 0 ? g.st_hi : kind == 1 ? g.st_lo : g.st_y, stg, diag, lane, col0, row_base, b);
         }
     }
-    if (gram_fused) {
-        // fixed-order warp reduction; each epilogue warp owns one of the tile's kEpiWarps slots
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s_sq += __shfl_xor_sync(0xffffffffu, s_sq, o);
-            s_tr += __shfl_xor_sync(0xffffffffu, s_tr, o);
-            s_dev += __shfl_xor_sync(0xffffffffu, s_dev, o);
-        }
-        if (lane == 0) {
-            const int ntiles = sym ? g.tiles_sym : g.tiles_m * g.tiles_n;
-            float* slot = g.part + ((g.part_base + static_cast<int64_t>(b) * ntiles + ti.tile) * kPartSlots +
-                                    static_cast<int>(crank) * kEpiWarps + half * 4 + eg) * 3;
-            slot[0] = s_sq;
-            slot[1] = s_tr;
-            slot[2] = s_dev;
-        }
-    }
+    if (gram_fused) gram_sums_store(g, ti, s_sq, s_tr, s_dev, eg, half, lane, crank);
 }
 
 // Position in the shared-memory ring; one pass around it flips the phase.
@@ -482,23 +516,24 @@ struct RingPos {
     uint32_t phase;
 };
 
-// Loads one tile's k-blocks into the ring (one thread of each CTA of the pair): this CTA's
-// rows of A and its half of B's rows, AMN / BMN their layouts.  The bytes of both CTAs
-// complete on rank 0's `full` barriers (shared::cluster address fbar0 of the first).  The
-// wait for the next stage is tested while this stage's loads are issued.  False on a timeout.
+// Loads k-blocks [from, to) of a tile into the ring (one thread of each CTA of the pair): this
+// CTA's rows of A and its half of B's rows, AMN / BMN their layouts, a and b their hi planes'
+// maps (the lo planes' follow them).  The bytes of both CTAs complete on rank 0's `full`
+// barriers (shared::cluster address fbar0 of the first).  The wait for the next stage is tested
+// while this stage's loads are issued.  False on a timeout.
 template <bool AMN, bool BMN>
-__device__ __forceinline__ bool load_tile(const GemmGroup& g, const TileInfo& ti, uint32_t sbase, uint32_t stride,
-                                          int nstages, uint64_t* full, uint64_t* empty, uint32_t fbar0,
-                                          uint32_t crank, RingPos& pos) {
-    const CUtensorMap *a_hi = g.a_hi, *a_lo = g.a_lo, *b_hi = g.b_hi, *b_lo = g.b_lo;
+__device__ __forceinline__ bool load_run(const CUtensorMap* a_hi, const CUtensorMap* b_hi, const TileInfo& ti, int from,
+                                         int to, uint32_t sbase, uint32_t stride, int nstages, uint64_t* full,
+                                         uint64_t* empty, uint32_t fbar0, uint32_t crank, RingPos& pos) {
+    const CUtensorMap *a_lo = a_hi + 1, *b_lo = b_hi + 1;
     const bool as = ti.a_split, bs = ti.b_split;
     const uint32_t off_b = kTileABytes * (as ? 2u : 1u);
     const uint32_t pair_bytes = 2u * (off_b + kTileBBytes * (bs ? 2u : 1u));
     const int m0 = ti.m0, nb0 = ti.n0 + static_cast<int>(crank) * kBRows, b = ti.b;
-    const int k_end = ti.kb_end * BK;
+    const int k_end = to * BK;
     bool ready = mbar_test(&empty[pos.stage], pos.phase ^ 1u);
 #pragma unroll 1
-    for (int k0 = ti.kb_begin * BK; k0 < k_end; k0 += BK) {
+    for (int k0 = from * BK; k0 < k_end; k0 += BK) {
         const int s = pos.stage;
         if (!ready && !mbar_wait(&empty[s], pos.phase ^ 1u)) return false;
         if (++pos.stage == nstages) {
@@ -533,7 +568,26 @@ __device__ __forceinline__ bool load_tile(const GemmGroup& g, const TileInfo& ti
     return true;
 }
 
-// Issues one tile's MMAs (one thread of rank 0) over nkb k-blocks of the ring: the passes
+// The maps of a run's operands (at / bt: read from the transposed tiles).
+__device__ __forceinline__ const CUtensorMap* map_a(const GemmGroup& g, bool at) { return g.a_hi + (at ? g.a_tri : 0); }
+__device__ __forceinline__ const CUtensorMap* map_b(const GemmGroup& g, bool bt) { return g.b_hi + (bt ? g.b_tri : 0); }
+
+// All of a tile's k-blocks.
+__device__ __forceinline__ bool load_tile(const GemmGroup& g, const TileInfo& ti, uint32_t sbase, uint32_t stride,
+                                          int nstages, uint64_t* full, uint64_t* empty, uint32_t fbar0, uint32_t crank,
+                                          RingPos& pos) {
+    return for_k_runs(ti, [&](int from, int to, bool at, bool bt) {
+        const CUtensorMap *a = map_a(g, at), *b = map_b(g, bt);
+        if (g.a_mn || at)
+            return g.b_mn || bt ? load_run<true, true>(a, b, ti, from, to, sbase, stride, nstages, full, empty, fbar0, crank, pos)
+                                : load_run<true, false>(a, b, ti, from, to, sbase, stride, nstages, full, empty, fbar0, crank, pos);
+        return g.b_mn || bt ? load_run<false, true>(a, b, ti, from, to, sbase, stride, nstages, full, empty, fbar0, crank, pos)
+                            : load_run<false, false>(a, b, ti, from, to, sbase, stride, nstages, full, empty, fbar0, crank, pos);
+    });
+}
+
+// Issues MMAs of a tile (one thread of rank 0) over nkb k-blocks of the ring, in one layout (acc 0
+// before the tile's first): the passes
 // hi hi (+ hi lo_B) (+ lo_A hi) of each 16-deep slice, accumulated in tensor memory at tacc.
 // a_lo, b_lo: low descriptor words of the hi planes in stage 0.  A stage or slice only moves
 // the start address (a 14-bit field; every shared address is below 256 KB, so the sum never
@@ -549,10 +603,9 @@ template <bool AS, bool BS>
 __device__ __forceinline__ bool issue_tile(uint64_t* full, uint64_t* empty, int nstages, uint32_t stride16, int nkb,
                                            uint32_t tacc, uint32_t idesc, uint32_t a_lo, uint32_t a_hi,
                                            uint32_t b_lo, uint32_t b_hi, uint32_t step_a, uint32_t step_b,
-                                           RingPos& pos) {
+                                           RingPos& pos, uint32_t& acc) {
     constexpr uint32_t kA16 = kTileABytes >> 4, kB16 = kTileBBytes >> 4;  // hi -> lo plane
     uint32_t so = pos.stage * stride16;
-    uint32_t acc = 0u;
     bool ready = mbar_test(&full[pos.stage], pos.phase);
 #pragma unroll 1
     for (int kb = 0; kb < nkb; ++kb) {

@@ -50,7 +50,9 @@ __global__ void __launch_bounds__(256) k_gs_init(const MatDesc* __restrict__ mat
         split16x2(a, 0.f, true, hw, lw);
         reinterpret_cast<uint16_t*>(anhi)[md.gsslot + o] = static_cast<uint16_t>(hw & 0xFFFFu);
         reinterpret_cast<uint16_t*>(anlo)[md.gsslot + o] = static_cast<uint16_t>(lw & 0xFFFFu);
-        const float z = __bfloat162float(phi[md.gslot + o]) + __bfloat162float(plo[md.gslot + o]);
+        // P's tiles below the diagonal are not stored: their entries come from the mirrored ones
+        const int64_t po = md.gslot + (r / kTileM > c / BN ? static_cast<int64_t>(c) * ld + r : o);
+        const float z = __bfloat162float(phi[po]) + __bfloat162float(plo[po]);
         split16x2(z, 0.f, true, hw, lw);
         const int64_t zo = md.slot + static_cast<int64_t>(r) * md.ld + c;
         reinterpret_cast<uint16_t*>(zhi)[zo] = static_cast<uint16_t>(hw & 0xFFFFu);

@@ -96,17 +96,19 @@ struct SlotRing {
     uint32_t hist = 0;     // slots of each k-block in flight, oldest in the low 4 bits
 };
 
+// As load_run (gemm_tile.cuh), each plane in its own slot.
 template <bool AMN, bool BMN>
-__device__ __forceinline__ bool loop_load(const GemmGroup& g, const TileInfo& ti, uint32_t sbase, uint64_t* full,
-                                          uint64_t* empty, uint32_t fbar0, uint32_t crank, SlotRing& r) {
-    const CUtensorMap *a_hi = g.a_hi, *a_lo = g.a_lo, *b_hi = g.b_hi, *b_lo = g.b_lo;
+__device__ __forceinline__ bool loop_load(const CUtensorMap* a_hi, const CUtensorMap* b_hi, const TileInfo& ti, int from,
+                                          int to, uint32_t sbase, uint64_t* full, uint64_t* empty, uint32_t fbar0,
+                                          uint32_t crank, SlotRing& r) {
+    const CUtensorMap *a_lo = a_hi + 1, *b_lo = b_hi + 1;
     const bool as = ti.a_split, bs = ti.b_split;
     const int need = 2 + (as ? 1 : 0) + (bs ? 1 : 0);
     const uint32_t pair_bytes = 2u * kSlotBytes * need;
     const int m0 = ti.m0, nb0 = ti.n0 + static_cast<int>(crank) * kBRows, b = ti.b;
-    const int k_end = ti.kb_end * BK;
+    const int k_end = to * BK;
 #pragma unroll 1
-    for (int k0 = ti.kb_begin * BK; k0 < k_end; k0 += BK) {
+    for (int k0 = from * BK; k0 < k_end; k0 += BK) {
         while (r.free_slots < need || r.inflight == kKb) {
             if (!mbar_wait(&empty[r.tail], r.tphase)) return false;
             r.free_slots += r.hist & 15u;
@@ -166,9 +168,8 @@ struct SlotPos {
 template <bool AS, bool BS>
 __device__ __forceinline__ bool loop_issue(uint64_t* full, uint64_t* empty, int nkb, uint32_t tacc, uint32_t idesc,
                                            uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                           uint32_t step_a, uint32_t step_b, SlotPos& pos) {
+                                           uint32_t step_a, uint32_t step_b, SlotPos& pos, uint32_t& acc) {
     constexpr uint32_t kSlot16 = kSlotBytes >> 4;
-    uint32_t acc = 0u;
     bool ready = mbar_test(&full[pos.kb], pos.phase);
 #pragma unroll 1
     for (int i = 0; i < nkb; ++i) {
@@ -299,12 +300,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                     }
                     if (good && ti.run_mma) {
                         const GemmGroup& g = p.groups[lt.group].g;
-                        if (g.a_mn)
-                            good = g.b_mn ? loop_load<true, true>(g, ti, sbase, full, empty, fbar0, crank, ring)
-                                          : loop_load<true, false>(g, ti, sbase, full, empty, fbar0, crank, ring);
-                        else
-                            good = g.b_mn ? loop_load<false, true>(g, ti, sbase, full, empty, fbar0, crank, ring)
-                                          : loop_load<false, false>(g, ti, sbase, full, empty, fbar0, crank, ring);
+                        good = for_k_runs(ti, [&](int from, int to, bool at, bool bt) {
+                            const CUtensorMap *a = map_a(g, at), *b = map_b(g, bt);
+                            if (g.a_mn || at)
+                                return g.b_mn || bt ? loop_load<true, true>(a, b, ti, from, to, sbase, full, empty, fbar0, crank, ring)
+                                                    : loop_load<true, false>(a, b, ti, from, to, sbase, full, empty, fbar0, crank, ring);
+                            return g.b_mn || bt ? loop_load<false, true>(a, b, ti, from, to, sbase, full, empty, fbar0, crank, ring)
+                                                : loop_load<false, false>(a, b, ti, from, to, sbase, full, empty, fbar0, crank, ring);
+                        });
                     }
                     if (!good) {
                         *abort_flag = 1;
@@ -528,9 +531,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                 }
                 const LoopTile& lt = tq[q];
                 const int kind = lt.kind;
-                const bool run = kind >= 0 && lt.ti.run_mma, as = lt.ti.a_split, bs = lt.ti.b_split;
-                const int nkb = lt.ti.kb_end - lt.ti.kb_begin, f16 = lt.f.in_f16;
-                const int grp = lt.group;
+                const TileInfo ti = lt.ti;
+                const int f16 = lt.f.in_f16, grp = lt.group;
                 mbar_arrive(&tq_empty[q]);
                 if (++q == kLoopQueue) {
                     q = 0;
@@ -546,21 +548,24 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                     break;
                 }
                 tc_fence_after();
-                if (run) {
-                    const bool a_mn = p.groups[grp].g.a_mn != 0, b_mn = p.groups[grp].g.b_mn != 0;
+                if (ti.run_mma) {
+                    const bool as = ti.a_split, bs = ti.b_split;
                     const uint32_t tacc = tmem_base + buf * kTmemCols;
-                    const uint32_t idesc = make_idesc_16bit(kTileM, BN, a_mn, b_mn, f16 != 0);
-                    const uint64_t da = operand_desc(sbase, a_mn), db = operand_desc(sbase, b_mn);
-                    const uint32_t a_lo = static_cast<uint32_t>(da), a_hi = static_cast<uint32_t>(da >> 32);
-                    const uint32_t b_lo = static_cast<uint32_t>(db), b_hi = static_cast<uint32_t>(db >> 32);
-                    const uint32_t sa = slice_step(a_mn), sb = slice_step(b_mn);
-                    bool ok;
-                    if (as)
-                        ok = bs ? loop_issue<true, true>(full, empty, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos)
-                                : loop_issue<true, false>(full, empty, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos);
-                    else
-                        ok = bs ? loop_issue<false, true>(full, empty, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos)
-                                : loop_issue<false, false>(full, empty, nkb, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos);
+                    uint32_t acc = 0u;
+                    const bool ok = for_k_runs(ti, [&](int from, int to, bool at, bool bt) {
+                        const bool a_mn = p.groups[grp].g.a_mn || at, b_mn = p.groups[grp].g.b_mn || bt;
+                        const uint32_t idesc = make_idesc_16bit(kTileM, BN, a_mn, b_mn, f16 != 0);
+                        const uint64_t da = operand_desc(sbase, a_mn), db = operand_desc(sbase, b_mn);
+                        const uint32_t a_lo = static_cast<uint32_t>(da), a_hi = static_cast<uint32_t>(da >> 32);
+                        const uint32_t b_lo = static_cast<uint32_t>(db), b_hi = static_cast<uint32_t>(db >> 32);
+                        const uint32_t sa = slice_step(a_mn), sb = slice_step(b_mn);
+                        const int n = to - from;
+                        if (as)
+                            return bs ? loop_issue<true, true>(full, empty, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc)
+                                      : loop_issue<true, false>(full, empty, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc);
+                        return bs ? loop_issue<false, true>(full, empty, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc)
+                                  : loop_issue<false, false>(full, empty, n, tacc, idesc, a_lo, a_hi, b_lo, b_hi, sa, sb, pos, acc);
+                    });
                     if (!ok) {
                         *abort_flag = 1;
                         atomicOr(p.err, kErrTimeout);
@@ -578,7 +583,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
         const int eg = warp & 3;
         const int half = (warp - 2) >> 2;
         const uint32_t stg = smem_u32(staging) + (warp - 2) * kStageBlocks * kStageBlockBytes;
-        uint32_t n = 0, sseq = 0;
+        uint32_t n = 0;
         int q = 0;
         uint32_t qphase = 0;
         for (;;) {
@@ -612,11 +617,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
             tc_fence_after();
             const uint32_t tacc = tmem_base + buf * kTmemCols;
             if (kind == kLoopPoly)
-                tile_epilogue<kEpiPoly, true>(f, g, ti, tacc, ok, eg, half, lane, crank, stg, sseq);
+                tile_epilogue<kEpiPoly, true>(f, g, ti, tacc, ok, eg, half, lane, crank, stg);
             else if (kind == kLoopGram || kind == kLoopGramGs)
-                tile_epilogue<kEpiGram, true>(f, g, ti, tacc, ok, eg, half, lane, crank, stg, sseq);
+                tile_epilogue<kEpiGram, true>(f, g, ti, tacc, ok, eg, half, lane, crank, stg);
             else
-                tile_epilogue<kEpiXSplit, true>(f, g, ti, tacc, ok, eg, half, lane, crank, stg, sseq);
+                tile_epilogue<kEpiXSplit, true>(f, g, ti, tacc, ok, eg, half, lane, crank, stg);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) {

@@ -78,15 +78,16 @@ __host__ __device__ constexpr int sym_first_tile_n(int tm) {
     return (tm * kTileM - BN + 1) <= 0 ? 0 : (tm * kTileM - BN + 1 + BN - 1) / BN;
 }
 
+constexpr int kSt64 = 2, kStY64 = 1;  // see GemmGroup::st_hi
+
 struct GemmGroup {
-    const CUtensorMap* a_hi;
-    const CUtensorMap* a_lo;
+    const CUtensorMap* a_hi;  // the lo plane's map follows
     const CUtensorMap* b_hi;
-    const CUtensorMap* b_lo;
     int M, N, K;  // output tile space M x N, reduction length K
     int batch;    // matrices in this group
     int tiles_m, tiles_n, splits, kblocks_per_split;
-    int sym;        // square symmetric output: compute only tiles touching col >= row
+    int sym;        // square symmetric output: compute and store only tiles touching col >= row
+                    // (fp32 outputs: mirrored as well)
     int tiles_sym;  // number of such tiles per matrix
     int cta_begin;  // (host bookkeeping) first tile of the group when every matrix is active
     int mat_base;   // index of the group's first matrix in the state array
@@ -94,6 +95,10 @@ struct GemmGroup {
     int gate_fb;    // 0: no condition; f > 0: only matrices whose Q is in buffer f - 1 (final_buf)
     int a_mn, b_mn; // operand layout: 1 MN-major (M or N index contiguous), 0 K-major
     int a_split, b_split;  // operand carries a lo plane in this group (one tensor pass each)
+    // 0, or the operand is a symmetric n x n matrix of which only the tiles on and above the
+    // diagonal are stored (G, Y, P): its k-blocks left of its diagonal tile are read from the
+    // transposed tiles, MN-major, through the map a_tri (b_tri) further in the bucket's maps
+    int a_tri, b_tri;
     // quintic steps whose index k lies in [one_from, one_to) run a single pass (no lo planes);
     // k = the matrix's step count for a Gram (the step it leads to), the step count - 1 for
     // the polynomial and the update (the step they form)
@@ -104,7 +109,8 @@ struct GemmGroup {
     int ld_f32;
     // 16-bit hi/lo output planes (kEpiGram, kEpiPoly, kEpiXSplit) and their TMA store maps
     // (kEpiXSplit: boxes of 64 columns x 32 rows, 128-byte swizzle; else 32 x 32, 64-byte
-    // swizzle); out_lo/st_lo may be null when no lo plane is kept
+    // swizzle, and the 64 x 32 one kSt64 or, for Y, kStY64 further in the bucket's maps);
+    // out_lo/st_lo may be null when no lo plane is kept
     __nv_bfloat16* out_hi;
     __nv_bfloat16* out_lo;
     const CUtensorMap* st_hi;
