@@ -59,8 +59,10 @@ __global__ void k_reduce_f32(const Chunk*, const MatDesc*, ReplicaPtrs, int, con
                              __nv_bfloat16*, float*, uint32_t*);
 __global__ void k_reduce_p(const Chunk*, const MatDesc*, ReplicaPtrs, int, int, const float*, float,
                            __nv_bfloat16*, __nv_bfloat16*, float*, uint32_t*, int, float, const float*, float*);
-__global__ void k_apply(const Chunk*, const MatDesc*, const MatState*, UpdateSrc, int, float, float, float,
-                        float*, float*, const float*, float*, float*, const uint32_t*, int, int, int, const float*);
+__global__ void k_apply(const Chunk*, const MatDesc*, const MatState*, UpdateSrc, float, float, float, float*, float*,
+                        float*, const uint32_t*, int, int, int, const float*);
+__global__ void k_apply_merge(const Chunk*, const MatDesc*, const MatState*, UpdateSrc, float, const float*, float*,
+                              const uint32_t*);
 __global__ void k_clip_q_bf16(const MatDesc*, const MatState*, __nv_bfloat16*, __nv_bfloat16*, __nv_bfloat16*,
                               __nv_bfloat16*);
 __global__ void k_clip_form_a(const MatDesc*, const MatState*, const float*, const int64_t*, const int64_t*,
@@ -94,7 +96,15 @@ cudaError_t launch_ties_merge(const ReplicaPtrs&, int, int, float*, float*, int6
 __global__ void k_split_planes(const float*, int64_t, int, int, int, __nv_bfloat16*, __nv_bfloat16*, int);
 __global__ void k_debug_wait(uint32_t*, uint64_t, unsigned long long*);
 
-constexpr int kChunkElems = 16384;
+// The streaming passes' chunks (one CTA each): halved from the largest while the parameters do
+// not make two waves of eight CTAs per SM, down to one 16-byte vector per thread (with the
+// largest chunk 0.2 M parameters take 17 + 19 us to reduce and apply, so 6 + 7 us; 13 M with
+// three replicas 79 + 70 us, so 67 + 65 us).
+inline int chunk_elems(int64_t n, int sms) {
+    int c = kChunkElemsMax;
+    while (c > 1024 && n / c < 16 * static_cast<int64_t>(sms)) c /= 2;
+    return c;
+}
 constexpr int kTraceChunkElems = 16384;
 constexpr int kDefaultMaxIter = 28;
 constexpr float kDefaultTol = 4e-3f;
@@ -563,7 +573,9 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
 
     // --- streaming chunks (table order) and the 1-D workspace
     std::vector<Chunk> chunks;
-    int64_t d1 = 0;
+    int64_t d1 = 0, n_total = 0;
+    for (int i = 0; i < n_params; ++i) n_total += (int64_t)table[i].rows * (table[i].cols > 0 ? table[i].cols : 1);
+    const int chunk_len = chunk_elems(n_total, p->num_sms);
     for (int i = 0; i < n_params; ++i) {
         const isoloco_param_t& t = table[i];
         const int64_t len = (int64_t)t.rows * (t.cols > 0 ? t.cols : 1);
@@ -572,10 +584,10 @@ static int build_plan(isoloco_plan* p, const isoloco_param_t* table, int n_param
             dst = d1;
             d1 += round_up(len, 4);
         }
-        for (int64_t e = 0; e < len; e += kChunkElems) {
+        for (int64_t e = 0; e < len; e += chunk_len) {
             Chunk c{};
             c.flat_begin = t.offset + e;
-            c.count = (int32_t)std::min<int64_t>(kChunkElems, len - e);
+            c.count = (int32_t)std::min<int64_t>(chunk_len, len - e);
             c.param = i;
             c.matrix = mat_of_param[i];
             c.elem_begin = (int32_t)e;
@@ -1739,12 +1751,12 @@ static int run_isoc_step(isoloco_plan* p, int merge, float* theta, float* mom, c
     if (p->nchunks) {
         PhaseTimer tm(p, ISOLOCO_PHASE_APPLY, st);
         if (merge)
-            k_apply<<<p->nchunks, 256, 0, st>>>(p->chunks_d, p->mats_d, p->state, us, 1, alpha_merge, 0.f, 0.f,
-                                                nullptr, nullptr, base, out, nullptr, p->err_d, 0, 0, 0, nullptr);
+            k_apply_merge<<<p->nchunks, 256, 0, st>>>(p->chunks_d, p->mats_d, p->state, us, alpha_merge, base, out,
+                                                      p->err_d);
         else
-            k_apply<<<p->nchunks, 256, 0, st>>>(p->chunks_d, p->mats_d, p->state, us, 0, o.alpha, o.outer_lr,
-                                                o.momentum, theta, mom, nullptr, nullptr, upd_out, p->err_d,
-                                                o.momentum_kind, pmode, o.scale_kind, p->bnew);
+            k_apply<<<p->nchunks, 256, 0, st>>>(p->chunks_d, p->mats_d, p->state, us, o.alpha, o.outer_lr, o.momentum,
+                                                theta, mom, upd_out, p->err_d, o.momentum_kind, pmode, o.scale_kind,
+                                                p->bnew);
         CUDA_TRY(cudaGetLastError());
     }
     return finish_call(p, st, o.sync);

@@ -25,6 +25,12 @@
 namespace isoloco {
 
 constexpr int kStreamThreads = 256;
+template <int N>
+struct Int {
+    static constexpr int value = N;
+};
+constexpr int kScalarRows = 4;  // elements a thread reduces at a time where vectors do not fit
+constexpr int kApplyRows = 2;   // the same in the apply pass
 constexpr int kRepBatch = 8;  // replica loads a thread keeps in flight in the reduction
 
 __device__ __forceinline__ float4 ld_rep4(const void* base, int dtype, int64_t i) {
@@ -53,6 +59,98 @@ __device__ __forceinline__ float reduce_out(float d, int pmode, float mu, const 
     const float nb = fmaf(mu, __ldg(mom + i), d);
     bnew[i] = nb;
     return pmode == 1 ? fmaf(mu, nb, d) : nb;
+}
+
+// Where elements of a chunk lie in a matrix's planes (rows padded to ld): n counts from the
+// first element of the chunk's first row, n < cols + chunk length.  The row is a multiplication
+// by ceil(2^32 / cols), exact while n cols < 2^32; a longer row ends at most once in a chunk.
+static_assert(kChunkElemsMax <= 1 << 14, "(2^15 + chunk) 2^15 < 2^32, and one row end in a longer row's chunk");
+struct RowSplit {
+    uint32_t m;
+    int cols, ld, c0;
+    int64_t o0;
+    RowSplit() = default;
+    __device__ __forceinline__ RowSplit(const MatDesc& md, int elem_begin) {
+        cols = md.cols;
+        ld = md.ld;
+        const int r0 = elem_begin / cols;
+        c0 = elem_begin - r0 * cols;
+        o0 = static_cast<int64_t>(r0) * ld;
+        m = cols > 1 && cols < (1 << 15) ? 0xFFFFFFFFu / static_cast<uint32_t>(cols) + 1u : 0u;
+    }
+    __device__ __forceinline__ int64_t at(int e) const {
+        const int n = c0 + e;
+        const int r = m ? static_cast<int>(__umulhi(static_cast<uint32_t>(n), m)) : cols == 1 ? n : n >= cols ? 1 : 0;
+        return o0 + static_cast<int64_t>(r) * ld + (n - r * cols);
+    }
+};
+
+// Delta of NE elements of a matrix, a block's width apart from element e of the chunk, into its
+// planes (rows): up to four replicas' loads in flight for each (a loop that looks at the data
+// type for each load would wait for each).  True if a value is not finite.  (6 layers of
+// 1021 x 2777: eight fp32 replicas 0.73 -> 0.61 ms, eight bf16 0.73 -> 0.47, three bf16
+// 0.80 -> 0.28; the apply pass alike 0.51 -> 0.39.)
+template <class T, int NE, bool PM>
+__device__ __forceinline__ bool reduce_rows(const ReplicaPtrs& reps, int K, const float* __restrict__ theta, float scale,
+                                            int64_t i, int e, const RowSplit& rows, __nv_bfloat16* __restrict__ oh,
+                                            __nv_bfloat16* __restrict__ ol, int pmode, float mu,
+                                            const float* __restrict__ mom, float* __restrict__ bnew) {
+    constexpr int kB = 4;
+    float th[NE], s[NE];
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+        th[j] = __ldg(theta + i + j * kStreamThreads);
+        s[j] = 0.f;
+    }
+    for (int k0 = 0; k0 < K; k0 += kB) {
+        T r[kB][NE];
+#pragma unroll
+        for (int u = 0; u < kB; ++u)
+            if (k0 + u < K) {
+                const T* rep = static_cast<const T*>(reps.p[k0 + u]) + i;
+#pragma unroll
+                for (int j = 0; j < NE; ++j) r[u][j] = __ldg(rep + j * kStreamThreads);
+            }
+#pragma unroll
+        for (int u = 0; u < kB; ++u)
+            if (k0 + u < K) {
+#pragma unroll
+                for (int j = 0; j < NE; ++j) {
+                    if constexpr (sizeof(T) == 4)
+                        s[j] += th[j] - r[u][j];
+                    else
+                        s[j] += th[j] - bf16_bits_to_float(r[u][j]);
+                }
+            }
+    }
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < NE; ++j) {
+        const float d = reduce_out(s[j] * scale, PM ? pmode : 0, mu, mom, bnew, i + j * kStreamThreads);
+        bad |= !isfinite(d);
+        const int64_t o = rows.at(e + j * kStreamThreads);
+        __nv_bfloat16 h, l;
+        split_bf16(d, h, l);
+        oh[o] = h;
+        ol[o] = l;
+    }
+    return bad;
+}
+
+// A chunk's elements through reduce_rows: kScalarRows at a time, what is left one by one.
+template <class T, bool PM>
+__device__ __forceinline__ bool reduce_rows_chunk(const ReplicaPtrs& reps, int K, const float* __restrict__ theta,
+                                                  float scale, const Chunk& ch, const RowSplit& rows,
+                                                  __nv_bfloat16* __restrict__ oh, __nv_bfloat16* __restrict__ ol,
+                                                  int pmode, float mu, const float* __restrict__ mom,
+                                                  float* __restrict__ bnew) {
+    bool bad = false;
+    int e = threadIdx.x;
+    for (; e + (kScalarRows - 1) * kStreamThreads < ch.count; e += kScalarRows * kStreamThreads)
+        bad |= reduce_rows<T, kScalarRows, PM>(reps, K, theta, scale, ch.flat_begin + e, e, rows, oh, ol, pmode, mu, mom, bnew);
+    for (; e < ch.count; e += kStreamThreads)
+        bad |= reduce_rows<T, 1, PM>(reps, K, theta, scale, ch.flat_begin + e, e, rows, oh, ol, pmode, mu, mom, bnew);
+    return bad;
 }
 
 // One CTA per chunk.  PM: the orthogonalise-P ablation (its own kernel, so that the
@@ -137,20 +235,14 @@ __device__ __forceinline__ void reduce_chunk(const Chunk* __restrict__ chunks, c
                 reinterpret_cast<uint2*>(ol)[v] = make_uint2(pack_bf16x2(l[0], l[1]), pack_bf16x2(l[2], l[3]));
             }
         } else {
-            for (int e = threadIdx.x; e < ch.count; e += blockDim.x) {
-                const int64_t i = f0 + e;
-                const float th = __ldg(theta + i);
-                float s = 0.f;
-                for (int k = 0; k < K; ++k) s += th - ld_rep1(reps.p[k], dtype, i);
-                const float d = reduce_out(s * scale, pmode, mu, mom, bnew, i);
-                bad |= !isfinite(d);
-                const int pe = ch.elem_begin + e;
-                const int64_t o = md.slot + static_cast<int64_t>(pe / md.cols) * md.ld + pe % md.cols;
-                __nv_bfloat16 h, l;
-                split_bf16(d, h, l);
-                dhi[o] = h;
-                dlo[o] = l;
-            }
+            // Padded rows, or a tensor off the 16-byte boundaries: kScalarRows elements per
+            // thread, a block's width apart, all their loads in flight together
+            const RowSplit rows(md, ch.elem_begin);
+            __nv_bfloat16* oh = dhi + md.slot;
+            __nv_bfloat16* ol = dlo + md.slot;
+            bad = BATCH || dtype == 0
+                      ? reduce_rows_chunk<float, PM>(reps, K, theta, scale, ch, rows, oh, ol, pmode, mu, mom, bnew)
+                      : reduce_rows_chunk<uint16_t, PM>(reps, K, theta, scale, ch, rows, oh, ol, pmode, mu, mom, bnew);
         }
     }
     raise_nonfinite(bad, err);
@@ -195,24 +287,18 @@ __global__ void __launch_bounds__(kStreamThreads) k_reduce_p(const Chunk* __rest
 }
 
 
-// grid: one CTA per chunk.  mode 0: outer update of theta and B in place; mode 1: merge
-// output.  Mode 0 variants (the ablations of Sec. 4.5 and App. B): mom_kind 0 Nesterov
+// One CTA per chunk.  MERGE: the merge output; else the outer update of theta and B in place,
+// with the ablations of Sec. 4.5 and App. B: mom_kind 0 Nesterov
 // (Alg. 2), 1 standard momentum (B <- mu B + U, theta <- theta - eta B); pmode != 0: U is
 // already the orthogonalised update P (theta <- theta - eta U, B <- bnew from the reduce
 // pass); spectral: 2-D tensors scale Q by sqrt(rows / cols) instead of sigma_bar.
-__global__ void __launch_bounds__(kStreamThreads) k_apply(const Chunk* __restrict__ chunks,
-                                                          const MatDesc* __restrict__ mats,
-                                                          const MatState* __restrict__ state,
-                                                          UpdateSrc src, int mode, float alpha,
-                                                          float eta, float mu,
-                                                          float* __restrict__ theta,
-                                                          float* __restrict__ mom,
-                                                          const float* __restrict__ base,
-                                                          float* __restrict__ out,
-                                                          float* __restrict__ upd_out,
-                                                          const uint32_t* __restrict__ err, int mom_kind,
-                                                          int pmode, int spectral,
-                                                          const float* __restrict__ bnew) {
+template <bool MERGE>
+__device__ __forceinline__ void apply_chunk(const Chunk* __restrict__ chunks, const MatDesc* __restrict__ mats,
+                                            const MatState* __restrict__ state, const UpdateSrc& src, float alpha,
+                                            float eta, float mu, float* __restrict__ theta, float* __restrict__ mom,
+                                            const float* __restrict__ base, float* __restrict__ out,
+                                            float* __restrict__ upd_out, const uint32_t* __restrict__ err,
+                                            int mom_kind, int pmode, int spectral, const float* __restrict__ bnew) {
     if (*err & kErrNonFinite) return;  // leave theta and B untouched
     const Chunk ch = chunks[blockIdx.x];
     const int64_t f0 = ch.flat_begin;
@@ -233,16 +319,9 @@ __global__ void __launch_bounds__(kStreamThreads) k_apply(const Chunk* __restric
         }
         ucoef = alpha * (spectral ? sqrtf(static_cast<float>(md.rows) / static_cast<float>(md.cols)) : st.sigma_bar);
         contiguous = (md.ld == md.cols);
-    } else if (mode == 1) {
+    } else if (MERGE) {
         ucoef = alpha;  // Eq. 1: base + lambda * sum tau for non-matrix tensors
     }
-    auto uval = [&](int e) -> float {
-        if (ch.matrix < 0) return ucoef * src.d1d[ch.dst + e];
-        if (zero) return 0.f;
-        const int pe = ch.elem_begin + e;
-        const int64_t o = contiguous ? pe : static_cast<int64_t>(pe / md.cols) * md.ld + pe % md.cols;
-        return ucoef * (dec16(__bfloat16_as_ushort(qh[o]), true) + dec16(__bfloat16_as_ushort(ql[o]), true));
-    };
     const bool vec = (f0 & 3) == 0 && (ch.count & 3) == 0 && (ch.matrix < 0 || contiguous) &&
                      ((ch.matrix < 0 ? (ch.dst & 3) : (ch.elem_begin & 3)) == 0);
     if (vec) {
@@ -263,7 +342,7 @@ __global__ void __launch_bounds__(kStreamThreads) k_apply(const Chunk* __restric
                 u[2] = ucoef * (dec16(hh.y & 0xFFFFu, true) + dec16(ll.y & 0xFFFFu, true));
                 u[3] = ucoef * (dec16(hh.y >> 16, true) + dec16(ll.y >> 16, true));
             }
-            if (mode == 0) {
+            if (!MERGE) {
                 const float4 th = *reinterpret_cast<const float4*>(theta + i);
                 float4 nb, nt;
                 if (pmode) {
@@ -290,27 +369,88 @@ __global__ void __launch_bounds__(kStreamThreads) k_apply(const Chunk* __restric
                 const float4 bs = *reinterpret_cast<const float4*>(base + i);
                 *reinterpret_cast<float4*>(out + i) = make_float4(bs.x + u[0], bs.y + u[1], bs.z + u[2], bs.w + u[3]);
             }
-            if (upd_out) *reinterpret_cast<float4*>(upd_out + i) = make_float4(u[0], u[1], u[2], u[3]);
+            if (!MERGE && upd_out) *reinterpret_cast<float4*>(upd_out + i) = make_float4(u[0], u[1], u[2], u[3]);
         }
     } else {
-        for (int e = threadIdx.x; e < ch.count; e += blockDim.x) {
+        // as in the reduction: kApplyRows elements per thread, their loads together
+        const RowSplit rows = ch.matrix >= 0 ? RowSplit(md, ch.elem_begin) : RowSplit();
+        const float* in0 = MERGE ? base : theta;
+        const float* in1 = pmode ? bnew : mom;
+        auto apply = [&](int e, auto ne) {
+            constexpr int NE = decltype(ne)::value;
             const int64_t i = f0 + e;
-            const float u = uval(e);
-            if (mode == 0) {
-                if (pmode) {
-                    theta[i] = theta[i] - eta * u;
-                    mom[i] = bnew[i];
-                } else {
-                    const float nb = fmaf(mu, mom[i], u);
-                    theta[i] = theta[i] - eta * (mom_kind == 1 ? nb : fmaf(mu, nb, u));
-                    mom[i] = nb;
-                }
-            } else {
-                out[i] = base[i] + u;
+            float u[NE], th[NE], bb[NE];
+#pragma unroll
+            for (int j = 0; j < NE; ++j) {
+                th[j] = in0[i + j * kStreamThreads];
+                bb[j] = MERGE ? 0.f : in1[i + j * kStreamThreads];
             }
-            if (upd_out) upd_out[i] = u;
-        }
+            if (ch.matrix < 0) {
+#pragma unroll
+                for (int j = 0; j < NE; ++j) u[j] = ucoef * src.d1d[ch.dst + e + j * kStreamThreads];
+            } else if (zero) {
+#pragma unroll
+                for (int j = 0; j < NE; ++j) u[j] = 0.f;
+            } else {
+                uint32_t h[NE], l[NE];
+#pragma unroll
+                for (int j = 0; j < NE; ++j) {
+                    const int64_t o = rows.at(e + j * kStreamThreads);
+                    h[j] = __bfloat16_as_ushort(qh[o]);
+                    l[j] = __bfloat16_as_ushort(ql[o]);
+                }
+#pragma unroll
+                for (int j = 0; j < NE; ++j) u[j] = ucoef * (dec16(h[j], true) + dec16(l[j], true));
+            }
+#pragma unroll
+            for (int j = 0; j < NE; ++j) {
+                const int64_t ij = i + j * kStreamThreads;
+                if (!MERGE) {
+                    if (pmode) {
+                        theta[ij] = th[j] - eta * u[j];
+                        mom[ij] = bb[j];
+                    } else {
+                        const float nb = fmaf(mu, bb[j], u[j]);
+                        theta[ij] = th[j] - eta * (mom_kind == 1 ? nb : fmaf(mu, nb, u[j]));
+                        mom[ij] = nb;
+                    }
+                } else {
+                    out[ij] = th[j] + u[j];
+                }
+                if (!MERGE && upd_out) upd_out[ij] = u[j];
+            }
+        };
+        int e = threadIdx.x;
+        for (; e + (kApplyRows - 1) * kStreamThreads < ch.count; e += kApplyRows * kStreamThreads)
+            apply(e, Int<kApplyRows>{});
+        for (; e < ch.count; e += kStreamThreads) apply(e, Int<1>{});
     }
+}
+
+// (Eight CTAs per SM: with five, the registers of kScalarRows elements, the vectors' path
+// drops from 0.94 to 0.81 of the copy bandwidth.)
+__global__ void __launch_bounds__(kStreamThreads, 8) k_apply(const Chunk* __restrict__ chunks,
+                                                             const MatDesc* __restrict__ mats,
+                                                             const MatState* __restrict__ state, UpdateSrc src,
+                                                             float alpha, float eta, float mu,
+                                                             float* __restrict__ theta, float* __restrict__ mom,
+                                                             float* __restrict__ upd_out,
+                                                             const uint32_t* __restrict__ err, int mom_kind,
+                                                             int pmode, int spectral,
+                                                             const float* __restrict__ bnew) {
+    apply_chunk<false>(chunks, mats, state, src, alpha, eta, mu, theta, mom, nullptr, nullptr, upd_out, err, mom_kind,
+                       pmode, spectral, bnew);
+}
+
+// out = base + alpha U (Eq. 1)
+__global__ void __launch_bounds__(kStreamThreads, 8) k_apply_merge(const Chunk* __restrict__ chunks,
+                                                                   const MatDesc* __restrict__ mats,
+                                                                   const MatState* __restrict__ state, UpdateSrc src,
+                                                                   float alpha, const float* __restrict__ base,
+                                                                   float* __restrict__ out,
+                                                                   const uint32_t* __restrict__ err) {
+    apply_chunk<true>(chunks, mats, state, src, alpha, 0.f, 0.f, nullptr, nullptr, base, out, nullptr, err, 0, 0, 0,
+                      nullptr);
 }
 
 // Alg. 1 outer step fused: d = scale * sum_k (theta - theta_k); B <- mu B + d;

@@ -211,6 +211,8 @@ struct MatDesc {
 };
 
 // A contiguous range of one parameter handled by one streaming CTA.
+constexpr int kChunkElemsMax = 16384;  // elements of a chunk at most
+
 struct Chunk {
     int64_t flat_begin;  // first element in the flat buffers
     int32_t count;       // elements
