@@ -220,6 +220,17 @@ __device__ __forceinline__ int shfl_i(int v, int src) { return __shfl_sync(0xfff
 
 }  // namespace
 
+// The matrix (of the phase's groups, in their order) at position i of a phase's walk.
+__device__ __forceinline__ int walk_matrix(const LoopPhase& L, int i) {
+    const int side = L.count - L.regular;
+    if (i >= L.side_at) {
+        if (i < L.side_at + side) return L.regular + i - L.side_at;
+        i -= side;
+    }
+    if (i < 2 * L.skip) i += i < L.skip ? L.skip : -L.skip;
+    return L.falling ? L.regular - 1 - i : i;
+}
+
 template <int NG>
 __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_constant__ LoopParams<NG> p) {
     extern __shared__ uint8_t smem_raw[];
@@ -362,10 +373,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                 const int passes = p.prof ? 2 : 1;  // profiling: first wait for the whole last phase
                 for (int pass = 0; ok && pass < passes; ++pass) {
                     const bool only_wait = pass + 1 < passes;
-                    for (int e0 = 0; ok && e0 < count; e0 += 32) {
-                        const bool valid = e0 + lane < count;
+                    int n = 0;  // matrices taken at a time: the next ones already decided, up to 32
+                    // (waiting for 32 at a time idled every cluster 3-7 % of an iteration)
+                    for (int e0 = 0; ok && e0 < count; e0 += n) {
+                        bool valid = e0 + lane < count;
                         // this lane's matrix of the phase
-                        int grp = L.first, b = e0 + lane;
+                        int grp = L.first, b = valid ? walk_matrix(L, e0 + lane) : 0;
                         if (valid)
                             while (b >= p.groups[grp].g.batch) b -= p.groups[grp++].g.batch;
                         const int mat = valid ? p.groups[grp].g.mat_base + b : 0;
@@ -381,7 +394,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                                     w = ld_acquire(&p.ctl[mat]);
                                     have = (w >> 4) >= need || (w & 8u);
                                 }
-                                if (__all_sync(0xffffffffu, have)) break;
+                                const unsigned wait = ~__ballot_sync(0xffffffffu, have);
+                                n = wait ? __ffs(wait) - 1 : 32;
+                                if (n > 0) break;
                                 if ((i & 63u) == 63u) {
                                     if (!t0) t0 = globaltimer_ns();
                                     const bool out = *abort_flag || globaltimer_ns() - t0 > kWaitTimeoutNs ||
@@ -394,6 +409,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                             }
                         }
                         if (!ok) break;
+                        valid = valid && lane < n;
                         // active: its Gram until it is done; its step in the iterations it decided
                         // one for (an undone matrix always steps; the last step is the one it
                         // finished in, unless it stopped without one)

@@ -24,6 +24,10 @@ struct LoopPhase {
     int kind;
     int first, ngroups;  // groups [first, first + ngroups)
     int count;           // their matrices
+    // order in which they come up (walk_matrix in polar_loop.cu): the first `regular` in rising
+    // or falling order, the first `skip` of these after the next `skip`, the others (Gram-side)
+    // at position side_at
+    int regular, side_at, skip, falling;
 };
 
 // Everything the loop reads besides the matrices' states and counters is in its parameters:

@@ -27,6 +27,29 @@ def iso():
     return isoloco
 
 
+def captured_step(plan, iso, wl):
+    """The step with its iterations as single launches."""
+    th, b, upd = wl.theta.clone(), wl.momentum.clone(), torch.empty_like(wl.theta)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan.outer_step(th, b, wl.replicas, iso.make_opts(1.0, 0.7, 0.9), update_out=upd)
+    graph.replay()
+    torch.cuda.synchronize()
+    return th, b, upd
+
+
+@pytest.mark.parametrize("count", [60, 76])  # Gram's tiles about the eight waves from which phases alternate
+def test_walk_in_both_directions(iso, count):
+    """Enough tiles that the phases walk in opposite directions, with Gram-side matrices beside."""
+    shapes = [(f"a{i}", 1000, 1021) for i in range(count)] + [("s0", 4100, 500), ("s1", 4100, 500)]
+    wl = W.make_workload(W.custom_spec(shapes, K=1, rank=2, momentum_std=1e-4), seed=24, device="cuda")
+    plan = iso.Plan(wl.table, wl.N, wl.K)
+    th, b, upd = wl.theta.clone(), wl.momentum.clone(), torch.empty_like(wl.theta)
+    assert plan.outer_step(th, b, wl.replicas, iso.make_opts(1.0, 0.7, 0.9, sync=True), update_out=upd) == 0
+    for got, want in zip((th, b, upd), captured_step(plan, iso, wl)):
+        assert torch.equal(got, want)
+
+
 @pytest.mark.parametrize("name", list(SETS))
 def test_loop_matches_oracle_and_single_launches(iso, name):
     spec = W.custom_spec(SETS[name], K=2, rank=2, momentum_std=1e-4)
@@ -38,10 +61,5 @@ def test_loop_matches_oracle_and_single_launches(iso, name):
     ref["theta_in"] = wl.theta.double().cpu().numpy()
     check_step(wl.table, th.double().cpu().numpy(), b.double().cpu().numpy(), upd.double().cpu().numpy(),
                plan.read_diag()["sigma_bar"], ref)
-    th2, b2, upd2 = wl.theta.clone(), wl.momentum.clone(), torch.empty_like(wl.theta)
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph):
-        plan.outer_step(th2, b2, wl.replicas, iso.make_opts(1.0, 0.7, 0.9), update_out=upd2)
-    graph.replay()
-    torch.cuda.synchronize()
+    th2, b2, upd2 = captured_step(plan, iso, wl)
     assert torch.equal(th, th2) and torch.equal(b, b2) and torch.equal(upd, upd2)
