@@ -344,15 +344,25 @@ __device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGrou
     for (int c64 = half * (BN / 128); c64 < (half + 1) * (BN / 128); ++c64) {
         const int col0 = ti.n0 + c64 * 64;
         if (col0 >= g.N || row_base >= g.M) break;
-        constexpr int kUnroll = ROLLED ? 1 : EPI == kEpiGram ? 3 : 2;
+        // kEpiPoly keeps the lo plane's words: reading G again for it made the first polynomial of
+        // 86 matrices of 1024 take 251 us, so 211
+        uint32_t lo[2][16];
+        constexpr bool kKeepLo = EPI == kEpiPoly;
+        constexpr int kUnroll = ROLLED && !kKeepLo ? 1 : EPI == kEpiGram ? 3 : 2;
 #pragma unroll kUnroll
         for (int pl = 0; pl < nplanes; ++pl) {
             const int kind = pl == 0 ? 0 : pl == lo_plane ? 1 : 2;
             if (elect_one()) bulk_wait_read0();
             __syncwarp();
-            constexpr int kUnrollH = ROLLED ? 1 : 2;
+            constexpr int kUnrollH = ROLLED && !kKeepLo ? 1 : 2;
 #pragma unroll kUnrollH
             for (int h = 0; h < 2; ++h) {
+                if (kKeepLo && pl == 1) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        st_shared4(row_addr ^ ((h * 4 + q) << 4), lo[h][4 * q], lo[h][4 * q + 1], lo[h][4 * q + 2], lo[h][4 * q + 3]);
+                    continue;
+                }
                 float v[32];
                 if (have) {
                     uint32_t r[32];
@@ -384,6 +394,7 @@ __device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGrou
                 }
                 uint32_t w[16];
                 plane_words(v, kind, of16, 0.f, ti.yc, false, 0, w);
+                if (kKeepLo && lo_plane) plane_words(v, 1, of16, 0.f, 0.f, false, 0, lo[h]);
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     st_shared4(row_addr ^ ((h * 4 + q) << 4), w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
