@@ -320,8 +320,16 @@ __device__ __forceinline__ void gram_sums_store(const GemmGroup& g, const TileIn
     }
 }
 
+// First of the blocks of `width` columns that a half of the epilogue's warps takes: the blocks
+// that the tile has, split evenly (one half took all of a tile of up to 128 columns: steps of
+// 64-wide matrices 373 -> 344 us).
+__device__ __forceinline__ int half_begin(const GemmGroup& g, const TileInfo& ti, int half, int width) {
+    const int blocks = (min(BN, g.N - ti.n0) + width - 1) / width;
+    return min(blocks, half * ((blocks + 1) / 2));
+}
+
 // Epilogue of an update tile (kEpiXSplit: X = xs acc) or of a tile above the diagonal of a
-// symmetric output (Gram, polynomial), for one warp's 32 rows and 128 columns.  A plane leaves
+// symmetric output (Gram, polynomial), for one warp's 32 rows and half of the columns.  A plane leaves
 // 64 columns at a time through the warp's whole staging (32 rows of 128 bytes, 128-byte
 // swizzle) and one TMA store: the TMA unit, which also brings the operands, takes a row of up
 // to 128 bytes every ~2 cycles, so 64-byte rows cost it twice.  The accumulator is read again
@@ -341,7 +349,7 @@ __device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGrou
     const uint32_t row_addr = stg + lane * 128 + ((lane & 7) << 4);
     float s_tq = 0.f, s_sq = 0.f;  // shares of tr(Q^T Delta) (ti.trace), of the sum of G^2
 #pragma unroll 1
-    for (int c64 = half * (BN / 128); c64 < (half + 1) * (BN / 128); ++c64) {
+    for (int c64 = half_begin(g, ti, half, 64); c64 < half_begin(g, ti, half + 1, 64); ++c64) {
         const int col0 = ti.n0 + c64 * 64;
         if (col0 >= g.N || row_base >= g.M) break;
         // kEpiPoly keeps the lo plane's words: reading G again for it made the first polynomial of
@@ -441,7 +449,7 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
     const int nplanes = 1 + lo_plane + ((EPI == kEpiGram && p.gram_y) ? 1 : 0);
     float s_sq = 0.f, s_tr = 0.f, s_dev = 0.f;
 #pragma unroll 1
-    for (int c32 = half * (BN / 64); c32 < (half + 1) * (BN / 64); ++c32) {
+    for (int c32 = half_begin(g, ti, half, 32); c32 < half_begin(g, ti, half + 1, 32); ++c32) {
         const int col0 = n0 + c32 * 32;
         if (col0 >= g.N || row_base >= g.M) break;
         if (sym && col0 < row_base) continue;  // block below the diagonal (warp-uniform)

@@ -12,6 +12,8 @@ pytestmark = pytest.mark.gpu
 SETS = {
     "one tile": [("a", 64, 64)],
     "tile edges": [("a", 255, 255), ("b", 256, 256), ("c", 257, 257), ("d", 256, 513), ("e", 513, 256)],
+    "columns split between the epilogue's halves": [("a", 33, 33), ("b", 65, 65), ("c", 97, 97), ("d", 129, 129),
+                                                    ("e", 160, 193), ("f", 290, 64), ("g", 64, 290), ("h", 300, 320)],
     "tiles read transposed": [("a", 513, 514), ("b", 600, 1100), ("c", 1100, 600), ("d", 2600, 300), ("e", 769, 1793)],
     "more matrices than a warp has lanes": [(f"a{i}", 24, 40) for i in range(37)] + [(f"b{i}", 40, 24) for i in range(3)],
     "Gram side beside others": [(f"a{i}", 2048, 16) for i in range(3)] + [("b", 300, 200), ("c", 520, 65)],
