@@ -270,17 +270,6 @@ def stream_bytes(table, K, replica_bytes):
 # tensor-core passes over hi/lo splits of fp32 operands with fp32 accumulation.
 DTYPE_ISO = "f32 streaming; polar GEMMs as bf16/fp16 hi+lo split passes, f32 accumulate"
 
-# DRAM bytes (read + write) of all k_gemm_split launches of one step, from ncu captures of
-# the current kernel, (workload, fast_steps, spectrum_kind) -> figure: the 180M step's four
-# shape buckets captured one at a time with ncu (dram__bytes_read.sum + dram__bytes_write.sum) and summed.
-GEMM_TRAFFIC = {
-    ("llama_180m_k8", 0, 0): {
-        "bytes_per_step": 24.45e9,
-        "note": "dram__bytes_read.sum + dram__bytes_write.sum of every k_gemm_split launch of one step, "
-                "captured per shape bucket (square48, tall12, wide24, embed2) and summed; same unit as "
-                "achieved (per step over all GEMM launches)"},
-}
-
 
 # --------------------------------------------------------------------------- CPU oracle arm
 CPU_SAMPLE = ["layers.0.attn_norm", "layers.0.wq", "layers.0.wk", "layers.0.ffn_norm", "layers.0.w_gate", "layers.0.w_up",
@@ -589,9 +578,9 @@ def main():
     launches = plan.launches - launches0
     diag = plan.read_diag()
 
-    # ---- kernel times: the same K steps again with per-phase CUDA events (the library then
-    # launches the polar iterations one by one, stopping once every matrix is done, since
-    # events cannot sit inside its graph); the timed numbers above are without them
+    # ---- kernel times: the same K steps again with per-phase times (CUDA events between
+    # launches; inside the polar loop's kernel the GPU's timer, each phase waiting for the one
+    # before to end); the timed numbers above are without them
     plan.profile(True)
     for i in range(args.steps):
         restore()
@@ -656,19 +645,19 @@ def main():
         ms, n = prof[phase]
         return nbytes * args.steps / (ms / 1000.0) / 1e9 if ms > 0 else 0.0
 
-    traffic = GEMM_TRAFFIC.get((args.workload, args.fast_steps, spectrum_kind))
-    roofline = {"bound": "tensor", "kernel": "k_gemm_split (Gram, G^2 and update GEMMs)",
+    roofline = {"bound": "tensor", "kernel": "k_gemm_split and k_polar_loop (Gram, polynomial and update GEMMs)",
                 "achieved": achieved_tf, "peak": tc_peak, "unit": "TFLOP/s",
                 "frac": achieved_tf / tc_peak if tc_peak else None,
-                "traffic": traffic["bytes_per_step"] if traffic else None,
-                "traffic_note": traffic["note"] if traffic else "no DRAM capture of the current kernel",
+                "traffic": None,
+                "traffic_note": "no DRAM capture: ncu reports no counters for the polar loop's kernel",
                 "peak_source": f"{peak_src} bf16_tflops_sustained (of measured: dense 16-bit tensor rate; the "
                                "kernel runs inside a 10-30 ms step, repeated)",
                 "frac_of_burst": achieved_tf / peaks["bf16_tflops"] if peaks.get("bf16_tflops") else None,
                 "counts": "algorithmic FLOPs of the polar GEMMs per step (fp32-equivalent products, full Gram: "
                           "4mn^2 + 2n^3 per quintic step, 4mn^2 per polish) over the GEMM launches' time",
-                "kernel_times": "per-phase CUDA events on the launch stream, in a profiled pass of the "
-                                "same steps right after the timed region",
+                "kernel_times": "per-phase CUDA events on the launch stream (the polar loop's phases by the "
+                                "GPU's timer inside it), in a profiled pass of the same steps right after the "
+                                "timed region",
                 "algorithmic_tflop_per_step": flops / args.steps / 1e12,
                 "rows_cols_tflop_per_step": sum(fl_rc.values()) / 1e12,
                 "rows_cols_note": "the same iteration counts priced as if every matrix iterated on its rows x cols "

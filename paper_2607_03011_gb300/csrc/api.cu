@@ -98,7 +98,7 @@ __global__ void k_debug_wait(uint32_t*, uint64_t, unsigned long long*);
 
 // The streaming passes' chunks (one CTA each): halved from the largest while the parameters do
 // not make two waves of eight CTAs per SM, down to one 16-byte vector per thread (with the
-// largest chunk 0.2 M parameters take 17 + 19 us to reduce and apply, so 6 + 7 us; 13 M with
+// largest chunk 66 k parameters take 17 + 19 us to reduce and apply, so 6 + 7 us; 15 M with
 // three replicas 79 + 70 us, so 67 + 65 us).
 inline int chunk_elems(int64_t n, int sms) {
     int c = kChunkElemsMax;

@@ -14,8 +14,8 @@
 // to tiles earlier in the sequence and all clusters are resident at once (cooperative launch),
 // so the walk cannot lock up; every wait is bounded all the same.
 //
-// Roles per CTA as in gemm.cu: warp 10 walks the sequence (all lanes: 32 matrices' control words
-// and states at a time) and queues this cluster's tiles; warp 0 waits for a tile's operands and
+// Roles per CTA as in gemm.cu: warp 10 walks the sequence (all lanes: the control words
+// and states of up to 32 matrices at a time) and queues this cluster's tiles; warp 0 waits for a tile's operands and
 // issues its TMA loads; warp 1 issues the MMAs; warps 2..9 run the epilogues.  The ring of shared memory is cut into 16 KB slots,
 // one operand plane each, so that single-, two- and three-pass tiles can follow one another:
 // a k-block takes two to four consecutive slots and one of kKb barrier pairs.
@@ -25,7 +25,8 @@
 // (K = 8) 10.70 -> 10.12 ms; 2048- and 3072-wide sets, whose phases are hundreds of waves long,
 // are level.  A scheduler warp of its own (the TMA thread used to walk: 5,800 cycles between two
 // tiles' loads, the MMAs idle for most of them): 180M 10.23 -> 9.59 ms, 2048-wide 31.0 -> 28.6,
-// 3072-wide 21.0 -> 19.8.  A phase of a few tiles takes 7 to 13 us: operands' arrival seen ~0.4, decode and
+// 3072-wide 21.0 -> 19.8.  Log of a 180M iteration (two passes): polynomial and update tiles start
+// every 17,000 to 18,000 cycles, their MMAs alone take 16,400.  A phase of a few tiles takes 7 to 13 us: operands' arrival seen ~0.4, decode and
 // loads ~1, MMAs, epilogue ~3 (its code is cold every time: ~12 cycles per instruction),
 // arrival ~1, control ~2.5.
 #include "control.cuh"

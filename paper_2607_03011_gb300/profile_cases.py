@@ -9,9 +9,9 @@ is the 48 square 1024 x 1024 matrices of the 180M recipe with K = 8 replicas
 `square12` a quarter of it; `wide12` / `tall12` twelve 1024 x 2816 matrices (the shape of
 w_gate and w_up) and twelve 2816 x 1024 ones (w_down); `wide24` the 24 w_gate / w_up matrices
 and `embed2` the 32000 x 1024 embedding and head (with `square48` and `tall12`, the 180M
-recipe's four shape buckets one at a time); with --per-launch the polar iterations are launched one
-by one (phase profiling on) instead of as the library's CUDA graph, so that every
-kernel is a plain launch.  `gemm` runs the split-precision GEMM entry point on random
+recipe's four shape buckets one at a time); with --per-launch phase profiling is on: the polar
+loop's phases run apart, and polar iterations outside its kernel are plain launches instead of
+a CUDA graph.  ncu reports no counters for the polar loop's kernel (leave it out of -k).  `gemm` runs the split-precision GEMM entry point on random
 inputs; `diloco` runs DiLoCo outer steps with a merging aggregator (Sec. 3.2), and
 `step --spectrum 1|2` the clip variants of Sec. 4.5; `hostlink` measures the host link
 (copy engines, and the host-buffer step's reduce reading pinned memory in place).
