@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_con
                     const bool ok = for_k_runs(ti, [&](int from, int to, bool at, bool bt) {
                         // instruction and operand descriptors for the layouts of this run
                         const bool a_mn = p.g[gi].a_mn || at, b_mn = p.g[gi].b_mn || bt;
-                        const uint32_t idesc = make_idesc_16bit(kTileM, BN, a_mn, b_mn, p.in_f16 != 0);
+                        const uint32_t idesc = make_idesc_16bit(kTileM, ti.n_mma, a_mn, b_mn, p.in_f16 != 0);
                         const uint64_t da = operand_desc(sbase, a_mn);
                         const uint64_t db = operand_desc(sbase + kTileABytes * (as ? 2u : 1u), b_mn);
                         const uint32_t a_lo = static_cast<uint32_t>(da), a_hi = static_cast<uint32_t>(da >> 32);

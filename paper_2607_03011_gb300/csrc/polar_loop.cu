@@ -106,7 +106,7 @@ __device__ __forceinline__ bool loop_load(const CUtensorMap* a_hi, const CUtenso
     const bool as = ti.a_split, bs = ti.b_split;
     const int need = 2 + (as ? 1 : 0) + (bs ? 1 : 0);
     const uint32_t pair_bytes = 2u * kSlotBytes * need;
-    const int m0 = ti.m0, nb0 = ti.n0 + static_cast<int>(crank) * kBRows, b = ti.b;
+    const int m0 = ti.m0, nb0 = ti.n0 + static_cast<int>(crank) * (ti.n_mma / 2), b = ti.b;
     const int k_end = to * BK;
 #pragma unroll 1
     for (int k0 = from * BK; k0 < k_end; k0 += BK) {
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_con
                     uint32_t acc = 0u;
                     const bool ok = for_k_runs(ti, [&](int from, int to, bool at, bool bt) {
                         const bool a_mn = p.groups[grp].g.a_mn || at, b_mn = p.groups[grp].g.b_mn || bt;
-                        const uint32_t idesc = make_idesc_16bit(kTileM, BN, a_mn, b_mn, f16 != 0);
+                        const uint32_t idesc = make_idesc_16bit(kTileM, ti.n_mma, a_mn, b_mn, f16 != 0);
                         const uint64_t da = operand_desc(sbase, a_mn), db = operand_desc(sbase, b_mn);
                         const uint32_t a_lo = static_cast<uint32_t>(da), a_hi = static_cast<uint32_t>(da >> 32);
                         const uint32_t b_lo = static_cast<uint32_t>(db), b_hi = static_cast<uint32_t>(db >> 32);
