@@ -323,12 +323,25 @@ __device__ __forceinline__ void gram_sums_store(const GemmGroup& g, const TileIn
     }
 }
 
-// First of the blocks of `width` columns that a half of the epilogue's warps takes: the blocks
-// that the tile has, split evenly (one half took all of a tile of up to 128 columns: steps of
-// 64-wide matrices 373 -> 344 us).
-__device__ __forceinline__ int half_begin(const GemmGroup& g, const TileInfo& ti, int half, int width) {
-    const int blocks = (min(BN, g.N - ti.n0) + width - 1) / width;
-    return min(blocks, half * ((blocks + 1) / 2));
+// The blocks of `width` columns that a half of the epilogue's warps takes: it stores [begin, end),
+// an even split of those that the tile has (one half stored all of a tile of up to 128 columns:
+// steps of 64-wide matrices 373 -> 344 us).  A tile's sums (of G^2, G's trace, tr(Q^T Delta)) go by
+// fixed columns instead, half 0's below BN / 2, so that their order, and with it every bit of
+// the result, does not depend on how the stores are dealt: half 0 looks at [end, sums_end) for
+// them alone, and half 1 sums from block sums_begin on.  (Sums dealt as the stores are: 336 us
+// instead of 338 there, another order for each width.)  Of an odd number of blocks half 1
+// stores one more, as half 0 has sums to add.
+struct HalfBlocks {
+    int begin, end, sums_begin, sums_end;
+};
+__device__ __forceinline__ HalfBlocks half_blocks(const GemmGroup& g, const TileInfo& ti, int half, int width, bool sums) {
+    const int blocks = (min(BN, g.N - ti.n0) + width - 1) / width, mid = blocks / 2, fixed = BN / 2 / width;
+    HalfBlocks r;
+    r.begin = half ? mid : 0;
+    r.end = half ? blocks : mid;
+    r.sums_begin = half ? fixed : 0;
+    r.sums_end = sums && !half ? min(blocks, fixed) : r.end;
+    return r;
 }
 
 // Epilogue of an update tile (kEpiXSplit: X = xs acc) or of a tile above the diagonal of a
@@ -351,17 +364,19 @@ __device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGrou
     const int st64 = EPI == kEpiXSplit ? 0 : kSt64;
     const uint32_t row_addr = stg + lane * 128 + ((lane & 7) << 4);
     float s_tq = 0.f, s_sq = 0.f;  // shares of tr(Q^T Delta) (ti.trace), of the sum of G^2
+    const HalfBlocks hb = half_blocks(g, ti, half, 64, EPI == kEpiGram || (EPI == kEpiXSplit && ti.trace));
 #pragma unroll 1
-    for (int c64 = half_begin(g, ti, half, 64); c64 < half_begin(g, ti, half + 1, 64); ++c64) {
+    for (int c64 = hb.begin; c64 < hb.sums_end; ++c64) {
         const int col0 = ti.n0 + c64 * 64;
         if (col0 >= g.N || row_base >= g.M) break;
+        const bool store = c64 < hb.end, sums = c64 >= hb.sums_begin;
         // kEpiPoly keeps the lo plane's words: reading G again for it made the first polynomial of
         // 86 matrices of 1024 take 251 us, so 211
         uint32_t lo[2][16];
         constexpr bool kKeepLo = EPI == kEpiPoly;
         constexpr int kUnroll = ROLLED && !kKeepLo ? 1 : EPI == kEpiGram ? 3 : 2;
 #pragma unroll kUnroll
-        for (int pl = 0; pl < nplanes; ++pl) {
+        for (int pl = 0; pl < (store ? nplanes : 1); ++pl) {
             const int kind = pl == 0 ? 0 : pl == lo_plane ? 1 : 2;
             if (elect_one()) bulk_wait_read0();
             __syncwarp();
@@ -388,8 +403,8 @@ __device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGrou
                 const int c0 = col0 + h * 32, nvalid = g.N - c0;
                 if (row_ok && nvalid > 0) {
                     if (EPI == kEpiPoly && !ti.horner) add_gram(g, ti, p.in_f16 != 0, row, c0, v);
-                    if (EPI == kEpiXSplit && ti.trace && pl == 0) s_tq = trace_share(g, ti, v, row, c0, s_tq);
-                    if (EPI == kEpiGram && pl == 0) {
+                    if (EPI == kEpiXSplit && ti.trace && pl == 0 && sums) s_tq = trace_share(g, ti, v, row, c0, s_tq);
+                    if (EPI == kEpiGram && pl == 0 && sums) {
                         // every entry counts twice, and (G - I) = G here
                         if (nvalid >= 32) {
                             float ss = 0.f;
@@ -403,6 +418,7 @@ __device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGrou
                         }
                     }
                 }
+                if (!store) continue;
                 uint32_t w[16];
                 plane_words(v, kind, of16, 0.f, ti.yc, false, 0, w);
                 if (kKeepLo && lo_plane) plane_words(v, 1, of16, 0.f, 0.f, false, 0, lo[h]);
@@ -410,6 +426,7 @@ __device__ __forceinline__ void wide_epilogue(const TileFlags& p, const GemmGrou
                 for (int q = 0; q < 4; ++q)
                     st_shared4(row_addr ^ ((h * 4 + q) << 4), w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
             }
+            if (!store) break;
             fence_proxy_async_smem();
             __syncwarp();
             if (elect_one()) {
@@ -451,8 +468,9 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
     const int lo_plane = (ti.horner || ti.hi_only || g.st_lo == nullptr) ? 0 : 1;
     const int nplanes = 1 + lo_plane + ((EPI == kEpiGram && p.gram_y) ? 1 : 0);
     float s_sq = 0.f, s_tr = 0.f, s_dev = 0.f;
+    const HalfBlocks hb = half_blocks(g, ti, half, 32, gram_fused);
 #pragma unroll 1
-    for (int c32 = half_begin(g, ti, half, 32); c32 < half_begin(g, ti, half + 1, 32); ++c32) {
+    for (int c32 = hb.begin; c32 < hb.sums_end; ++c32) {
         const int col0 = n0 + c32 * 32;
         if (col0 >= g.N || row_base >= g.M) break;
         if (sym && col0 < row_base) continue;  // block below the diagonal (warp-uniform)
@@ -477,14 +495,15 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
             for (int j = 0; j < 32; ++j)
                 if (j == d) v[j] += ca;
         }
-        if (gram_fused && row_ok && sym && !diag && nvalid == 32) {
+        const bool sums = gram_fused && row_ok && c32 >= hb.sums_begin;
+        if (sums && sym && !diag && nvalid == 32) {
             // block strictly above the diagonal: every entry counts twice and (G - I) = G
             float ss = 0.f;
 #pragma unroll
             for (int j = 0; j < 32; ++j) ss = fmaf(v[j], v[j], ss);
             s_sq = fmaf(2.f, ss, s_sq);
             s_dev = fmaf(2.f, ss, s_dev);
-        } else if (gram_fused && row_ok) {
+        } else if (sums) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
                 if (j < nvalid && (!sym || j >= d)) {
@@ -497,6 +516,7 @@ __device__ __forceinline__ void tile_epilogue(const TileFlags& p, const GemmGrou
                 }
             }
         }
+        if (c32 >= hb.end) continue;
         if (f32_out) {
             if (!row_ok) continue;
             float* base = g.out_f32 + split * g.f32_split_stride + b * g.f32_batch_stride;
