@@ -82,7 +82,7 @@ struct GemmTile {
 // is double buffered in tensor memory (2 x 256 columns): the epilogue of one tile
 // overlaps the MMAs of the next.
 template <int EPI>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_constant__ GemmParams p) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_constant__ GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint8_t* staging = smem + kRingBytes;  // kEpiWarps x (direct, mirror) blocks

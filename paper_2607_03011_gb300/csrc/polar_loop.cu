@@ -232,8 +232,11 @@ __device__ __forceinline__ int walk_matrix(const LoopPhase& L, int i) {
     return L.falling ? L.regular - 1 - i : i;
 }
 
+// The cluster size is part of the kernel, not only of its launch: a profiler that launches a
+// cooperative kernel in its own way drops the launch's cluster attribute (seen with ncu 2025.3), and
+// pair instructions outside a cluster of two fault.
 template <int NG>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_constant__ LoopParams<NG> p) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_polar_loop(const __grid_constant__ LoopParams<NG> p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
     uint8_t* staging = smem + kRingBytes;
