@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "isoloco.h"
+#include "per_device.h"
 #include "polar_loop.h"
 #include "types.h"
 
@@ -1540,11 +1541,11 @@ static int run_svd(isoloco_plan* p, cudaStream_t st) {
     int nmax = 1;
     for (int i = 0; i < p->nmat; ++i) nmax = std::max(nmax, p->mats_h[i].n);
     const size_t smem = sizeof(float) * (4 * (size_t)nmax + 32);
-    static bool attr = false;
-    if (!attr) {
-        CUDA_TRY(cudaFuncSetAttribute(k_svd_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        attr = true;
-    }
+    static PerDevice attr;
+    int unused = 0;
+    CUDA_TRY(attr.get<cudaError_t>(p->device, &unused, [](int*) {
+        return cudaFuncSetAttribute(k_svd_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    }));
     if (smem > 200 * 1024) return fail(ISOLOCO_ERR_INVALID, "exact singular values: matrices up to 12,792 wide");
     PhaseTimer tm(p, ISOLOCO_PHASE_CLIP, st);
     k_svd_tridiag<<<p->nmat, kSvdThreads, smem, st>>>(p->mats_d, p->state, p->hbuf, p->hoff_d, p->hss_d, p->nsplit_d,

@@ -26,6 +26,7 @@
 #include <cstdio>
 
 #include "gemm_tile.cuh"
+#include "per_device.h"
 
 namespace isoloco {
 
@@ -370,18 +371,20 @@ cudaLaunchConfig_t pair_config(unsigned grid, cudaStream_t stream, cudaLaunchAtt
 
 template <int EPI>
 cudaError_t launch_epi(const GemmParams& p, int max_ctas, cudaStream_t stream) {
-    static int max_clusters = 0;  // clusters of two that can be resident at once
+    static PerDevice clusters_that_fit;  // clusters of two that can be resident at once
     cudaLaunchAttribute at[1];
-    if (!max_clusters) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_split<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kGemmSmemBytes);
-        if (e != cudaSuccess) return e;
+    int device = 0, max_clusters = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    e = clusters_that_fit.get<cudaError_t>(device, &max_clusters, [&](int* n) {
+        const cudaError_t r = cudaFuncSetAttribute(k_gemm_split<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kGemmSmemBytes);
+        if (r != cudaSuccess) return r;
         const cudaLaunchConfig_t cfg = pair_config(static_cast<unsigned>(max_ctas & ~1), stream, at);
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k_gemm_split<EPI>, &cfg);
-        if (e != cudaSuccess) return e;
-        max_clusters = n > 0 ? n : 1;
-    }
+        return cudaOccupancyMaxActiveClusters(n, k_gemm_split<EPI>, &cfg);
+    });
+    if (e != cudaSuccess) return e;
+    if (max_clusters < 1) max_clusters = 1;
     int clusters = p.total_tiles;
     clusters = clusters < max_clusters ? clusters : max_clusters;
     clusters = clusters < max_ctas / 2 ? clusters : (max_ctas / 2 > 0 ? max_ctas / 2 : 1);

@@ -31,6 +31,7 @@
 // arrival ~1, control ~2.5.
 #include "control.cuh"
 #include "gemm_tile.cuh"
+#include "per_device.h"
 #include "polar_loop.h"
 
 namespace isoloco {
@@ -706,7 +707,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_p
 // ------------------------------------------------------------------ host launcher
 template <int NG>
 cudaError_t launch_polar_loop(const LoopParams<NG>& p, int clusters, cudaStream_t stream) {
-    static int max_clusters = 0;
+    static PerDevice clusters_that_fit;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2;
@@ -721,14 +722,15 @@ cudaError_t launch_polar_loop(const LoopParams<NG>& p, int clusters, cudaStream_
     cfg.stream = stream;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    if (!max_clusters) {
-        cudaError_t e = cudaFuncSetAttribute(k_polar_loop<NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLoopSmemBytes);
-        if (e != cudaSuccess) return e;
-        int n = 0;
-        e = cudaOccupancyMaxActiveClusters(&n, k_polar_loop<NG>, &cfg);
-        if (e != cudaSuccess) return e;
-        max_clusters = n > 0 ? n : 1;
-    }
+    int device = 0, max_clusters = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    e = clusters_that_fit.get<cudaError_t>(device, &max_clusters, [&](int* n) {
+        const cudaError_t r = cudaFuncSetAttribute(k_polar_loop<NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLoopSmemBytes);
+        return r != cudaSuccess ? r : cudaOccupancyMaxActiveClusters(n, k_polar_loop<NG>, &cfg);
+    });
+    if (e != cudaSuccess) return e;
+    if (max_clusters < 1) max_clusters = 1;
     cfg.gridDim = dim3(static_cast<unsigned>(2 * (clusters < max_clusters ? clusters : max_clusters)));
     return cudaLaunchKernelEx(&cfg, k_polar_loop<NG>, p);
 }
