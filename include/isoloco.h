@@ -226,6 +226,12 @@ int isoloco_check_guards(isoloco_plan_t plan, void* stream);
  * fill, with cudaMemset inside the region's own allocation.  Returns OK or INVALID. */
 int isoloco_debug_touch_guard(isoloco_plan_t plan, int region, int after);
 
+/* Test support: the plan's next `launches` launches of the kernel that runs the polar iterations
+ * after the first are taken as refused by the driver (its CTAs have to be resident together, which
+ * a restricted share of the GPU may not allow), without being made.  Those calls run the
+ * iterations as ordinary launches, with the same results.  Returns OK or INVALID. */
+int isoloco_debug_refuse_loop(isoloco_plan_t plan, int launches);
+
 /* Singular values of 2-D tensor `matrix` (table order over the 2-D tensors) from the
  * plan's last call with spectrum_kind = 3 (Alg. 2: Delta = U S V^T; here sigma_i of the
  * reduced pseudo-gradient), in descending order, copied to host memory out[0 .. r-1],

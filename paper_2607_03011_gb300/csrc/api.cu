@@ -204,6 +204,7 @@ struct isoloco_plan {
     unsigned long long* loop_prof = nullptr;  // per-phase nanoseconds (phase profiling)
     int loop_clusters = 0;
     long long loop_key[3] = {-1, -1, -2};
+    int loop_refuse = 0;  // launches of the loop still to be taken as refused (isoloco_debug_refuse_loop)
     int64_t* gpart_off_d = nullptr;
     int64_t* gpart_sstride_d = nullptr;
     int* nsplit_d = nullptr;
@@ -1204,21 +1205,37 @@ static cudaError_t run_loop_n(isoloco_plan* p, int max_iter, float tol, cudaStre
     return launch_polar_loop<NG>(lp, p->loop_clusters, st);
 }
 
+// Launch errors that say that a cooperative launch of this size cannot run here (all its CTAs at
+// once: fewer SMs than the device has under MPS or in a green context).  Nothing was launched.
+static bool loop_refused(cudaError_t e) {
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported ||
+           e == cudaErrorLaunchOutOfResources || e == cudaErrorInvalidConfiguration || e == cudaErrorInvalidClusterSize;
+}
+
 // Iterations 1, 2, ... as one launch of the polar loop (polar_loop.cu).  Not taken (false) by
 // plans with more groups than its parameters hold, or with a bucket that is not Gram-side and
 // splits its Gram over K: split partials need the finalize pass between the Gram and the
 // control step, and an unsplit Gram of that length would leave most of the GPU waiting for a
-// few tiles.  Those keep the graph of launches.
+// few tiles.  Those keep the graph of launches, and so does a call whose launch is refused.
 static bool run_loop(isoloco_plan* p, int max_iter, float tol, cudaStream_t st, cudaError_t* e) {
     if (gram_side_on(p) ? p->nftiles_reg > 0 : p->nftiles > 0) return false;
     build_loop(p);
     const int n = (int)p->loop_groups.size();
     if (n > kLoopGroups) return false;
+    if (p->loop_refuse > 0) {
+        --p->loop_refuse;
+        *e = cudaErrorCooperativeLaunchTooLarge;
+    } else {
+        *e = n <= kLoopGroupsSmall ? run_loop_n<kLoopGroupsSmall>(p, max_iter, tol, st)
+                                   : run_loop_n<kLoopGroups>(p, max_iter, tol, st);
+    }
+    if (loop_refused(*e)) {
+        (void)cudaGetLastError();
+        return false;
+    }
     // one launch; under phase profiling its phases are timed inside (isoloco_profile_read)
     p->launches += 1;
     p->prof_n[ISOLOCO_PHASE_GRAM] += 1;
-    *e = n <= kLoopGroupsSmall ? run_loop_n<kLoopGroupsSmall>(p, max_iter, tol, st)
-                               : run_loop_n<kLoopGroups>(p, max_iter, tol, st);
     return true;
 }
 
@@ -2159,6 +2176,12 @@ int isoloco_debug_touch_guard(isoloco_plan_t p, int region, int after) {
     uint8_t* base = p->guards[region].first;
     uint8_t* at = after ? base + kGuardBytes + p->guards[region].second : base + kGuardBytes - 1;
     CUDA_TRY(cudaMemset(at, 0x5A, 1));  // one guard byte, inside the allocation
+    return ISOLOCO_OK;
+}
+
+int isoloco_debug_refuse_loop(isoloco_plan_t p, int launches) {
+    if (!p || launches < 0) return fail(ISOLOCO_ERR_INVALID, "plan is NULL or launches < 0");
+    p->loop_refuse = launches;
     return ISOLOCO_OK;
 }
 

@@ -82,6 +82,7 @@ def lib():
             L.isoloco_read_singular_values.argtypes = [_vp, _vp, ctypes.c_int, _vp, ctypes.c_int]
             L.isoloco_check_guards.argtypes = [_vp, _vp]
             L.isoloco_debug_touch_guard.argtypes = [_vp, ctypes.c_int, ctypes.c_int]
+            L.isoloco_debug_refuse_loop.argtypes = [_vp, ctypes.c_int]
             L.isoloco_profile_enable.argtypes = [_vp, ctypes.c_int]
             L.isoloco_profile_read.argtypes = [_vp, _vp, _vp, _vp, ctypes.c_int]
             L.isoloco_plan_launches.argtypes = [_vp]
