@@ -332,7 +332,9 @@ enum {
  * iterations that run inside one kernel are timed by that kernel (device timer): their
  * phases then run one after the other instead of overlapping, a phase's time counts to its
  * last tile's arrival (the Gram's includes the control steps), and the kernel counts as one
- * launch of GRAM. */
+ * launch of GRAM.  enable = 2: as 1, with every phase of every iteration as launches of its own
+ * (as a captured step has them), for a profiler that looks at single launches; the host then waits
+ * for each iteration's decisions. */
 int isoloco_profile_enable(isoloco_plan_t plan, int enable);
 
 /* Synchronizes `stream`, then writes the accumulated milliseconds and launch

@@ -228,7 +228,7 @@ struct isoloco_plan {
     // polynomial, and those whose update, run a single pass
     long long prec_code = 0;
     int gp_from[2] = {0, 0}, gp_to[2] = {0, 0}, up_from[2] = {0, 0}, up_to[2] = {0, 0};
-    bool per_launch = false;        // polar iterations as plain launches (no graph), with early stop
+    bool per_launch = false;        // polar iterations as plain launches (no loop, no graph), with early stop
     bool full_prec = false;         // every polar step with three passes and no Horner form
                                     // (the clip variants' sign iteration)
     int fast_steps = 0;             // this call's fast-variant step count (0: exact Iso-C)
@@ -1346,8 +1346,9 @@ static int gs_final(isoloco_plan* p, cudaStream_t st) {
 // The polar iteration for every matrix, from Delta (planes dhi/dlo) to Q and sigma_bar.
 // Iteration 0 is launched directly; the rest run as one persistent kernel (run_loop) or, where
 // that does not apply, as one graph launch that stops as soon as every matrix is done.  When
-// `st` is being captured (and with phase profiling, without the kernel), iterations 1 ..
-// max_iter are launched one by one instead (empty launches once every matrix is done).
+// `st` is being captured, iterations 1 .. max_iter are launched one by one instead (empty
+// launches once every matrix is done); so are they with phase profiling where the kernel does
+// not apply or single launches are asked for, until every matrix is done.
 static int run_polar(isoloco_plan* p, int max_iter, float tol, cudaStream_t st) {
     if (p->nmat == 0) return ISOLOCO_OK;
     // the Gram partial slots of Gram-side matrices: iteration 0's finalize fills fewer of them
@@ -1362,7 +1363,7 @@ static int run_polar(isoloco_plan* p, int max_iter, float tol, cudaStream_t st) 
     const bool capturing = cs != cudaStreamCaptureStatusNone;
     const bool use_graph = !p->prof && !p->per_launch && !capturing;
     cudaError_t le = cudaSuccess;
-    if (!capturing && run_loop(p, max_iter, tol, st, &le)) {
+    if (!capturing && !p->per_launch && run_loop(p, max_iter, tol, st, &le)) {
         CUDA_TRY(le);
     } else if (use_graph) {
         if (!p->gexec || p->g_max_iter != max_iter || p->g_tol != tol || p->g_fast != p->fast_steps ||
@@ -1603,7 +1604,7 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
     a->fast_steps = 0;
     a->skip_trace = true;
     a->full_prec = true;  // sign(A') is used to first order (P A' P): no single-plane steps
-    a->per_launch = p->prof;  // under phase profiling, plain launches as in this plan
+    a->per_launch = p->per_launch;
     if ((rc = run_polar(a, max_iter, tol, st))) return rc;
     k_clip_form_p<<<dim3(64, a->nmat), 256, 0, st>>>(a->mats_d, a->state, a->xhi[0], a->xlo[0], a->xhi[1],
                                                      a->xlo[1], kind == 1 ? -1.f : 1.f);
@@ -2082,6 +2083,7 @@ int isoloco_profile_enable(isoloco_plan_t p, int enable) {
     }
     CUDA_TRY(cudaMemset(p->loop_prof, 0, sizeof(unsigned long long) * kLoopPhases));
     p->prof = enable != 0;
+    p->per_launch = enable == 2;
     return ISOLOCO_OK;
 }
 

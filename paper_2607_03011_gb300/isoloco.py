@@ -241,9 +241,10 @@ class Plan:
     def last_status(self, stream=None) -> int:
         return int(self._L.isoloco_last_status(self._h, _stream(stream)))
 
-    def profile(self, enable: bool = True):
-        """Turns per-phase CUDA-event timing on or off (resets the accumulators)."""
-        _check(self._L.isoloco_profile_enable(self._h, int(bool(enable))), "isoloco_profile_enable")
+    def profile(self, enable=True):
+        """Turns per-phase timing on or off (resets the accumulators); 2: on, with the polar
+        iterations as single launches instead of one kernel."""
+        _check(self._L.isoloco_profile_enable(self._h, int(enable)), "isoloco_profile_enable")
 
     def profile_read(self, stream=None):
         """{phase: (milliseconds, launches)} accumulated since profile() was called."""

@@ -9,10 +9,9 @@ is the 48 square 1024 x 1024 matrices of the 180M recipe with K = 8 replicas
 `square12` a quarter of it; `wide12` / `tall12` twelve 1024 x 2816 matrices (the shape of
 w_gate and w_up) and twelve 2816 x 1024 ones (w_down); `wide24` the 24 w_gate / w_up matrices
 and `embed2` the 32000 x 1024 embedding and head (with `square48` and `tall12`, the 180M
-recipe's four shape buckets one at a time); with --per-launch phase profiling is on: the polar
-loop's phases run apart, and polar iterations outside its kernel are plain launches instead of
-a CUDA graph.  ncu reports no counters for the polar loop's kernel (leave it out of -k).  `gemm` runs the split-precision GEMM entry point on random
-inputs; `diloco` runs DiLoCo outer steps with a merging aggregator (Sec. 3.2), and
+recipe's four shape buckets one at a time); with --per-launch every phase of the
+polar iterations is a launch of its own instead of one kernel (or a CUDA graph).  `gemm` runs the
+split-precision GEMM entry point on random inputs; `diloco` runs DiLoCo outer steps with a merging aggregator (Sec. 3.2), and
 `step --spectrum 1|2` the clip variants of Sec. 4.5; `hostlink` measures the host link
 (copy engines, and the host-buffer step's reduce reading pinned memory in place).
 """
@@ -48,7 +47,7 @@ def run_step(workload: str, steps: int, per_launch: bool = False, spectrum_kind:
     wl = W.make_workload(spec, seed=0, device="cuda")
     plan = isoloco.Plan(wl.table, wl.N, wl.K, wl.replicas.dtype)
     if per_launch:
-        plan.profile(True)
+        plan.profile(2)
     opts = isoloco.make_opts(spec.alpha, spec.outer_lr, spec.momentum, spectrum_kind=spectrum_kind)
     th0, b0 = wl.theta.clone(), wl.momentum.clone()
     for _ in range(steps):
