@@ -86,7 +86,7 @@ __global__ void k_ties_init(int, uint64_t, uint64_t, uint64_t, unsigned long lon
                             uint64_t*, uint64_t*, uint64_t*, unsigned long long*, int*);
 __global__ void k_ties_sample(ReplicaPtrs, int, int, const float*, int64_t, int64_t, uint32_t*);
 __global__ void k_ties_hist_buf(const uint32_t*, const uint32_t*, int, int64_t, int, int, int, const uint64_t*,
-                                unsigned long long*);
+                                const uint64_t*, unsigned long long*);
 __global__ void k_ties_check(int, int, int64_t, uint64_t, const unsigned long long*, const uint32_t*, uint64_t*,
                              int*);
 __global__ void k_ties_hist(ReplicaPtrs, int, int, const float*, int64_t, int, const uint64_t*, unsigned long long*,
@@ -1407,14 +1407,18 @@ static int finish_call(isoloco_plan* p, cudaStream_t st, int sync) {
 }
 
 // ---------------------------------------------------------------- TIES trim buffers
+// m of a sample of S keys at sparsity 1/2: 8 standard deviations of a sample count, and 16.
+static int ties_widest(int64_t S) { return static_cast<int>(8.0 * std::sqrt((double)S * 0.25) + 16.0); }
+
 // Sized once for the plan: a sample of S = min(N, 2^20) keys per worker, and candidate
-// segments (one per CTA of the bracket pass) for the widest bracket (sparsity 1/2), with 4x
-// headroom over the expected count per CTA.
+// segments (one per CTA of the bracket pass) for the widest rank distance (2 m + 1 of the sample,
+// sparsity 1/2), with 4x headroom over the expected count per CTA.  Widening an end of the bracket
+// to its bin adds at most m of the sample, so that 2x is left.
 static int ensure_ties(isoloco_plan* p, int nseg) {
     if (p->ties_hist) return ISOLOCO_OK;
     const int K = p->K;
     const int64_t S = std::min<int64_t>(p->N, int64_t(1) << 20);
-    const double m = 8.0 * std::sqrt((double)S * 0.25) + 16.0;
+    const double m = ties_widest(S);
     const double expected = (2.0 * m + 1.0) / (double)S * (double)p->N;  // candidates per worker
     const int64_t segcap = round_up((int64_t)std::ceil(4.0 * expected / nseg) + 256, 4);
     int rc;
@@ -1950,18 +1954,19 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
         const uint64_t r_hi = (uint64_t)std::max(1.0, std::floor(r_mid - m));
         const uint64_t r_lo = (uint64_t)std::min(S, std::ceil(r_mid + m));
         {
-            PhaseTimer tm(p, ISOLOCO_PHASE_TRIM, st, select ? 25 : 1);
+            PhaseTimer tm(p, ISOLOCO_PHASE_TRIM, st, select ? 29 : 1);
             k_ties_init<<<1, 256, 0, st>>>(K, n_keep, r_hi, r_lo, p->ties_hist, p->ties_rank_s, p->ties_prefix_s,
                                            p->ties_rank_c, p->ties_prefix_c, p->ties_rank_f, p->ties_prefix_f,
                                            p->ties_above, p->ties_fail);
             if (select) {
                 k_ties_sample<<<(unsigned)((p->ties_S + 255) / 256), 256, 0, st>>>(rp, K, p->dtype, theta, p->N,
                                                                                  p->ties_S, p->ties_samp);
-                for (int pass = 0; pass < 2; ++pass) {
+                for (int pass = 0; pass < 4; ++pass) {  // (the last two end at once where the bins were widened)
                     k_ties_hist_buf<<<dim3(1, 256), 256, 2 * K * 256 * 4, st>>>(
-                        p->ties_samp, nullptr, 1, p->ties_S, 2 * K, 2, pass, p->ties_prefix_s, p->ties_hist);
+                        p->ties_samp, nullptr, 1, p->ties_S, 2 * K, 2, pass, p->ties_rank_s, p->ties_prefix_s,
+                        p->ties_hist);
                     k_ties_select<<<(2 * K * 32 + 255) / 256, 256, 0, st>>>(2 * K, pass, p->ties_hist, p->ties_rank_s, p->ties_prefix_s,
-                                                     nullptr, pass == 1);
+                                                     nullptr, pass == 1 ? ties_widest(p->ties_S) : 0);
                 }
                 CUDA_TRY(launch_ties_bracket(rp, K, p->dtype, theta, p->N, p->ties_prefix_s, p->ties_cand, p->ties_cnt,
                                              p->ties_segcap, p->ties_above, p->ties_nseg, st));
@@ -1969,8 +1974,8 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
                                                p->ties_rank_c, p->ties_fail);
                 for (int pass = 0; pass < 4; ++pass) {
                     k_ties_hist_buf<<<dim3(p->ties_nseg, 1), 256, K * 256 * 4, st>>>(
-                        p->ties_cand, p->ties_cnt, p->ties_nseg, p->ties_segcap, K, 1, pass, p->ties_prefix_c,
-                        p->ties_hist);
+                        p->ties_cand, p->ties_cnt, p->ties_nseg, p->ties_segcap, K, 1, pass, p->ties_rank_c,
+                        p->ties_prefix_c, p->ties_hist);
                     k_ties_select<<<(K * 32 + 255) / 256, 256, 0, st>>>(K, pass, p->ties_hist, p->ties_rank_c, p->ties_prefix_c,
                                                     nullptr, 0);
                 }

@@ -644,10 +644,11 @@ cudaError_t launch_dare(const ReplicaPtrs& reps, int K, bool bf16, float* theta,
 // the replicas, the library brackets the threshold first:
 //   1. k_ties_sample: S keys per worker at jittered strided positions;
 //   2. radix select on the sample for two ranks per worker, the expected rank of the
-//      threshold -/+ 8 standard deviations (and 16), in its first two digits only: the
-//      bracket [lo, hi] is widened to the ends of the 2^15-key bins that hold them (0.4 % of
-//      the magnitude each, against ~1 % between the ranks), which the exact selection below
-//      does not depend on;
+//      threshold -/+ 8 standard deviations (and 16): the bracket [lo, hi].  After two digits an
+//      end is widened to that of the 2^15-key bin that holds it (0.4 % of the magnitude), which
+//      the exact selection below does not depend on, unless the bin holds more of the sample
+//      than the candidate buffer has room for (magnitudes close together): such an end takes
+//      its last two digits too;
 //   3. k_ties_bracket, one pass over the replicas: A = #(key > hi) and the keys in [lo, hi]
 //      collected per CTA (its own segment of the candidate buffer);
 //   4. k_ties_check: if A < n_keep <= A + #candidates and no segment overflowed, the
@@ -720,21 +721,26 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_hist(ReplicaPtrs reps, 
 
 // A radix pass over keys already in a buffer [K][nseg][segcap] (counts[k][seg] valid keys,
 // clamped to segcap; all segcap when counts is null), for nw selections: selection v reads
-// worker v / vdiv.  grid = (nseg, splits of a segment).
+// worker v / vdiv, unless it is decided (rank 0).  grid = (nseg, splits of a segment).
 __global__ void __launch_bounds__(kStreamThreads) k_ties_hist_buf(const uint32_t* __restrict__ keys,
                                                                   const uint32_t* __restrict__ counts, int nseg,
                                                                   int64_t segcap, int nw, int vdiv, int pass,
+                                                                  const uint64_t* __restrict__ rank,
                                                                   const uint64_t* __restrict__ prefix,
                                                                   unsigned long long* __restrict__ hist) {
     extern __shared__ uint32_t sh[];
     const int shift = ties_shift(pass);
     const int hs = pass == 0 ? 31 : ties_shift(pass - 1);
     const uint32_t mask = static_cast<uint32_t>(ties_bins(pass) - 1);
+    bool open = false;
+    for (int v = threadIdx.x & 31; v < nw; v += 32) open |= rank[v] != 0;
+    if (!__any_sync(0xffffffffu, open)) return;  // (the same in every warp)
     for (int j = threadIdx.x; j < nw * 256; j += blockDim.x) sh[j] = 0u;
     __syncthreads();
     const int seg = blockIdx.x;
     const int lane = threadIdx.x & 31;
     for (int v = 0; v < nw; ++v) {
+        if (rank[v] == 0) continue;
         const int k = v / vdiv;
         const int64_t n = counts ? min(static_cast<int64_t>(counts[static_cast<int64_t>(k) * nseg + seg]), segcap)
                                  : segcap;
@@ -927,8 +933,9 @@ __global__ void __launch_bounds__(256) k_ties_check(int K, int nseg, int64_t seg
 // One warp per selection: the bin holding the rank-th largest key (counting from the top),
 // appended to the prefix; the histogram row is cleared for the next pass.  Lane l holds bins
 // 8 l .. 8 l + 7; a suffix sum over the warp finds the bin.  With only_if_fail it runs only
-// when *only_if_fail != 0 (the fallback passes).  widen: the last pass of the sample's bracket;
-// the prefix of an even selection (hi) gets ones, of an odd one (lo) zeros below its digits.
+// when *only_if_fail != 0 (the fallback passes).  A bin of at most `widen` keys ends the selection
+// here (the sample's bracket, widened): rank 0, and the prefix of an even selection (hi) gets
+// ones, of an odd one (lo) zeros below its digits.
 __global__ void __launch_bounds__(256) k_ties_select(int nw, int pass, unsigned long long* __restrict__ hist,
                                                      uint64_t* __restrict__ rank, uint64_t* __restrict__ prefix,
                                                      const int* __restrict__ only_if_fail, int widen) {
@@ -963,19 +970,23 @@ __global__ void __launch_bounds__(256) k_ties_select(int nw, int pass, unsigned 
         }
         return;
     }
-    unsigned long long rr = r - above;
+    unsigned long long rr = r - above, in_bin = 0;
     int digit = 8 * lane;
 #pragma unroll
     for (int q = 7; q >= 0; --q) {
         if (rr <= c[q]) {
             digit = 8 * lane + q;
+            in_bin = c[q];
             break;
         }
         rr -= c[q];
     }
     rank[w] = rr;
     prefix[w] |= static_cast<uint64_t>(digit) << ties_shift(pass);
-    if (widen && (w & 1) == 0) prefix[w] |= (1ull << ties_shift(pass)) - 1ull;
+    if (in_bin <= static_cast<unsigned long long>(widen)) {
+        rank[w] = 0;
+        if ((w & 1) == 0) prefix[w] |= (1ull << ties_shift(pass)) - 1ull;
+    }
 }
 
 // TIES elect and disjoint merge.  Entry kept when its key >= the threshold (ties kept).  P and N
