@@ -1954,7 +1954,9 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
         const uint64_t r_hi = (uint64_t)std::max(1.0, std::floor(r_mid - m));
         const uint64_t r_lo = (uint64_t)std::min(S, std::ceil(r_mid + m));
         {
-            PhaseTimer tm(p, ISOLOCO_PHASE_TRIM, st, select ? 29 : 1);
+            // init, sample, check, three selections of four digits in two launches each, and the bracket
+            // pass of every group of workers
+            PhaseTimer tm(p, ISOLOCO_PHASE_TRIM, st, select ? 27 + (K + kTiesWorkers - 1) / kTiesWorkers : 1);
             k_ties_init<<<1, 256, 0, st>>>(K, n_keep, r_hi, r_lo, p->ties_hist, p->ties_rank_s, p->ties_prefix_s,
                                            p->ties_rank_c, p->ties_prefix_c, p->ties_rank_f, p->ties_prefix_f,
                                            p->ties_above, p->ties_fail);

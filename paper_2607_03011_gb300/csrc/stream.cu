@@ -804,7 +804,6 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_sample(ReplicaPtrs reps
 // and a worker's four keys share the test for the rare push, whose position comes from a
 // shared atomic.  180M x 8: 1.84 -> 1.27 ms fp32 (6.2 TB/s) and 2.5 -> 1.0 ms bf16, against
 // counters per thread in shared memory, four loads in flight and the type tested between them.
-constexpr int kTiesWorkers = 8;
 template <bool BF16>
 __global__ void __launch_bounds__(kStreamThreads) k_ties_bracket(ReplicaPtrs reps, int K,
                                                                  const float* __restrict__ theta, int64_t N,

@@ -230,6 +230,7 @@ struct UpdateSrc {
 };
 
 constexpr int kMaxK = 64;
+constexpr int kTiesWorkers = 8;  // workers of one launch of the TIES bracket pass
 struct ReplicaPtrs {
     const void* p[kMaxK];
 };
