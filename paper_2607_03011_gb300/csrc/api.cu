@@ -1569,7 +1569,7 @@ static int run_svd(isoloco_plan* p, cudaStream_t st) {
         return cudaFuncSetAttribute(k_svd_tridiag, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     }));
     if (smem > 200 * 1024) return fail(ISOLOCO_ERR_INVALID, "exact singular values: matrices up to 12,792 wide");
-    PhaseTimer tm(p, ISOLOCO_PHASE_CLIP, st);
+    PhaseTimer tm(p, ISOLOCO_PHASE_CLIP, st, 3);
     k_svd_tridiag<<<p->nmat, kSvdThreads, smem, st>>>(p->mats_d, p->state, p->hbuf, p->hoff_d, p->hss_d, p->nsplit_d,
                                                       p->tri, p->tri_off_d);
     CUDA_TRY(cudaGetLastError());
@@ -1578,7 +1578,6 @@ static int run_svd(isoloco_plan* p, cudaStream_t st) {
     CUDA_TRY(cudaGetLastError());
     k_svd_sigma_bar<<<(p->nmat + 7) / 8, 256, 0, st>>>(p->mats_d, p->nmat, p->state, p->sv, p->sv_off_d);
     CUDA_TRY(cudaGetLastError());
-    p->launches += 4;
     return ISOLOCO_OK;
 }
 

@@ -42,7 +42,8 @@ def test_diloco_launches(K, kw):
     assert n == seen
 
 
-@pytest.mark.parametrize("shapes,kw", [(MATS, {}), (MATS + GRAM_SIDE, {}), (MATS, {"fast_steps": 5}), (MATS, {"spectrum_kind": 1})])
+@pytest.mark.parametrize("shapes,kw", [(MATS, {}), (MATS + GRAM_SIDE, {}), (MATS, {"fast_steps": 5}), (MATS, {"spectrum_kind": 1}),
+                                       (MATS, {"spectrum_kind": 3})])
 def test_outer_step_launches(shapes, kw):
     from paper_2607_03011_gb300 import isoloco as iso
     wl = W.make_workload(W.custom_spec(shapes, K=2, rank=2, momentum_std=1e-4), seed=34, device="cuda")
