@@ -17,8 +17,12 @@ enum : uint32_t {
     kErrTimeout = 4u,
 };
 
-// Any single wait on an mbarrier gives up after this long (ns) and raises
-// kErrTimeout; the kernel then drains and returns instead of hanging the GPU.
+// The limit of a wait (ns): a wait that has gone on for longer gives up and raises kErrTimeout, and
+// the kernel then drains and returns instead of hanging the GPU.  Every wait in k_gemm_split and
+// the polar loop's waits for data have this limit; the polar loop's waits for a queue slot or an
+// accumulator have twice, those for the next tile three times the limit, since what they wait
+// for may itself be waiting for data.  The copies in flight at the end share one limit
+// (drain_barriers).
 constexpr uint64_t kWaitTimeoutNs = 2000000000ull;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -106,6 +110,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
     for (uint32_t i = 1;; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
         if ((i & 63u) == 0 && globaltimer_ns() - t0 > limit_ns) return false;
+    }
+}
+
+// Waits for n barriers after a failure, within one limit for all of them: at(i, bar, parity) names
+// the i-th and returns whether it is to be waited for.
+template <class F>
+__device__ __forceinline__ void drain_barriers(int n, F at) {
+    const uint64_t t0 = globaltimer_ns();
+    for (int i = 0; i < n; ++i) {
+        uint64_t* bar = nullptr;
+        uint32_t parity = 0u;
+        if (!at(i, bar, parity)) continue;
+        const uint64_t gone = globaltimer_ns() - t0;
+        (void)mbar_wait(bar, parity, gone < kWaitTimeoutNs ? kWaitTimeoutNs - gone : 0ull);
     }
 }
 

@@ -187,8 +187,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_g
                 if (leader) {
                     // stages before pos were last filled in this pass of the ring, the others in
                     // the pass before it (if there was one)
-                    for (int s = 0; s < nstages; ++s)
-                        if (s < pos.stage || wrapped) (void)mbar_wait(&full[s], s < pos.stage ? pos.phase : pos.phase ^ 1u);
+                    drain_barriers(nstages, [&](int s, uint64_t*& bar, uint32_t& parity) {
+                        bar = &full[s];
+                        parity = s < pos.stage ? pos.phase : pos.phase ^ 1u;
+                        return s < pos.stage || wrapped;
+                    });
                 } else {
                     const uint64_t t0 = globaltimer_ns();
                     while (globaltimer_ns() - t0 < 100000ull) {

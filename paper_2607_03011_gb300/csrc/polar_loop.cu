@@ -340,15 +340,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_p
                 // let the copies in flight land before the CTA exits (rank 0's barriers also
                 // count rank 1's copies; rank 1 cannot observe its own, so it leaves a margin)
                 if (leader) {
-                    int k = ring.tail;
-                    uint32_t ph = ring.tphase;
-                    for (int i = 0; i < ring.inflight; ++i) {
-                        (void)mbar_wait(&full[k], ph);
-                        if (++k == kKb) {
-                            k = 0;
-                            ph ^= 1u;
-                        }
-                    }
+                    drain_barriers(ring.inflight, [&](int i, uint64_t*& bar, uint32_t& parity) {
+                        const int k = ring.tail + i;
+                        bar = &full[k < kKb ? k : k - kKb];
+                        parity = k < kKb ? ring.tphase : ring.tphase ^ 1u;
+                        return true;
+                    });
                 } else {
                     const uint64_t t0 = globaltimer_ns();
                     while (globaltimer_ns() - t0 < 100000ull) {
@@ -530,9 +527,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_p
         // no more tiles
         __syncwarp();
         if (elect_one()) {
-            if (mbar_wait(&tq_empty[q], qphase ^ 1u)) {
+            if (mbar_wait(&tq_empty[q], qphase ^ 1u, 2 * kWaitTimeoutNs)) {
                 tq[q].kind = -1;
                 mbar_arrive(&tq_full[q]);
+            } else {
+                *abort_flag = 1;
+                atomicOr(p.err, kErrTimeout);
             }
         }
         __syncwarp();
