@@ -281,11 +281,17 @@ def test_deterministic(iso):
     assert torch.equal(r1[1], r2[1]) and torch.equal(r1[2], r2[2]) and torch.equal(r1[3], r2[3])
 
 
-def test_graph_loop_matches_per_launch_loop(iso):
-    """The polar loop runs as one CUDA graph whose while-node stops once every matrix is
-    done; under phase profiling it runs launch by launch instead.  Both give the same bits,
-    the graph running at most one extra (empty) iteration, and a new max_iter rebuilds it."""
-    spec = W.custom_spec(RAGGED, K=3, rank=2, momentum_std=1e-4)
+# Grams split over K that are not Gram-side, of more than one tile: the plan keeps the graph of launches
+SPLIT_GRAM = [("a", 4200, 600), ("b", 600, 4200), ("c", 300, 257), ("v", 5, 0)]
+
+
+@pytest.mark.parametrize("shapes,graph", [(RAGGED, False), (SPLIT_GRAM, True)], ids=["kernel", "graph"])
+def test_graph_loop_matches_per_launch_loop(iso, shapes, graph):
+    """The polar loop runs as one kernel, its phases apart under phase profiling; or, where a
+    Gram is split over K, as one CUDA graph whose while-node stops once every matrix is done,
+    launch by launch under phase profiling.  Both give the same bits, the graph running at most
+    one extra (empty) iteration, and a new max_iter rebuilds it."""
+    spec = W.custom_spec(shapes, K=3, rank=2, momentum_std=1e-4)
     wl = W.make_workload(spec, seed=11, device="cuda")
     plan = iso.Plan(wl.table, wl.N, wl.K)
     for max_iter in (0, 20):
@@ -301,6 +307,10 @@ def test_graph_loop_matches_per_launch_loop(iso):
         assert torch.equal(g[1], h[1]) and torch.equal(g[2], h[2]) and torch.equal(g[3], h[3])
         assert g[4]["iters"] == h[4]["iters"] and g[4]["sigma_bar"] == h[4]["sigma_bar"]
         assert lh <= lg <= lh + lh // 2, (lg, lh)
+        # a launch per phase of each iteration, or one for them all
+        assert (lg > 4 * max(g[4]["iters"])) == graph, (lg, g[4]["iters"])
+    if graph:
+        compare(wl, *g[:5], 1.0, 0.7, 0.9)
 
 
 # ---- the fast variant of Sec. 4.3: a fixed number of quintic steps, sigma_bar = ||Delta||_F / sqrt(r)
