@@ -819,7 +819,6 @@ static int flush_set(isoloco_plan* pl, int phase, LaunchSet& s, cudaStream_t st)
         int cta = 0;
         for (size_t i = first; i < s.groups.size() && p.num_groups < kMaxGroups; ++i) {
             GemmGroup g = s.groups[i];
-            g.cta_begin = cta;
             cta += g.batch * group_tiles(g) * g.splits;
             p.g[p.num_groups++] = g;
         }
@@ -928,8 +927,6 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
             w.b_hi = m + z_map(zb, 1, 0);
             set_group_common(w, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
             w.bucket = (int)b;
-            w.out_hi = p->whi + bk.gs_off;
-            w.out_lo = p->wlo + bk.gs_off;
             w.st_hi = m + w_st_map(0);
             w.st_lo = m + w_st_map(1);
             w.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
@@ -939,8 +936,6 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
             g.b_hi = m + w_mn_map(0);
             set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
-            g.out_hi = p->ghi + bk.gplane_off;
-            g.out_lo = p->glo + bk.gplane_off;
             g.st_hi = m + gp_st_map(0, 0);
             g.st_lo = m + gp_st_map(0, 1);
             g.st_y = m + y_st_map();
@@ -962,8 +957,6 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
         g.f32_batch_stride = (int64_t)bk.n * bk.ld_n;
         g.f32_split_stride = (int64_t)bk.count * bk.n * bk.ld_n;
         g.ld_f32 = bk.ld_n;
-        g.out_hi = p->ghi + bk.gplane_off;
-        g.out_lo = p->glo + bk.gplane_off;
         g.st_hi = m + gp_st_map(0, 0);
         g.st_lo = m + gp_st_map(0, 1);
         g.st_y = m + y_st_map();
@@ -990,8 +983,6 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
         g.b_tri = (first || full) ? kTriB : kTriY;
         set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
         g.bucket = (int)b;
-        g.out_hi = p->phi + bk.gplane_off;
-        g.out_lo = p->plo + bk.gplane_off;
         g.st_hi = m + gp_st_map(1, 0);
         g.st_lo = m + gp_st_map(1, 1);
         g.bf_batch_stride = (int64_t)bk.n * bk.ld_n;
@@ -1022,8 +1013,6 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
             g.b_tri = kTriB;
             set_group_common(g, bk.n, bk.n, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
-            g.out_hi = p->xhi[dst] + bk.plane_off;
-            g.out_lo = p->xlo[dst] + bk.plane_off;
             g.st_hi = m + z_map(dst, 2, 0);
             g.st_lo = m + z_map(dst, 2, 1);
             g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
@@ -1042,8 +1031,6 @@ static void build_iteration(isoloco_plan* p, int t, IterSets& s) {
         }
         set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
         g.bucket = (int)b;
-        g.out_hi = p->xhi[dst] + bk.plane_off;
-        g.out_lo = p->xlo[dst] + bk.plane_off;
         g.st_hi = m + x_st_map(dst, 0);
         g.st_lo = m + x_st_map(dst, 1);
         g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
@@ -1159,8 +1146,7 @@ static void build_loop(isoloco_plan* p) {
             L = LoopPhase{};
             L.kind = ph;
             L.first = (int)p->loop_groups.size();
-            L.ngroups = (int)ls.groups.size();
-            if (L.ngroups)
+            if (!ls.groups.empty())
                 L.f = {ls.p.gate, ls.p.in_f16, ls.p.out_f16, ls.p.split_on_polish, ls.p.gram_y, ls.p.poly_horner,
                        ls.p.unit_scale};
             const int dep = ph == kLoopUpdate ? kLoopPoly : ph == kLoopGramGs ? kLoopW : kLoopUpdate;
@@ -1323,8 +1309,6 @@ static int gs_final(isoloco_plan* p, cudaStream_t st) {
             set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
             g.gate_fb = fb + 1;
-            g.out_hi = p->xhi[1 - fb] + bk.plane_off;
-            g.out_lo = p->xlo[1 - fb] + bk.plane_off;
             g.st_hi = m + x_st_map(1 - fb, 0);
             g.st_lo = m + x_st_map(1 - fb, 1);
             g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
@@ -1630,15 +1614,11 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
                 if (step == 0) {
                     g.a_hi = m + src_map(psrc, kRoleKA, 0);
                     g.b_hi = m + src_map(0, kRoleKB, 0);
-                    g.out_hi = a->ghi + bk.gplane_off;
-                    g.out_lo = a->glo + bk.gplane_off;
                     g.st_hi = m + gp_st_map(0, 0) + kSt64;
                     g.st_lo = m + gp_st_map(0, 1) + kSt64;
                 } else {
                     g.a_hi = m + g_map(kRoleKA, 0);
                     g.b_hi = m + src_map(psrc, kRoleKB, 0);
-                    g.out_hi = a->phi + bk.gplane_off;
-                    g.out_lo = a->plo + bk.gplane_off;
                     g.st_hi = m + gp_st_map(1, 0) + kSt64;
                     g.st_lo = m + gp_st_map(1, 1) + kSt64;
                 }
@@ -1678,8 +1658,6 @@ static int run_clip(isoloco_plan* p, int kind, int max_iter, float tol, cudaStre
             set_group_common(g, bk.rows, bk.cols, bk.n, bk.count, 1, bk.mat_base);
             g.bucket = (int)b;
             g.gate_fb = fb + 1;
-            g.out_hi = p->xhi[dst] + bk.plane_off;
-            g.out_lo = p->xlo[dst] + bk.plane_off;
             g.st_hi = m + x_st_map(dst, 0);
             g.st_lo = m + x_st_map(dst, 1);
             g.bf_batch_stride = (int64_t)bk.rows * bk.ld;
@@ -2288,7 +2266,6 @@ int isoloco_debug_gemm(int a_mn, int b_mn, int precision, int batch, int M, int 
     g.a_split = gp.a_split;
     g.b_split = gp.b_split;
     set_group_common(g, M, N, K, batch, 1, 0);
-    g.cta_begin = 0;
     g.out_f32 = D;
     g.f32_batch_stride = (int64_t)M * N;
     g.f32_split_stride = 0;
@@ -2407,7 +2384,6 @@ int isoloco_debug_gemm_noalloc(int a_mn, int b_mn, int precision, int batch, int
     g.a_split = gp.a_split;
     g.b_split = gp.b_split;
     set_group_common(g, M, N, K, batch, 1, 0);
-    g.cta_begin = 0;
     g.out_f32 = D;
     g.f32_batch_stride = (int64_t)M * N;
     g.f32_split_stride = 0;

@@ -14,8 +14,9 @@
 // Roles (352 threads): warp 0 issues TMA loads into a ring of shared
 // memory stages; warp 1 owns the tensor-memory accumulator and issues tcgen05.mma
 // from one thread; warps 2..9 drain the accumulator (tcgen05.ld) and run the
-// epilogue; warp 10 decodes the tiles for all of them, through a queue in shared memory.  Stage hand-off uses mbarriers: `full` (TMA bytes landed), `empty`
-// (the MMAs reading a stage finished, via tcgen05.commit), `acc` (all MMAs done).
+// epilogue; warp 10 decodes the tiles for all of them, through a queue in shared memory.
+// Stage hand-off uses mbarriers: `full` (TMA bytes landed), `empty` (the MMAs reading a stage
+// finished, via tcgen05.commit), `tfull` / `tempty` (an accumulator written / read).
 //
 // Operand layouts: K-major operands (K contiguous in global memory) use swizzled
 // tiles BK deep; MN-major operands (M or N contiguous) use 128-byte swizzled tiles of
@@ -86,14 +87,14 @@ template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_gemm_split(const __grid_constant__ GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align1024(smem_raw);
-    uint8_t* staging = smem + kRingBytes;  // kEpiWarps x (direct, mirror) blocks
+    uint8_t* staging = smem + kRingBytes;  // kEpiWarps x kStageBlocks blocks
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRingBytes + kEpiStagingBytes);
     uint64_t* empty = full + kMaxStages;
     uint64_t* tfull = empty + kMaxStages;  // [2] accumulator buffer ready for the epilogue
     uint64_t* tempty = tfull + 2;        // [2] accumulator buffer released by the epilogue
     uint64_t* drain = tempty + 2;        // teardown: every issued MMA has completed
-    uint64_t* tq_full = drain + 1;       // [kTileQueue] tile written by the producer
-    uint64_t* tq_empty = tq_full + kTileQueue;  // [kTileQueue] read by the MMA and epilogue warps
+    uint64_t* tq_full = drain + 1;       // [kTileQueue] tile written by the scheduler
+    uint64_t* tq_empty = tq_full + kTileQueue;  // [kTileQueue] read by the TMA, MMA and epilogue warps
     GemmTile* tq = reinterpret_cast<GemmTile*>(tq_empty + kTileQueue);
     int* pre = reinterpret_cast<int*>(tq + kTileQueue);  // [kMaxGroups + 1] active-tile prefix
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pre + kMaxGroups + 1);
@@ -296,7 +297,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_g
         }
     } else {
         // ================= epilogue (warps 2..9): warp w reads TMEM lanes 32 (w % 4) ..,
-        // warps 2..5 take columns 0..127 of the tile and warps 6..9 columns 128..255
+        // warps 2..5 store the first half of the tile's column blocks, warps 6..9 the others
         const int eg = warp & 3;  // tensor-memory lane quarter this warp may access
         const int half = (warp - 2) >> 2;
         uint32_t n = 0;

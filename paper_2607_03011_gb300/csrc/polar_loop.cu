@@ -15,10 +15,11 @@
 // so the walk cannot lock up; every wait is bounded all the same.
 //
 // Roles per CTA as in gemm.cu: warp 10 walks the sequence (all lanes: the control words
-// and states of up to 32 matrices at a time) and queues this cluster's tiles; warp 0 waits for a tile's operands and
-// issues its TMA loads; warp 1 issues the MMAs; warps 2..9 run the epilogues.  The ring of shared memory is cut into 16 KB slots,
-// one operand plane each, so that single-, two- and three-pass tiles can follow one another:
-// a k-block takes two to four consecutive slots and one of kKb barrier pairs.
+// and states of up to 32 matrices at a time) and queues this cluster's tiles; warp 0 waits for
+// a tile's operands and issues its TMA loads; warp 1 issues the MMAs; warps 2..9 run the
+// epilogues.  The ring of shared memory is cut into 16 KB slots, one operand plane each, so that
+// single-, two- and three-pass tiles can follow one another: a k-block takes two to four
+// consecutive slots and one of kKb barrier pairs.
 //
 // Measured (GB300, whole outer step against the same kernels as a graph of launches): eight
 // matrices of 64 to 256 (K = 2) 586 -> 399 us, ragged 515-wide set (K = 3) 2052 -> 1546, the 180M set
@@ -446,13 +447,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1) k_p
                         const bool has = j0 < tiles;
                         off = (off + total) % C;
                         // this cluster's matrices: their states, and whether their operands are there
-                        // (if not, the TMA thread waits for them)
+                        // (if not, the TMA thread waits for them).  A state is that of the decision this
+                        // phase follows: the next one waits for this cluster's tiles
                         TileState st = {};
                         bool there = true;
                         if (has) {
                             load_state(p.state + mat, st);
                             if (kind != kLoopPoly) there = ld_acquire(cnt) >= want;
-                            if (stepping && decided > need) st.mode = 1;
                         }
                         unsigned m = __ballot_sync(0xffffffffu, has);
                         while (m && ok) {

@@ -22,8 +22,8 @@ struct LoopGroup {
 struct LoopPhase {
     TileFlags f;
     int kind;
-    int first, ngroups;  // groups [first, first + ngroups)
-    int count;           // their matrices
+    int first;           // its first group
+    int count;           // the matrices of its groups
     // order in which they come up (walk_matrix in polar_loop.cu): the first `regular` in rising
     // or falling order, the first `skip` of these after the next `skip`, the others (Gram-side)
     // at position side_at

@@ -47,8 +47,8 @@ constexpr int kGramSideRatio = 8;
 // residual below the convergence tolerance, so the Gram cannot be the one the polish uses.
 constexpr float kOnePassGramResid = 0.5f;
 // Epilogue staging: per epilogue warp two blocks of 32 x 32 16-bit values (2 KB, 64-byte
-// swizzled rows), written to global memory by TMA stores: a symmetric output's block and its
-// transpose, or alternately single blocks.
+// swizzled rows), written to global memory by TMA stores: a block of a symmetric output's
+// diagonal tile and its transpose; or, taken together, 32 rows of 64 values (128-byte swizzle).
 constexpr int kStageBlockBytes = 32 * 32 * 2;
 constexpr int kStageBlocks = 2;
 constexpr int kEpiStagingBytes = kEpiWarps * kStageBlocks * kStageBlockBytes;
@@ -89,7 +89,6 @@ struct GemmGroup {
     int sym;        // square symmetric output: compute and store only tiles touching col >= row
                     // (fp32 outputs: mirrored as well)
     int tiles_sym;  // number of such tiles per matrix
-    int cta_begin;  // (host bookkeeping) first tile of the group when every matrix is active
     int mat_base;   // index of the group's first matrix in the state array
     int bucket;     // shape bucket: index into the work-list counts
     int gate_fb;    // 0: no condition; f > 0: only matrices whose Q is in buffer f - 1 (final_buf)
@@ -110,9 +109,7 @@ struct GemmGroup {
     // 16-bit hi/lo output planes (kEpiGram, kEpiPoly, kEpiXSplit) and their TMA store maps
     // (kEpiXSplit: boxes of 64 columns x 32 rows, 128-byte swizzle; else 32 x 32, 64-byte
     // swizzle, and the 64 x 32 one kSt64 or, for Y, kStY64 further in the bucket's maps);
-    // out_lo/st_lo may be null when no lo plane is kept
-    __nv_bfloat16* out_hi;
-    __nv_bfloat16* out_lo;
+    // st_lo may be null when no lo plane is kept
     const CUtensorMap* st_hi;
     const CUtensorMap* st_lo;
     const CUtensorMap* st_y;  // kEpiGram with gram_y: store map of the Y plane
