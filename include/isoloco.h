@@ -30,6 +30,12 @@
  *   and return without waiting, unless opts->sync is set.  A plan's workspace is
  *   used by one call at a time: calls on the same plan from different streams
  *   must be ordered by the caller.
+ * - The polar iterations after the first are one kernel with a CTA on every SM (as many as there
+ *   are output tiles, if fewer), all resident together: it starts once the SMs it needs are free
+ *   and holds them until the last matrix is done (5 ms at 180M parameters), so kernels on other
+ *   streams run before or after it, not between its phases.  Copies by the copy engines overlap
+ *   with it.  Where the driver refuses such a launch, on a stream under capture, and for plans whose
+ *   Gram of a long matrix is split over K, every phase is a launch of its own, with the same results.
  * - Return values are isoloco_status_t codes.  No C++ exception crosses the ABI.
  *   isoloco_last_error() gives a thread-local message for the last failure.
  * - Sign convention (Alg. 1/2): Delta_k = theta - theta_k, and theta moves by
