@@ -270,6 +270,15 @@ def stream_bytes(table, K, replica_bytes):
 # tensor-core passes over hi/lo splits of fp32 operands with fp32 accumulation.
 DTYPE_ISO = "f32 streaming; polar GEMMs as bf16/fp16 hi+lo split passes, f32 accumulate"
 
+# DRAM bytes (read + write) of all GEMM launches of one step, k_gemm_split's and k_polar_loop's, from
+# an ncu capture of the whole step: (workload, fast_steps, spectrum_kind) -> figure.
+GEMM_TRAFFIC = {
+    ("llama_180m_k8", 0, 0): {
+        "bytes_per_step": 22.73e9,
+        "note": "dram__bytes_read.sum + dram__bytes_write.sum of the four k_gemm_split launches and the "
+                "k_polar_loop launch of one step, one ncu pass; same unit as achieved (per step over all "
+                "GEMM launches)"},
+}
 
 # --------------------------------------------------------------------------- CPU oracle arm
 CPU_SAMPLE = ["layers.0.attn_norm", "layers.0.wq", "layers.0.wk", "layers.0.ffn_norm", "layers.0.w_gate", "layers.0.w_up",
@@ -645,11 +654,12 @@ def main():
         ms, n = prof[phase]
         return nbytes * args.steps / (ms / 1000.0) / 1e9 if ms > 0 else 0.0
 
+    traffic = GEMM_TRAFFIC.get((args.workload, args.fast_steps, spectrum_kind))
     roofline = {"bound": "tensor", "kernel": "k_gemm_split and k_polar_loop (Gram, polynomial and update GEMMs)",
                 "achieved": achieved_tf, "peak": tc_peak, "unit": "TFLOP/s",
                 "frac": achieved_tf / tc_peak if tc_peak else None,
-                "traffic": None,
-                "traffic_note": "no DRAM capture: ncu reports no counters for the polar loop's kernel",
+                "traffic": traffic["bytes_per_step"] if traffic else None,
+                "traffic_note": traffic["note"] if traffic else "no DRAM capture of this configuration",
                 "peak_source": f"{peak_src} bf16_tflops_sustained (of measured: dense 16-bit tensor rate; the "
                                "kernel runs inside a 10-30 ms step, repeated)",
                 "frac_of_burst": achieved_tf / peaks["bf16_tflops"] if peaks.get("bf16_tflops") else None,
