@@ -273,7 +273,9 @@ __device__ __forceinline__ void plane_words(const float (&v)[32], int kind, bool
 }
 
 // kEpiPoly without Horner's form: v = cc v + cb G for this lane's row and 32 columns from c0 (G past
-// L1: within the polar loop other SMs rewrite it in every iteration).
+// L1: within the polar loop other SMs rewrite it in every iteration).  Which product is rounded is
+// spelled out: left to the compiler it differs between instantiations and columns, and with it
+// the result's bits.  A block cut short rounds the other product than a whole one, as it always has.
 __device__ __forceinline__ void add_gram(const GemmGroup& g, const TileInfo& ti, bool f16, int row, int c0,
                                          float (&v)[32]) {
     const int64_t goff = ti.b * g.bf_batch_stride + static_cast<int64_t>(row) * g.ld_bf + c0;
@@ -292,14 +294,14 @@ __device__ __forceinline__ void add_gram(const GemmGroup& g, const TileInfo& ti,
             for (int w = 0; w < 4; ++w) {
                 const float g0 = dec16(hw[w] & 0xFFFFu, f16) + dec16(lw[w] & 0xFFFFu, f16);
                 const float g1 = dec16(hw[w] >> 16, f16) + dec16(lw[w] >> 16, f16);
-                v[8 * q + 2 * w] = cc * v[8 * q + 2 * w] + cb * g0;
-                v[8 * q + 2 * w + 1] = cc * v[8 * q + 2 * w + 1] + cb * g1;
+                v[8 * q + 2 * w] = fmaf(cb, g0, cc * v[8 * q + 2 * w]);
+                v[8 * q + 2 * w + 1] = fmaf(cb, g1, cc * v[8 * q + 2 * w + 1]);
             }
         }
     } else {
 #pragma unroll
         for (int j = 0; j < 32; ++j)
-            if (j < g.N - c0) v[j] = cc * v[j] + cb * (dec16(__ldcg(gh + j), f16) + dec16(__ldcg(gl + j), f16));
+            if (j < g.N - c0) v[j] = fmaf(cc, v[j], cb * (dec16(__ldcg(gh + j), f16) + dec16(__ldcg(gl + j), f16)));
     }
 }
 
