@@ -1942,8 +1942,8 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
                                                                                  p->ties_S, p->ties_samp);
                 for (int pass = 0; pass < 4; ++pass) {  // (the last two end at once where the bins were widened)
                     k_ties_hist_buf<<<dim3(1, 256), 256, 2 * K * 256 * 4, st>>>(
-                        p->ties_samp, nullptr, 1, p->ties_S, 2 * K, 2, pass, p->ties_rank_s, p->ties_prefix_s,
-                        p->ties_hist);
+                        p->ties_samp, nullptr, 1, p->ties_S, 2 * K, 2, pass, pass < 2 ? nullptr : p->ties_rank_s,
+                        p->ties_prefix_s, p->ties_hist);
                     k_ties_select<<<(2 * K * 32 + 255) / 256, 256, 0, st>>>(2 * K, pass, p->ties_hist, p->ties_rank_s, p->ties_prefix_s,
                                                      nullptr, pass == 1 ? ties_widest(p->ties_S) : 0);
                 }
@@ -1953,8 +1953,8 @@ int diloco_outer_step(isoloco_plan_t p, float* theta, float* momentum, const voi
                                                p->ties_rank_c, p->ties_fail);
                 for (int pass = 0; pass < 4; ++pass) {
                     k_ties_hist_buf<<<dim3(p->ties_nseg, 1), 256, K * 256 * 4, st>>>(
-                        p->ties_cand, p->ties_cnt, p->ties_nseg, p->ties_segcap, K, 1, pass, p->ties_rank_c,
-                        p->ties_prefix_c, p->ties_hist);
+                        p->ties_cand, p->ties_cnt, p->ties_nseg, p->ties_segcap, K, 1, pass, nullptr, p->ties_prefix_c,
+                        p->ties_hist);
                     k_ties_select<<<(K * 32 + 255) / 256, 256, 0, st>>>(K, pass, p->ties_hist, p->ties_rank_c, p->ties_prefix_c,
                                                     nullptr, 0);
                 }

@@ -732,7 +732,8 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_hist(ReplicaPtrs reps, 
 
 // A radix pass over keys already in a buffer [K][nseg][segcap] (counts[k][seg] valid keys,
 // clamped to segcap; all segcap when counts is null), for nw selections: selection v reads
-// worker v / vdiv, unless it is decided (rank 0).  grid = (nseg, splits of a segment).
+// worker v / vdiv, unless it is decided (rank 0; rank null: none is).  grid = (nseg, splits of a
+// segment).
 __global__ void __launch_bounds__(kStreamThreads) k_ties_hist_buf(const uint32_t* __restrict__ keys,
                                                                   const uint32_t* __restrict__ counts, int nseg,
                                                                   int64_t segcap, int nw, int vdiv, int pass,
@@ -743,15 +744,17 @@ __global__ void __launch_bounds__(kStreamThreads) k_ties_hist_buf(const uint32_t
     const int shift = ties_shift(pass);
     const int hs = pass == 0 ? 31 : ties_shift(pass - 1);
     const uint32_t mask = static_cast<uint32_t>(ties_bins(pass) - 1);
-    bool open = false;
-    for (int v = threadIdx.x & 31; v < nw; v += 32) open |= rank[v] != 0;
-    if (!__any_sync(0xffffffffu, open)) return;  // (the same in every warp)
+    if (rank) {
+        bool open = false;
+        for (int v = threadIdx.x & 31; v < nw; v += 32) open |= rank[v] != 0;
+        if (!__any_sync(0xffffffffu, open)) return;  // (the same in every warp)
+    }
     for (int j = threadIdx.x; j < nw * 256; j += blockDim.x) sh[j] = 0u;
     __syncthreads();
     const int seg = blockIdx.x;
     const int lane = threadIdx.x & 31;
     for (int v = 0; v < nw; ++v) {
-        if (rank[v] == 0) continue;
+        if (rank && rank[v] == 0) continue;
         const int k = v / vdiv;
         const int64_t n = counts ? min(static_cast<int64_t>(counts[static_cast<int64_t>(k) * nseg + seg]), segcap)
                                  : segcap;
